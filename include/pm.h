@@ -420,7 +420,8 @@ int64_t pm_launch_count(pm_ctx* ctx);
 /* Bytes of device memory the context holds now (what pm_config.mem_limit is checked against). */
 int64_t pm_memory_used(pm_ctx* ctx);
 /* Testing aid for the failure paths (no counterpart in the paper).  what = PM_INJECT_DROP_COPY:
- * in the next TMA-pipelined FFT pass (meshes up to 512^3) the first CTA does not issue its
+ * the next plain y or x FFT pass (meshes up to 512^3) runs TMA-pipelined and its first CTA (or
+ * that of a fused k-space x pass, if that comes first) does not issue its
  * first tile copy, so its bounded wait on that copy runs out (after a short limit), the CTA
  * waits for its other copies in flight and returns, and the next pm_sync reports PM_ETIMEOUT;
  * the pass's output is then invalid, the context stays usable.  One shot: consumed by that

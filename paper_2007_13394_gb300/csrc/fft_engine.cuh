@@ -1,7 +1,7 @@
 // Stockham FFT engine shared by the FFT kernels (device code only).
 //
 // A line of M points (M a power of two, 16 <= M <= 2048) is held by M/V threads,
-// V = 16 (8 or 32) values each (value s of thread j is element j + s M/V).  Stockham
+// V = 8, 16 or 32 values each (value s of thread j is element j + s M/V).  Stockham
 // stages of radix V (the last stage radix 2..V) run in registers; between stages the line
 // goes through shared memory, padded by one float2 per 16 (per 32 when V = 32) so that
 // the stride-V writes of the first stage are free of bank conflicts.  A line's elements may be
@@ -142,8 +142,9 @@ __device__ __forceinline__ void line_sync() {
 }
 
 // One Stockham stage on a line of M points (sub-transform length NS, radix R), V values
-// a thread (value s of thread j is element j + s M / V).
-template <int M, int TWN, int NS, int R, bool INV, bool LAST, int V = 16, bool WARP = false>
+// a thread (value s of thread j is element j + s M / V).  TAIL: a barrier after the values
+// are read back (false when nothing writes the shared memory after this exchange).
+template <int M, int TWN, int NS, int R, bool INV, bool LAST, int V = 16, bool WARP = false, bool TAIL = true>
 __device__ __forceinline__ void stage(float2 (&v)[V], int j, float2* sm, int cs,
                                       const float2* __restrict__ tw) {
   constexpr int B = V / R;  // butterflies per thread
@@ -176,18 +177,21 @@ __device__ __forceinline__ void stage(float2 (&v)[V], int j, float2* sm, int cs,
     line_sync<WARP>();
 #pragma unroll
     for (int s = 0; s < V; ++s) v[s] = sm[padv<V>(j + s * Q) * cs];
-    line_sync<WARP>();
+    if constexpr (TAIL) line_sync<WARP>();
   }
 }
 
-template <int M, int TWN, int NS, bool INV, int V = 16, bool WARP = false>
+// All stages of a line.  ENDS: the shared memory is not written again after this transform,
+// so its last exchange needs no trailing barrier.
+template <int M, int TWN, int NS, bool INV, int V = 16, bool WARP = false, bool ENDS = false>
 __device__ __forceinline__ void run_stages(float2 (&v)[V], int j, float2* sm, int cs,
                                            const float2* __restrict__ tw) {
   constexpr int REM = M / NS;
   constexpr int R = REM >= V ? V : REM;
   constexpr bool LAST = (NS * R == M);
-  stage<M, TWN, NS, R, INV, LAST, V, WARP>(v, j, sm, cs, tw);
-  if constexpr (!LAST) run_stages<M, TWN, NS * R, INV, V, WARP>(v, j, sm, cs, tw);
+  constexpr bool LASTX = !LAST && M / (NS * R) <= V;  // the transform's last exchange
+  stage<M, TWN, NS, R, INV, LAST, V, WARP, !(ENDS && LASTX)>(v, j, sm, cs, tw);
+  if constexpr (!LAST) run_stages<M, TWN, NS * R, INV, V, WARP, ENDS>(v, j, sm, cs, tw);
 }
 
 // Twiddles a thread's stages use, held in registers.  They depend only on the thread's
@@ -377,16 +381,15 @@ __device__ __forceinline__ int nsq_index(int kx, int ky, int kz) {
 enum { EPI_NONE = 0, EPI_GREEN = 1, EPI_POT = 2 };  // EPI_POT: Green's function, then inverse
 enum { PRO_NONE = 0, PRO_GRAD = 1 };
 
-// MODE_POT: forward x FFT, Green's function, inverse x FFT (the potential, one output)
-enum { MODE_PLAIN = 0, MODE_GREEN = 1, MODE_GRAD = 2, MODE_FUSED = 3, MODE_POT = 4 };
+// passes of the TMA kernel
+enum { MODE_PLAIN = 0, MODE_FUSED = 3 };
 
 }  // namespace fft
 
 // TMA-pipelined strided pass over one of the context's force meshes (k_fft_tma.cu);
 // returns PM_EINVAL when it does not apply (no tensor maps, foreign buffer or size),
-// so the caller runs the classic kernel instead.
+// so the caller runs the other kernel instead.
 int strided_tma(pm_ctx* c, const Geom& g, const float2* src, float2* d0, float2* d1, float2* d2,
-                int axis, bool inv, int mode, int comp, const float2* tw, const fft::KTables& kt,
-                cudaStream_t s);
+                int axis, bool inv, int mode, const float2* tw, const fft::KTables& kt, cudaStream_t s);
 
 }  // namespace pmnu

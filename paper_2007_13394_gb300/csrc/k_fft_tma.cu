@@ -1,18 +1,19 @@
-// Strided FFT passes (y and x) with TMA-prefetched column tiles.
+// Strided FFT passes with TMA-prefetched column tiles: the fused x pass of the k-space force,
+// and the plain passes while a dropped copy is pending (pm_test_inject).  Every other strided
+// pass runs in k_fft.cu's register-resident kernel, which is faster at every size (the plain
+// passes 3 % at 64^3 to 37 % at 256^3, the potential's x pass 40 to 50 %).
 //
 // A persistent CTA walks its share of the column tiles (TK adjacent kz columns of
 // one y plane or one x line set).  One thread issues the tensor-memory-accelerator
 // copies (cp.async.bulk.tensor.3d) of the tiles one and two ahead (one ahead in the
-// two-transform passes) into further shared-memory buffers while the whole CTA
-// transforms the current one, so DRAM stays busy during the radix stages.  The tile arrives dense, element (column c, line index i) at
-// i * TK + c, which is exactly what the first Stockham stage reads.  Results go
-// back to global memory with ordinary coalesced stores.
+// fused pass) into further shared-memory buffers while the whole CTA transforms the
+// current one, so DRAM stays busy during the radix stages.  The tile arrives dense, element
+// (column c, line index i) at i * TK + c, which is exactly what the first Stockham stage
+// reads.  Results go back to global memory with ordinary coalesced stores.
 //
-// Variants: plain (y or x), x with the Green's function epilogue, x with the
-// -i k_j prologue, the x pass of the potential (forward, Green's function, inverse;
-// in place), and the fused x pass of the k-space force (forward, Green's function,
-// then IFFT(-i k_x phi) and IFFT(phi) scaled by -i k_y and -i k_z; phi parks in the
-// tile's own input buffer, which nothing else touches until the next prefetch).
+// Variants: plain (y or x), and the fused x pass of the k-space force (forward, Green's
+// function, then IFFT(-i k_x phi) and IFFT(phi) scaled by -i k_y and -i k_z; phi parks in
+// the tile's own input buffer, which nothing else touches until the next prefetch).
 // In-place passes are safe: a tile's columns are read (by its CTA's prefetch) and
 // written (by the same CTA, later) by one CTA only.
 //
@@ -76,14 +77,10 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-// Shared memory.  Single-transform passes (plain, Green's function, gradient): three
-// tile buffers (copies run two tiles ahead of the transform), each sized for the
-// padded work layout (rounded up to 128 bytes, the alignment of a tensor copy's
-// destination) because the Stockham stages run in the buffer of the tile just read.
-// Two-transform passes (potential, fused) keep two tile buffers and a separate work
-// area: measured with 16 values a thread, where the in-buffer layout meant three CTAs
-// at 80 registers, the spills and the extra barrier cost more than the deeper prefetch
-// gained; the potential pass is close to issue-bound, so prefetch depth is not its limit.
+// Shared memory.  Plain passes: three tile buffers (copies run two tiles ahead of the
+// transform), each sized for the padded work layout (rounded up to 128 bytes, the
+// alignment of a tensor copy's destination) because the Stockham stages run in the buffer
+// of the tile just read.  The fused pass keeps two tile buffers and a separate work area.
 // values a thread holds: 8 (radix-8 stages, 64 registers, twice the resident warps of
 // the 16-value form) from 256-point lines up
 template <int LOGM>
@@ -100,7 +97,7 @@ struct TmaShape {
   static constexpr int THREADS = TK * M / V;
   static constexpr uint32_t TILE_BYTES = (uint32_t)M * TK * 8;
   static constexpr size_t WORK_BYTES = (size_t)(M + M / 16 + 1) * TK * 8;
-  static constexpr bool WORK_IN_TILE = MODE != MODE_FUSED && MODE != MODE_POT;
+  static constexpr bool WORK_IN_TILE = MODE != MODE_FUSED;
   static constexpr int NBUF = WORK_IN_TILE ? 3 : 2;
   static constexpr size_t BUF_BYTES = WORK_IN_TILE ? (WORK_BYTES + 127) / 128 * 128 : (size_t)TILE_BYTES;
   static constexpr size_t SMEM = NBUF * BUF_BYTES + (WORK_IN_TILE ? 0 : WORK_BYTES);
@@ -111,7 +108,7 @@ template <int LOGM, int TK, bool INV, int MODE, bool WIN>
 __global__ void __launch_bounds__(TmaShape<LOGM, TK, MODE>::THREADS, 2) k_fft_strided_tma(
     const __grid_constant__ CUtensorMap map, float2* __restrict__ d0, float2* __restrict__ d1,
     float2* __restrict__ d2, int axis, int pc, int ntiles_z, int ntiles,
-    const float2* __restrict__ tw, KTables kt, int comp, int* __restrict__ err, int drop) {
+    const float2* __restrict__ tw, KTables kt, int* __restrict__ err, int drop) {
   using S = TmaShape<LOGM, TK, MODE>;
   constexpr int M = S::M, V = S::V, Q = M / V, NBUF = S::NBUF;
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -184,37 +181,22 @@ __global__ void __launch_bounds__(TmaShape<LOGM, TK, MODE>::THREADS, 2) k_fft_st
 #pragma unroll
     for (int s = 0; s < V; ++s) v[s] = in[(j + s * Q) * TK + c];
     if constexpr (S::WORK_IN_TILE) __syncthreads();  // every input read before the stages overwrite it
-    if constexpr (MODE == MODE_GRAD) {  // v *= -i k_comp; x pass: element index kx, outer ky
-#pragma unroll
-      for (int s = 0; s < V; ++s) {
-        const int kx = j + s * Q;
-        const float kk = comp == 0 ? __ldg(kt.kvec0 + kx)
-                                   : (comp == 1 ? __ldg(kt.kvec0 + outer) : (ok ? __ldg(kt.kvec0 + kz) : 0.f));
-        v[s] = make_float2(kk * v[s].y, -kk * v[s].x);
-      }
-    }
     run_stages_reg<M, 1, INV, 0, NTW, V>(v, j, work + c, TK, twr);
-    if constexpr (MODE == MODE_GREEN || MODE == MODE_FUSED || MODE == MODE_POT) {
+    if constexpr (MODE == MODE_FUSED) {
       const float wy = WIN ? __ldg(kt.winv + outer) : 1.0f, ky2 = __ldg(kt.ksq + outer);
       const float wz = !ok ? 0.f : (WIN ? __ldg(kt.winv + kz) : 1.0f), kz2 = ok ? __ldg(kt.ksq + kz) : 0.f;
 #pragma unroll
       for (int s = 0; s < V; ++s) {
         const int kx = j + s * Q;
         const float k2 = __ldg(kt.ksq + kx) + ky2 + kz2;
-        // fast division (2 ulp), as in the classic passes
         float g = kt.gcoef * (WIN ? __ldg(kt.winv + kx) : 1.0f) * wy * wz / k2;
         if (k2 == 0.0f) g = 0.0f;
         if (kt.mtab && ok) g *= __ldg(kt.mtab + nsq_index<M>(kx, outer, kz));
         v[s] = cscale(v[s], g);
-        if constexpr (MODE == MODE_FUSED) {
-          in[(j + s * Q) * TK + c] = v[s];               // phi, read back by this thread only
-          const float kk = __ldg(kt.kvec0 + kx);
-          v[s] = make_float2(kk * v[s].y, -kk * v[s].x);  // -i k_x phi
-        }
+        in[(j + s * Q) * TK + c] = v[s];               // phi, read back by this thread only
+        const float kk = __ldg(kt.kvec0 + kx);
+        v[s] = make_float2(kk * v[s].y, -kk * v[s].x);  // -i k_x phi
       }
-    }
-    if constexpr (MODE == MODE_POT) run_stages_reg<M, 1, true, 0, NTW, V>(v, j, work + c, TK, twr);
-    if constexpr (MODE == MODE_FUSED) {
       run_stages_reg<M, 1, true, 0, NTW, V>(v, j, work + c, TK, twr);
       if (ok) {
 #pragma unroll
@@ -242,19 +224,19 @@ __global__ void __launch_bounds__(TmaShape<LOGM, TK, MODE>::THREADS, 2) k_fft_st
   }
 }
 
-// columns per tile: TK * M = 4096 points, 8..16 columns
+// columns per tile: 16, 8 for lines of 512 points
 template <int LOGM>
 constexpr int tk_tma() {
-  return LOGM >= 11 ? 2 : (LOGM == 10 ? 4 : (LOGM == 9 ? 8 : 16));
+  return LOGM == 9 ? 8 : 16;
 }
 
 template <int LOGM, bool INV, int MODE>
 int launch(pm_ctx* c, const CUtensorMap* map, float2* d0, float2* d1, float2* d2, int axis, int pc,
-           const float2* tw, const KTables& kt, int comp, cudaStream_t s) {
+           const float2* tw, const KTables& kt, cudaStream_t s) {
   constexpr int TK = tk_tma<LOGM>();
   using SH = TmaShape<LOGM, TK, MODE>;
   constexpr int M = SH::M;
-  constexpr bool GREEN = MODE == MODE_GREEN || MODE == MODE_FUSED || MODE == MODE_POT;  // read the window
+  constexpr bool GREEN = MODE == MODE_FUSED;  // reads the window
   const int w = (GREEN && kt.winv) ? 1 : 0;
   auto kern = w ? k_fft_strided_tma<LOGM, TK, INV, MODE, GREEN> : k_fft_strided_tma<LOGM, TK, INV, MODE, false>;
   static int blocks_per_sm[2] = {0, 0};
@@ -273,22 +255,20 @@ int launch(pm_ctx* c, const CUtensorMap* map, float2* d0, float2* d1, float2* d2
   if (grid > ntiles) grid = ntiles;
   const int drop = c->inject == PM_INJECT_DROP_COPY ? 1 : 0;
   c->inject = 0;  // one shot
-  kern<<<grid, SH::THREADS, SH::SMEM, s>>>(*map, d0, d1, d2, axis, pc, ntz, ntiles, tw, kt, comp,
-                                            c->err_dev, drop);
+  kern<<<grid, SH::THREADS, SH::SMEM, s>>>(*map, d0, d1, d2, axis, pc, ntz, ntiles, tw, kt, c->err_dev,
+                                            drop);
   return PM_OK;
 }
 
 template <bool INV, int MODE>
 int dispatch(pm_ctx* c, const Geom& g, const CUtensorMap* map, float2* d0, float2* d1, float2* d2,
-             int axis, const float2* tw, const KTables& kt, int comp, cudaStream_t s) {
+             int axis, const float2* tw, const KTables& kt, cudaStream_t s) {
   switch (g.logn) {
-    case 5: return launch<5, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, comp, s);
-    case 6: return launch<6, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, comp, s);
-    case 7: return launch<7, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, comp, s);
-    case 8: return launch<8, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, comp, s);
-    case 9: return launch<9, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, comp, s);
-    case 10: return launch<10, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, comp, s);
-    case 11: return launch<11, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, comp, s);
+    case 5: return launch<5, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, s);
+    case 6: return launch<6, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, s);
+    case 7: return launch<7, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, s);
+    case 8: return launch<8, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, s);
+    case 9: return launch<9, INV, MODE>(c, map, d0, d1, d2, axis, g.pc, tw, kt, s);
     default: return PM_EINVAL;
   }
 }
@@ -312,17 +292,15 @@ PFN_cuTensorMapEncodeTiled_v12000 encoder() {
 
 // Tensor maps of the three force meshes, one per pass direction (box TK x 256 along y
 // or along x).  Returns false (and the callers keep the non-TMA kernels) when the
-// driver entry point is missing.
+// driver entry point is missing or the lines are too long (see strided_tma).
 bool tma_init(pm_ctx* c) {
   c->tma_ok = false;
+  if (c->g.logn >= 10) return false;
   auto enc = encoder();
   if (!enc) return false;
   const Geom& g = c->g;
   const int M = g.n, BOXR = M < 256 ? M : 256;
-  int tk = 16;
-  if (g.logn >= 11) tk = 2;
-  else if (g.logn == 10) tk = 4;
-  else if (g.logn == 9) tk = 8;
+  const int tk = g.logn == 9 ? tk_tma<9>() : tk_tma<8>();
   float2* bufs[3] = {c->meshA, c->meshB, c->meshC};
   for (int b = 0; b < 3; ++b) {
     for (int axis = 0; axis < 2; ++axis) {  // 0: x pass box, 1: y pass box
@@ -351,22 +329,18 @@ static int mesh_index(pm_ctx* c, const float2* p) {
 }
 
 int strided_tma(pm_ctx* c, const Geom& g, const float2* src, float2* d0, float2* d1, float2* d2,
-                int axis, bool inv, int mode, int comp, const float2* tw, const fft::KTables& kt,
-                cudaStream_t s) {
+                int axis, bool inv, int mode, const float2* tw, const fft::KTables& kt, cudaStream_t s) {
   using namespace fft;
   if (!c->tma_ok || g.n != c->g.n) return PM_EINVAL;
   // Columns of 1024 or more points only fit 2- or 4-column tiles (16-32 B rows), which the
-  // TMA engine serves far below the classic kernels' rate: TMA for up to 512 points.
+  // TMA engine serves far below the other kernels' rate: TMA for up to 512 points.
   if (g.logn >= 10) return PM_EINVAL;
   const int bi = mesh_index(c, src);
   if (bi < 0) return PM_EINVAL;
   const CUtensorMap* map = &c->tmap[bi][axis == 1 ? 1 : 0];
-  if (!inv && mode == MODE_PLAIN) return dispatch<false, MODE_PLAIN>(c, g, map, d0, d1, d2, axis, tw, kt, comp, s);
-  if (inv && mode == MODE_PLAIN) return dispatch<true, MODE_PLAIN>(c, g, map, d0, d1, d2, axis, tw, kt, comp, s);
-  if (!inv && mode == MODE_GREEN) return dispatch<false, MODE_GREEN>(c, g, map, d0, d1, d2, axis, tw, kt, comp, s);
-  if (inv && mode == MODE_GRAD) return dispatch<true, MODE_GRAD>(c, g, map, d0, d1, d2, axis, tw, kt, comp, s);
-  if (!inv && mode == MODE_FUSED) return dispatch<false, MODE_FUSED>(c, g, map, d0, d1, d2, axis, tw, kt, comp, s);
-  if (!inv && mode == MODE_POT) return dispatch<false, MODE_POT>(c, g, map, d0, d1, d2, axis, tw, kt, comp, s);
+  if (!inv && mode == MODE_PLAIN) return dispatch<false, MODE_PLAIN>(c, g, map, d0, d1, d2, axis, tw, kt, s);
+  if (inv && mode == MODE_PLAIN) return dispatch<true, MODE_PLAIN>(c, g, map, d0, d1, d2, axis, tw, kt, s);
+  if (!inv && mode == MODE_FUSED) return dispatch<false, MODE_FUSED>(c, g, map, d0, d1, d2, axis, tw, kt, s);
   return PM_EINVAL;
 }
 
