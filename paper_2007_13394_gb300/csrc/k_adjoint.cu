@@ -8,8 +8,11 @@
 //   kernel so G_j^T = -G_j):
 //     dL/dx_i = sum_j lambda_F,ij grad R[G_j rho](x_i) + m_i grad R[B](x_i),
 //     B_k = sum_j i D(k_j) g(k) FFT(paint(lambda_F,j))_k, D the gradient kernel.
-//   With the 4-point kernel (and no learned factor) both terms run on one potential
-//   mesh at a time: G_j rho = -S_j phi, and B = G * (sum_j S_j paint(lambda_F,j)).
+//   With the 4-point kernel both terms run on one potential mesh each: G_j rho = -S_j phi,
+//   and B = G * (sum_j S_j paint(lambda_F,j)).  With the learned factor the first term keeps
+//   its three force meshes (the stencil of an FP32 potential would carry seven times their
+//   rounding error), and the factor's gradient needs only the spectra of rho and of the
+//   divergence (k_vjp_combine).
 // * KDK step VJP (p_h = p0 + K1 F(x0), x1 = x0 + Delta p_h, p1 = p_h + K2 F(x1)).
 // * Zel'dovich IC transpose: s_j = T_j omega with T_j = IFFT diag(S_j) FFT, so
 //   dL/domega = IFFT(sum_j conj(S_j) FFT(lambda_s,j)), neutrino sites with the
@@ -134,16 +137,26 @@ __device__ __forceinline__ void vjp_cp_async16(void* smem_dst, const void* gmem_
                : "memory");
 }
 
-// out[d][perm[i]] = sum_j lambda_j(i) d/dx_d R[F_j](x_i), F_j = -S_j phi, one CTA per
-// tile: the tile's potential with the stencil halo staged like the forward readout's,
-// F_j at the particle's 8 CIC corners from the 56 values, then the CIC weight
-// derivatives (the pattern of k_readout_grad).
-__global__ void __launch_bounds__(kVjpThreads) k_readout_grad_fd4(
-    const uint32_t* __restrict__ us, int64_t n, const uint32_t* __restrict__ bstart,
-    const float* __restrict__ phi, int nm, int shift, int ntl, int row_pitch, float inv12h, float inv_h,
-    const float* __restrict__ lam, const uint32_t* __restrict__ perm, float* __restrict__ out,
-    int* __restrict__ err) {
-  __shared__ __align__(16) float sp[kVjpSpanXY * kVjpSpanXY * kVjpSpanZ];
+// Both terms of the force VJP in one pass over the sorted particles, one CTA per tile:
+//   out[d][perm[i]] = sum_j lambda_j(i) d/dx_d R[F_j](x_i) + m_i d/dx_d R[B](x_i),  F_j = -S_j phi.
+// The tile's potential with the stencil halo is staged like the forward readout's, B with the
+// halo of the CIC corners; F_j at the particle's 8 corners comes from 56 values of phi, then
+// the CIC weight derivatives.  Bound by the shared-memory pipe (56 + 8 random gathers a
+// particle); a separate pass over B gathered 8 values from global memory and updated the
+// gradient a second time (step_vjp at 256^3: 124 us a force).
+constexpr int kVjpSpanB = kTile + 1;                   // cells 0 .. 16 along x and y
+constexpr int kVjpSpanBZ = kTile + 4;                  // cells 0 .. 19 along z
+constexpr int kVjpStageB = kVjpSpanB * kVjpSpanB * (kVjpSpanBZ / 4);
+constexpr int kVjpBSY = kVjpSpanBZ, kVjpBSX = kVjpSpanB * kVjpSpanBZ;
+constexpr size_t kVjpSmem = sizeof(float) * (kVjpSpanXY * kVjpSX + kVjpSpanB * kVjpBSX);
+
+__global__ void __launch_bounds__(kVjpThreads) k_force_vjp_readout(
+    const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n, const uint32_t* __restrict__ bstart,
+    const float* __restrict__ phi, const float* __restrict__ B, int nm, int shift, int ntl, int row_pitch,
+    float inv12h, float inv_h, const float* __restrict__ lam, MassTable mt, const uint32_t* __restrict__ perm,
+    float* __restrict__ out, int* __restrict__ err) {
+  extern __shared__ __align__(16) float sp[];
+  float* const sb = sp + kVjpSpanXY * kVjpSX;
   const int t = threadIdx.x;
   const uint32_t tile = blockIdx.x;
   const uint32_t lo = bstart[8 * tile], hi = bstart[8 * tile + 8];
@@ -157,6 +170,12 @@ __global__ void __launch_bounds__(kVjpThreads) k_readout_grad_fd4(
     const int y = r / kVjpChunksZ, k = r - y * kVjpChunksZ;
     const int gx = (ox + x - 2) & wrap, gy = (oy + y - 2) & wrap, gz = (oz - 4 + 4 * k) & wrap;
     vjp_cp_async16(sp + x * kVjpSX + y * kVjpSY + 4 * k, phi + ((size_t)gx * nm + gy) * (size_t)row_pitch + gz);
+  }
+  for (int c = t; c < kVjpStageB; c += kVjpThreads) {
+    const int x = c / (kVjpSpanB * (kVjpSpanBZ / 4)), r = c - x * (kVjpSpanB * (kVjpSpanBZ / 4));
+    const int y = r / (kVjpSpanBZ / 4), k = r - y * (kVjpSpanBZ / 4);
+    const int gx = (ox + x) & wrap, gy = (oy + y) & wrap, gz = (oz + 4 * k) & wrap;
+    vjp_cp_async16(sb + x * kVjpBSX + y * kVjpBSY + 4 * k, B + ((size_t)gx * nm + gy) * (size_t)row_pitch + gz);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
   asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -174,6 +193,15 @@ __global__ void __launch_bounds__(kVjpThreads) k_readout_grad_fd4(
     const float fx = (float)(ux & fmask) * fscale, fy = (float)(uy & fmask) * fscale,
                 fz = (float)(uz & fmask) * fscale;
     const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
+    // CIC derivative of corner values v[a][b][c]
+    auto grad = [&](const float (*v)[2][2], float& dX, float& dY, float& dZ) {
+      dX = gy * (gz * (v[1][0][0] - v[0][0][0]) + fz * (v[1][0][1] - v[0][0][1])) +
+           fy * (gz * (v[1][1][0] - v[0][1][0]) + fz * (v[1][1][1] - v[0][1][1]));
+      dY = gx * (gz * (v[0][1][0] - v[0][0][0]) + fz * (v[0][1][1] - v[0][0][1])) +
+           fx * (gz * (v[1][1][0] - v[1][0][0]) + fz * (v[1][1][1] - v[1][0][1]));
+      dZ = gx * (gy * (v[0][0][1] - v[0][0][0]) + fy * (v[0][1][1] - v[0][1][0])) +
+           fx * (gy * (v[1][0][1] - v[1][0][0]) + fy * (v[1][1][1] - v[1][1][0]));
+    };
     const float* q = sp + (lx + 2) * kVjpSX + (ly + 2) * kVjpSY + (lz + 4);
     // F_j at corner (a, b, c) of the cell, Fj[a][b][c] = -S_j phi / ... (scaled below)
     float Fx[2][2][2], Fy[2][2][2], Fz[2][2][2];
@@ -191,29 +219,206 @@ __global__ void __launch_bounds__(kVjpThreads) k_readout_grad_fd4(
         line(q + a * kVjpSX + b * kVjpSY, 1, Fz[a][b][0], Fz[a][b][1]);  // z line at (x, y) = (a, b)
       }
     }
-    const float l0 = lam[i], l1 = lam[n + i], l2 = lam[2 * n + i];
     float o[3] = {0.f, 0.f, 0.f};
     const float (*Fs[3])[2][2] = {Fx, Fy, Fz};
-    const float ls[3] = {l0, l1, l2};
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      const float (*v)[2][2] = Fs[j];
-      const float dX = gy * (gz * (v[1][0][0] - v[0][0][0]) + fz * (v[1][0][1] - v[0][0][1])) +
-                       fy * (gz * (v[1][1][0] - v[0][1][0]) + fz * (v[1][1][1] - v[0][1][1]));
-      const float dY = gx * (gz * (v[0][1][0] - v[0][0][0]) + fz * (v[0][1][1] - v[0][0][1])) +
-                       fx * (gz * (v[1][1][0] - v[1][0][0]) + fz * (v[1][1][1] - v[1][0][1]));
-      const float dZ = gx * (gy * (v[0][0][1] - v[0][0][0]) + fy * (v[0][1][1] - v[0][1][0])) +
-                       fx * (gy * (v[1][0][1] - v[1][0][0]) + fy * (v[1][1][1] - v[1][1][0]));
-      o[0] += ls[j] * dX;
-      o[1] += ls[j] * dY;
-      o[2] += ls[j] * dZ;
+      float dX, dY, dZ;
+      grad(Fs[j], dX, dY, dZ);
+      const float lj = lam[(int64_t)j * n + i];
+      o[0] += lj * dX;
+      o[1] += lj * dY;
+      o[2] += lj * dZ;
     }
+    const float* qb = sb + lx * kVjpBSX + ly * kVjpBSY + lz;
+    float vb[2][2][2], bX, bY, bZ;
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) vb[a][b][c] = qb[a * kVjpBSX + b * kVjpBSY + c];
+    grad(vb, bX, bY, bZ);
+    const float m = id_mass(mt, ids[i], PM_SPECIES_ALL, &bad) * inv_h;
     const int64_t dst = perm ? (int64_t)perm[i] : (int64_t)i;
     const float scale = -inv12h * inv_h;  // F_j = -(stencil sum) / (12 H); d/dx: 1 / H
-#pragma unroll
-    for (int d = 0; d < 3; ++d) out[(int64_t)d * n + dst] = scale * o[d];
+    out[dst] = fmaf(scale, o[0], m * bX);
+    out[n + dst] = fmaf(scale, o[1], m * bY);
+    out[2 * n + dst] = fmaf(scale, o[2], m * bZ);
   }
   if (bad) atomicOr(err, 1);
+}
+
+// One mesh's or three meshes' worth of the VJP, staged per tile like B above (the learned path):
+// NM = 1: tmp[d][i] = m_i d/dx_d R[B](x_i) in sorted order; NM = 3: out[d][perm[i]] = tmp[d][i] +
+// sum_j lambda_j(i) d/dx_d R[F_j](x_i).  Staging replaces 8 NM scattered global reads a particle.
+template <int NM>
+__global__ void __launch_bounds__(kVjpThreads) k_vjp_readout(
+    const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n, const uint32_t* __restrict__ bstart,
+    const float* __restrict__ m0, const float* __restrict__ m1, const float* __restrict__ m2, int nm, int shift,
+    int ntl, int row_pitch, float inv_h, const float* __restrict__ lam, MassTable mt,
+    const uint32_t* __restrict__ perm, float* __restrict__ tmp, float* __restrict__ out, int* __restrict__ err) {
+  extern __shared__ __align__(16) float sb[];
+  const int t = threadIdx.x;
+  const uint32_t tile = blockIdx.x;
+  const uint32_t lo = bstart[8 * tile], hi = bstart[8 * tile + 8];
+  if (lo == hi) return;
+  const int nt = 1 << ntl;
+  const int ox = (int)(tile >> (2 * ntl)) * kTile, oy = (int)((tile >> ntl) & (nt - 1)) * kTile,
+            oz = (int)(tile & (nt - 1)) * kTile;
+  const int wrap = nm - 1;
+#pragma unroll
+  for (int j = 0; j < NM; ++j) {
+    const float* const M = j == 0 ? m0 : (j == 1 ? m1 : m2);
+    float* const dst = sb + j * kVjpSpanB * kVjpBSX;
+    for (int c = t; c < kVjpStageB; c += kVjpThreads) {
+      const int x = c / (kVjpSpanB * (kVjpSpanBZ / 4)), r = c - x * (kVjpSpanB * (kVjpSpanBZ / 4));
+      const int y = r / (kVjpSpanBZ / 4), k = r - y * (kVjpSpanBZ / 4);
+      const int gx = (ox + x) & wrap, gy = (oy + y) & wrap, gz = (oz + 4 * k) & wrap;
+      vjp_cp_async16(dst + x * kVjpBSX + y * kVjpBSY + 4 * k, M + ((size_t)gx * nm + gy) * (size_t)row_pitch + gz);
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  const float fscale = 1.0f / (float)(1u << shift);
+  const uint32_t fmask = (1u << shift) - 1u;
+  bool bad = false;
+  for (uint32_t i = lo + t; i < hi; i += kVjpThreads) {
+    const uint32_t ux = us[i], uy = us[n + i], uz = us[2 * n + i];
+    const int lx = (int)(ux >> shift) - ox, ly = (int)(uy >> shift) - oy, lz = (int)(uz >> shift) - oz;
+    if ((unsigned)lx >= (unsigned)kTile || (unsigned)ly >= (unsigned)kTile || (unsigned)lz >= (unsigned)kTile) {
+      bad = true;
+      continue;
+    }
+    const float fx = (float)(ux & fmask) * fscale, fy = (float)(uy & fmask) * fscale,
+                fz = (float)(uz & fmask) * fscale;
+    const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
+    float o[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < NM; ++j) {
+      const float a = NM == 1 ? id_mass(mt, ids[i], PM_SPECIES_ALL, &bad) : lam[(int64_t)j * n + i];
+      const float* const q = sb + j * kVjpSpanB * kVjpBSX + lx * kVjpBSX + ly * kVjpBSY + lz;
+      const float v000 = q[0], v001 = q[1], v010 = q[kVjpBSY], v011 = q[kVjpBSY + 1];
+      const float v100 = q[kVjpBSX], v101 = q[kVjpBSX + 1], v110 = q[kVjpBSX + kVjpBSY],
+                  v111 = q[kVjpBSX + kVjpBSY + 1];
+      const float dX = gy * (gz * (v100 - v000) + fz * (v101 - v001)) +
+                       fy * (gz * (v110 - v010) + fz * (v111 - v011));
+      const float dY = gx * (gz * (v010 - v000) + fz * (v011 - v001)) +
+                       fx * (gz * (v110 - v100) + fz * (v111 - v101));
+      const float dZ = gx * (gy * (v001 - v000) + fy * (v011 - v010)) +
+                       fx * (gy * (v101 - v100) + fy * (v111 - v110));
+      o[0] += a * dX;
+      o[1] += a * dY;
+      o[2] += a * dZ;
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int64_t k = (int64_t)d * n + i;
+      if constexpr (NM == 1) {
+        tmp[k] = o[d] * inv_h;
+      } else {
+        out[(int64_t)d * n + perm[i]] = fmaf(o[d], inv_h, tmp[k]);
+      }
+    }
+  }
+  if (bad) atomicOr(err, 1);
+}
+
+// C <- S_x A + S_y B + S_z C on real meshes (row pitch rp): the divergence of the painted
+// cotangents with the 4-point stencil, periodic, in place on the third.  A thread takes four
+// cells along z and walks kDivSteps planes along x with the five A values it needs in
+// registers; its CTA holds whole rows of C, read before any is written.  One pass over the
+// three meshes: three single-axis passes that add into one mesh took 307 us at 256^3.
+constexpr int kDivThreads = 256;
+constexpr int kDivSteps = 8;
+__global__ void __launch_bounds__(kDivThreads) k_stencil_div(const float* __restrict__ A, const float* __restrict__ B,
+                                                             float* C, int nm, int rp, float inv12h) {
+  const int quads = nm / 4, rows = kDivThreads / quads;  // rows of z quads a CTA (nm <= 1024)
+  const int q = threadIdx.x % quads, z = 4 * q, w = nm - 1;
+  const int y = (blockIdx.x % (nm / rows)) * rows + threadIdx.x / quads;
+  const int x0 = (blockIdx.x / (nm / rows)) * kDivSteps;
+  auto at = [&](const float* M, int x, int yy, int zz) -> float4 {
+    return *reinterpret_cast<const float4*>(M + ((size_t)(x & w) * nm + (yy & w)) * rp + (zz & w));
+  };
+  float4 a[5];  // A at x - 2 .. x + 2
+#pragma unroll
+  for (int k = 0; k < 4; ++k) a[k + 1] = at(A, x0 - 2 + k, y, z);
+  for (int s = 0; s < kDivSteps; ++s) {
+    const int x = x0 + s;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = a[k + 1];
+    a[4] = at(A, x + 2, y, z);
+    const float4 b0 = at(B, x, y - 2, z), b1 = at(B, x, y - 1, z), b3 = at(B, x, y + 1, z), b4 = at(B, x, y + 2, z);
+    const float4 c0 = at(C, x, y, z - 4), c1 = at(C, x, y, z), c2 = at(C, x, y, z + 4);
+    auto st = [](float m2, float m1, float p1, float p2) { return 8.0f * (p1 - m1) - (p2 - m2); };
+    float4 r;
+    r.x = st(a[0].x, a[1].x, a[3].x, a[4].x) + st(b0.x, b1.x, b3.x, b4.x) + st(c0.z, c0.w, c1.y, c1.z);
+    r.y = st(a[0].y, a[1].y, a[3].y, a[4].y) + st(b0.y, b1.y, b3.y, b4.y) + st(c0.w, c1.x, c1.z, c1.w);
+    r.z = st(a[0].z, a[1].z, a[3].z, a[4].z) + st(b0.z, b1.z, b3.z, b4.z) + st(c1.x, c1.y, c1.w, c2.x);
+    r.w = st(a[0].w, a[1].w, a[3].w, a[4].w) + st(b0.w, b1.w, b3.w, b4.w) + st(c1.y, c1.z, c2.x, c2.y);
+    __syncthreads();  // the row's C values are read
+    *reinterpret_cast<float4*>(C + ((size_t)x * nm + y) * rp + z) =
+        make_float4(inv12h * r.x, inv12h * r.y, inv12h * r.z, inv12h * r.w);
+  }
+}
+
+// The same divergence from the three half spectra, C <- i (D_x A + D_y B + D_z C): the learned
+// path's form.  The factor's gradient weighs the largest scales by 1 / k^2, and there the
+// transform of the real-space divergence has lost digits to its smallest scales.
+__global__ void __launch_bounds__(256) k_spectrum_div(const float2* __restrict__ A, const float2* __restrict__ B,
+                                                      float2* __restrict__ C, int nm, int pc,
+                                                      const float* __restrict__ kvec0) {
+  const long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);  // x N + y: a warp a row
+  const float kx = __ldg(kvec0 + row / nm), ky = __ldg(kvec0 + row % nm);
+  for (int kz = threadIdx.x & 31; kz <= nm / 2; kz += 32) {
+    const size_t i = (size_t)row * pc + kz;
+    const float kq = __ldg(kvec0 + kz);
+    const float2 a = A[i], b = B[i], c = C[i];
+    C[i] = make_float2(-(kx * a.y + ky * b.y + kq * c.y), kx * a.x + ky * b.x + kq * c.x);
+  }
+}
+
+// The learned factor's part of the force VJP between the transforms: rho (the density's half
+// spectrum) and C = FFT(sum_j S_j paint(lambda_j)) become the spectra of the two potentials,
+// rho <- g m rho, C <- g m C, and d <lambda_F, F> / d m(k) = g Re[rho_k conj(C_k)] (twice for
+// 0 < k_z < N/2) is added to gbin by s = |n|^2.  The rows (+-n_x, +-n_y), (+-n_y, +-n_x) share
+// g, m and s: a warp takes all of them, its lanes walk k_z, and one FP64 atomic serves eight
+// modes (their products added error-free in FP32 pairs).
+__global__ void __launch_bounds__(256) k_vjp_combine(float2* __restrict__ rho, float2* __restrict__ C, int nm, int pc,
+                                                     int units, const float* __restrict__ ksq,
+                                                     const float* __restrict__ winv, float gcoef,
+                                                     const float* __restrict__ mtab, double* __restrict__ gbin) {
+  const int wu = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31, half = nm / 2;
+  if (wu >= units) return;
+  int a = (int)((sqrtf(8.0f * (float)wu + 1.0f) - 1.0f) * 0.5f);  // (a, b), 0 <= b <= a <= N/2
+  while (a * (a + 1) / 2 > wu) --a;
+  while ((a + 1) * (a + 2) / 2 <= wu) ++a;
+  const int b = wu - a * (a + 1) / 2;
+  const bool ra = a != 0 && a != half, rb = b != 0 && b != half, rs = a != b;
+  const float kab = ksq[a] + ksq[b], wab = winv[a] * winv[b];
+  for (int kz = lane; kz <= half; kz += 32) {
+    const int s = a * a + b * b + kz * kz;
+    const float k2 = kab + ksq[kz];
+    const float g = k2 == 0.0f ? 0.0f : gcoef * wab * winv[kz] / k2;
+    const float gm = g * mtab[s];
+    float sum = 0.0f, e = 0.0f;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      if (((r & 1) && !ra) || ((r & 2) && !rb) || ((r & 4) && !rs)) continue;
+      const int ia = (r & 1) ? nm - a : a, ib = (r & 2) ? nm - b : b;
+      const size_t idx = ((size_t)((r & 4) ? ib : ia) * nm + ((r & 4) ? ia : ib)) * pc + kz;
+      const float2 v = rho[idx], c = C[idx];
+      const float p = v.x * c.x + v.y * c.y;
+      const float t = sum + p, d = t - sum;  // Knuth's two-sum
+      e += (sum - (t - d)) + (p - d);
+      sum = t;
+      rho[idx] = cscale(v, gm);
+      C[idx] = cscale(c, gm);
+    }
+    const float q = ((kz > 0 && kz < half) ? 2.0f : 1.0f) * g;
+    if (q != 0.0f) atomicAdd(gbin + s, (double)q * ((double)sum + (isfinite(sum) ? (double)e : 0.0)));
+  }
 }
 
 // B (+)= S_j A on real meshes (row pitch rp): the 4-point stencil along axis j, periodic.
@@ -233,39 +438,50 @@ __global__ void k_stencil_axis(const float* __restrict__ A, float* __restrict__ 
   }
 }
 
-// u1 = u0 + rne(Delta (p0 + K1 f0) 2^32 / L), p_h = p0 + K1 f0 (no sort keys)
-__global__ void k_drift_only(const uint32_t* __restrict__ u0, const float* __restrict__ p0,
-                             const float* __restrict__ f0, int64_t n, float K1, float dscale,
-                             uint32_t* __restrict__ u1) {
+// Start of a step's VJP, in state order: the cotangents by id, the drifted positions
+// u1 = u0 + rne(Delta (p0 + K1 f0) 2^32 / L) and the force cotangent K2 lambda_p of x1.
+__global__ void k_vjp_begin(const float* __restrict__ lx1, const float* __restrict__ lp1,
+                            const uint32_t* __restrict__ id, const uint32_t* __restrict__ u0,
+                            const float* __restrict__ p0, const float* __restrict__ f0, int64_t n, float K1,
+                            float dscale, float K2, float* __restrict__ Lx, float* __restrict__ Lp,
+                            float* __restrict__ lamF, uint32_t* __restrict__ u1) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  const int64_t j = (int64_t)id[i];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
+    const float lp = lp1[d * n + j];
+    Lx[d * n + i] = lx1[d * n + j];
+    Lp[d * n + i] = lp;
+    lamF[d * n + i] = K2 * lp;
     const float ph = p0[d * n + i] + K1 * f0[d * n + i];
-    const long long step = __float2ll_rn(dscale * ph);
-    u1[d * n + i] = u0[d * n + i] + (uint32_t)(unsigned long long)step;
+    u1[d * n + i] = u0[d * n + i] + (uint32_t)(unsigned long long)__float2ll_rn(dscale * ph);
   }
 }
 
-// dst[d][i] = src[d][id[i]] (canonical -> state order) or dst[d][id[i]] = src[d][i]
-__global__ void k_by_id(const float* __restrict__ src, float* __restrict__ dst,
-                        const uint32_t* __restrict__ id, int64_t n, int to_canonical, float scale) {
+// Between the two force VJPs, over 3n: Lx += g, Lp += Delta Lx, lamF = K1 Lp.
+__global__ void k_vjp_middle(const float* __restrict__ g, int64_t m, float delta, float K1, float* __restrict__ Lx,
+                             float* __restrict__ Lp, float* __restrict__ lamF) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= m) return;
+  const float x = Lx[i] + g[i], p = fmaf(delta, x, Lp[i]);
+  Lx[i] = x;
+  Lp[i] = p;
+  lamF[i] = K1 * p;
+}
+
+// End: lx0 = Lx + g and lp0 = Lp in canonical order.
+__global__ void k_vjp_end(const float* __restrict__ g, const float* __restrict__ Lx, const float* __restrict__ Lp,
+                          const uint32_t* __restrict__ id, int64_t n, float* __restrict__ lx0,
+                          float* __restrict__ lp0) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int64_t j = id ? (int64_t)id[i] : i;
+  const int64_t j = (int64_t)id[i];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    if (to_canonical)
-      dst[d * n + j] = scale * src[d * n + i];
-    else
-      dst[d * n + i] = scale * src[d * n + j];
+    lx0[d * n + j] = Lx[d * n + i] + g[d * n + i];
+    lp0[d * n + j] = Lp[d * n + i];
   }
-}
-
-// y = a x + b y over 3n
-__global__ void k_axpby(const float* __restrict__ x, float* __restrict__ y, int64_t m, float a, float b) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m) y[i] = a * x[i] + b * y[i];
 }
 
 // gather per-component weights into the sorted order: ws[j][k] = w[j][perm[k]]
@@ -394,26 +610,86 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
   float* realA = reinterpret_cast<float*>(c->meshA);
   float* realB = reinterpret_cast<float*>(c->meshB);
   const int rp = 2 * c->g.pc;
-  if (!learned && (c->cfg.flags & (PM_FLAG_SPECTRAL_KERNEL | PM_FLAG_KSPACE_GRADIENT)) == 0) {
-    // one mesh at a time, five FFT passes a term (see k_readout_grad_fd4)
+  if ((c->cfg.flags & (PM_FLAG_SPECTRAL_KERNEL | PM_FLAG_KSPACE_GRADIENT)) == 0) {
+    // two potentials, phi in realA and B in pot (see k_force_vjp_readout)
     const float inv12h = (float)((double)c->g.n / (12.0 * c->cfg.box));
     const float inv_h = (float)(c->g.n / c->cfg.box);
+    float2* const pot = c->meshC ? c->meshC : c->meshB;
+    float* const realP = reinterpret_cast<float*>(pot);
+    if (c->meshC) {
+      paint_weights3(c, c->us, n, lam_s, realA, realB, realP, rp, s);
+      if (learned) {
+        fft_forward(c, c->g, c->meshA, c->meshA, 0, s);
+        fft_forward(c, c->g, c->meshB, c->meshB, 0, s);
+        fft_forward(c, c->g, pot, pot, 0, s);
+      }
+      LaunchScope L(c, s, K_ADJOINT);
+      const int rows = kDivThreads / (c->g.n / 4);
+      if (learned)
+        k_spectrum_div<<<(unsigned)(c->g.rows() / 8), 256, 0, s>>>(c->meshA, c->meshB, pot, c->g.n, c->g.pc, c->kvec0);
+      else
+        k_stencil_div<<<(unsigned)(c->g.n / rows * (c->g.n / kDivSteps)), kDivThreads, 0, s>>>(
+            realA, realB, realP, c->g.n, rp, inv12h);
+    } else {  // two meshes: one component at a time
+      for (int j = 0; j < 3; ++j) {
+        paint_tiles(c, c->us, c->ids, n, PM_SPECIES_ALL, realA, rp, s, lam_s + (int64_t)j * n);
+        LaunchScope L(c, s, K_ADJOINT);
+        k_stencil_axis<<<(unsigned)(c->g.n * c->g.n), 256, 0, s>>>(realA, realP, c->g.n, rp, j, inv12h, j > 0);
+      }
+    }
     paint_tiles(c, c->us, c->ids, n, PM_SPECIES_ALL, realA, rp, s);
+    if (learned) {
+      mlp_table(c, a, s);
+      fft_forward(c, c->g, c->meshA, c->meshA, 0, s);
+      {
+        LaunchScope L(c, s, K_ADJOINT);
+        const double nn = (double)c->g.n;
+        const int units = (c->g.n / 2 + 1) * (c->g.n / 2 + 2) / 2;
+        k_vjp_combine<<<(units + 7) / 8, 256, 0, s>>>(c->meshA, pot, c->g.n, c->g.pc, units, c->ksq, c->wforce,
+                                                      (float)(-1.5 * c->cosmo.omega_m0 / (nn * nn * nn)), c->mlp_tab,
+                                                      c->mlp_gbin);
+      }
+      fft_inverse_plain(c, c->g, pot, s);  // B
+      const size_t sm1 = sizeof(float) * kVjpSpanB * kVjpBSX;
+      static bool attr3 = false;
+      if (!attr3) {
+        cudaFuncSetAttribute(k_vjp_readout<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(3 * sm1));
+        attr3 = true;
+      }
+      const unsigned tiles = (unsigned)(c->nt * c->nt * c->nt);
+      float* const tmp = c->adj + 7 * 3 * n;  // the second term, sorted order
+      {
+        LaunchScope L(c, s, K_ADJOINT);
+        k_vjp_readout<1><<<tiles, kVjpThreads, sm1, s>>>(c->us, c->ids, n, c->bstart, realP, nullptr, nullptr, c->g.n,
+                                                        32 - c->g.logn, c->ntl, rp, inv_h, nullptr, c->mt, nullptr, tmp,
+                                                        nullptr, c->err_dev);
+      }
+      // F_y, F_z into the other meshes, F_x in place over phi_k
+      fft_inverse_component(c, c->g, c->meshA, c->meshB, 1, s);
+      fft_inverse_component(c, c->g, c->meshA, pot, 2, s);
+      fft_inverse_component(c, c->g, c->meshA, c->meshA, 0, s);
+      {
+        LaunchScope L(c, s, K_ADJOINT);
+        k_vjp_readout<3><<<tiles, kVjpThreads, 3 * sm1, s>>>(c->us, c->ids, n, c->bstart, realA, realB, realP, c->g.n,
+                                                            32 - c->g.logn, c->ntl, rp, inv_h, lam_s, c->mt,
+                                                            c->vals[0], tmp, grad, c->err_dev);
+      }
+      mlp_backward(c, a, s);
+      return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ECUDA;
+    }
     fft_potential(c, c->g, c->meshA, s);
+    fft_potential(c, c->g, pot, s);
+    static bool attr = false;
+    if (!attr) {
+      cudaFuncSetAttribute(k_force_vjp_readout, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVjpSmem);
+      attr = true;
+    }
     {
       LaunchScope L(c, s, K_ADJOINT);
-      k_readout_grad_fd4<<<(unsigned)(c->nt * c->nt * c->nt), kVjpThreads, 0, s>>>(
-          c->us, n, c->bstart, realA, c->g.n, 32 - c->g.logn, c->ntl, rp, inv12h, inv_h, lam_s, c->vals[0], grad,
-          c->err_dev);
+      k_force_vjp_readout<<<(unsigned)(c->nt * c->nt * c->nt), kVjpThreads, kVjpSmem, s>>>(
+          c->us, c->ids, n, c->bstart, realA, realP, c->g.n, 32 - c->g.logn, c->ntl, rp, inv12h, inv_h, lam_s, c->mt,
+          c->vals[0], grad, c->err_dev);
     }
-    for (int j = 0; j < 3; ++j) {
-      paint_tiles(c, c->us, c->ids, n, PM_SPECIES_ALL, realA, rp, s, lam_s + (int64_t)j * n);
-      LaunchScope L(c, s, K_ADJOINT);
-      k_stencil_axis<<<(unsigned)(c->g.n * c->g.n), 256, 0, s>>>(realA, realB, c->g.n, rp, j, inv12h, j > 0);
-    }
-    fft_potential(c, c->g, c->meshB, s);
-    const float* m[1] = {realB};
-    readout_grad(c, n, m, 1, rp, nullptr, c->vals[0], grad, true, s);
     return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ECUDA;
   }
   // term 1: sum_j lambda_j grad R[G_j rho]
@@ -462,30 +738,23 @@ int step_vjp(pm_ctx* c, const pm_state* st, double a0, double ah, double a1, con
   float* lamF = c->adj + 2 * m3;
   float* g = c->adj + 3 * m3;
   uint32_t* u1 = reinterpret_cast<uint32_t*>(c->adj + 4 * m3);
-#define ADJ(launch)                      \
-  do {                                   \
-    LaunchScope L_(c, s, K_ADJOINT);     \
-    launch;                              \
-  } while (0)
-  ADJ((k_by_id<<<blocks(n), 256, 0, s>>>(lx1, Lx, st->id, n, 0, 1.0f)));
-  ADJ((k_by_id<<<blocks(n), 256, 0, s>>>(lp1, Lp, st->id, n, 0, 1.0f)));
-  ADJ((k_drift_only<<<blocks(n), 256, 0, s>>>(st->u, st->p, st->f, n, (float)k[0],
-                                              (float)(k[1] * 4294967296.0 / c->cfg.box), u1)));
-  // lambda_x1' = lambda_x1 + F_vjp(x1; K2 lambda_p1)
-  ADJ((k_by_id<<<blocks(n), 256, 0, s>>>(Lp, lamF, nullptr, n, 0, (float)k[2])));
+  {  // lambda_F of x1: K2 lambda_p1
+    LaunchScope L(c, s, K_ADJOINT);
+    k_vjp_begin<<<blocks(n), 256, 0, s>>>(lx1, lp1, st->id, st->u, st->p, st->f, n, (float)k[0],
+                                          (float)(k[1] * 4294967296.0 / c->cfg.box), (float)k[2], Lx, Lp, lamF, u1);
+  }
   rc = force_vjp(c, u1, st->id, n, lamF, a1, g, s);
   if (rc != PM_OK) return rc;
-  ADJ((k_axpby<<<blocks(m3), 256, 0, s>>>(g, Lx, m3, 1.0f, 1.0f)));
-  // lambda_ph = lambda_p1 + Delta lambda_x1'
-  ADJ((k_axpby<<<blocks(m3), 256, 0, s>>>(Lx, Lp, m3, (float)k[1], 1.0f)));
-  // lambda_x0 = lambda_x1' + F_vjp(x0; K1 lambda_ph)
-  ADJ((k_by_id<<<blocks(n), 256, 0, s>>>(Lp, lamF, nullptr, n, 0, (float)k[0])));
+  {  // lambda_x1' = lambda_x1 + F_vjp(x1), lambda_ph = lambda_p1 + Delta lambda_x1', lambda_F of x0: K1 lambda_ph
+    LaunchScope L(c, s, K_ADJOINT);
+    k_vjp_middle<<<blocks(m3), 256, 0, s>>>(g, m3, (float)k[1], (float)k[0], Lx, Lp, lamF);
+  }
   rc = force_vjp(c, st->u, st->id, n, lamF, a0, g, s);
   if (rc != PM_OK) return rc;
-  ADJ((k_axpby<<<blocks(m3), 256, 0, s>>>(g, Lx, m3, 1.0f, 1.0f)));
-  ADJ((k_by_id<<<blocks(n), 256, 0, s>>>(Lx, lx0, st->id, n, 1, 1.0f)));
-  ADJ((k_by_id<<<blocks(n), 256, 0, s>>>(Lp, lp0, st->id, n, 1, 1.0f)));
-#undef ADJ
+  {  // lambda_x0 = lambda_x1' + F_vjp(x0)
+    LaunchScope L(c, s, K_ADJOINT);
+    k_vjp_end<<<blocks(n), 256, 0, s>>>(g, Lx, Lp, st->id, n, lx0, lp0);
+  }
   return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ECUDA;
 }
 

@@ -16,8 +16,10 @@
 // 256 mean cell masses, so nearly every corner costs one 32-bit shared atomic (those
 // run ~4x faster than 64-bit ones, and the 32-bit conversions of the write-out avoid
 // the narrow FP64 pipe that 64-bit float <-> integer conversions use).  Masses of 128
-// or more and the signed weights of the adjoint use one 64-bit accumulator instead
-// (resolution 2^-24 for masses, so both forms give the same bits; 2^-32 for weights).
+// or more and the signed weights of the adjoint are 64-bit integers in the same two words
+// (resolution 2^-24 for masses, so both forms give the same bits; 2^-32 for weights): the
+// low word is added with a 32-bit atomic and the high word only when it changes, which for
+// weights is when a cell's sum crosses a multiple of 2^32.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -63,36 +65,60 @@ __device__ __noinline__ bool record_wrap(unsigned int* accw, unsigned int ad) {
   return true;
 }
 
+// __float2ll_rn without the narrow FP64 pipe: below 2^31 the 32-bit conversion (same rounding),
+// above it the value is an integer already (24-bit mantissa), so shift the mantissa.
+__device__ __forceinline__ long long fixed64(float x) {
+  if (fabsf(x) < 2147483648.0f) return (long long)__float2int_rn(x);
+  if (!(fabsf(x) < 9.0e18f)) return __float2ll_rn(x);  // saturation, NaN
+  const uint32_t bits = __float_as_uint(x);
+  const long long m = (long long)(unsigned long long)((bits & 0x7fffffu) | 0x800000u) << (((bits >> 23) & 255u) - 150u);
+  return (bits >> 31) ? -m : m;
+}
+
+// 64-bit sum in two 32-bit words: lo += low word of q, hi += high word + carry (only if not 0)
+__device__ __forceinline__ void add64(unsigned int* lo, unsigned int* hi, long long q) {
+  const unsigned int ql = (unsigned int)q, old = atomicAdd(lo, ql);
+  const unsigned int h = (unsigned int)(q >> 32) + (old + ql < old ? 1u : 0u);
+  if (h) atomicAdd(hi, h);
+}
+
+// __ll2float_rn of the two-word sum; the usual cases (|value| < 2^32) by 32-bit conversions
+__device__ __forceinline__ float float64w(unsigned int hi, unsigned int lo) {
+  if (hi == 0u) return __uint2float_rn(lo);
+  if (hi == 0xffffffffu && lo != 0u) return -__uint2float_rn(0u - lo);
+  return __ll2float_rn((long long)(((unsigned long long)hi << 32) | (unsigned long long)lo));
+}
+
 // Paint of one tile.  FAST: 32-bit low words only (half the shared memory of the carry form:
 // zeroed, and read at the write-out, once per cell).  A low word that wraps past 2^32 (the
 // cell passes another 256 mean cell masses) is recorded as an event -- the cell's bit in a
 // bitmap, its index in a list of up to kWraps events -- and at the write-out a cell whose
 // bit is set counts its events in the list: value = events 2^32 + low word.  A tile with
 // more events than the list holds is written to the redo list and left unwritten; the redo
-// pass paints it in full with the 32-bit carry (or 64-bit) form.  Every form sums the same
-// exact integers, so all give the same floats.
-template <bool FAST>
+// pass paints it in full in the two-word form.  Every form sums the same exact integers, so
+// all give the same floats.  Else two words a cell and NW = 0 (masses), or NW = 1 or 3 signed
+// weights a particle (wts[j n + k]), weight j painted onto mesh j (mesh, mesh1, mesh2).
+template <bool FAST, int NW, int NT>
 __device__ __forceinline__ void paint_tile(
     uint32_t tile, unsigned int* __restrict__ accw, uint32_t* __restrict__ run_lo, uint32_t* __restrict__ run_pre,
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
     const uint32_t* __restrict__ bstart, float* __restrict__ mesh, const MassTable& mt, int species, int nm,
     int shift, int ntl, int row_pitch, int* __restrict__ err, const float* __restrict__ wts, float mmax,
-    uint32_t* __restrict__ redo) {
-  // FAST: low words, then the wrap bitmap, the event count and the event list.  Else one
-  // 64-bit accumulator, or the same bytes as two 32-bit halves (hi words, then lo words) in the
-  // carry form.
-  long long* const acc = reinterpret_cast<long long*>(accw);
-  unsigned int* const acc_hi = accw;
-  unsigned int* const acc_lo = FAST ? accw : accw + kAccWords;
+    uint32_t* __restrict__ redo, float* __restrict__ mesh1 = nullptr, float* __restrict__ mesh2 = nullptr) {
+  constexpr int NA = NW > 1 ? NW : 1;  // meshes painted
+  // FAST: low words, then the wrap bitmap, the event count and the event list.  Else per
+  // mesh the low words, then the high words.
+  unsigned int* const acc_lo = accw;
   volatile unsigned int* const wbits = accw + kAccWords;          // FAST: kWrapBits words
   unsigned int* const wcount = accw + kAccWords + kWrapBits;       // FAST: one word
   volatile unsigned short* const wlist = reinterpret_cast<unsigned short*>(accw + kAccWords + kWrapBits + 1);
   const int t = threadIdx.x;
   if constexpr (FAST) {
-    for (int i = t; i < (kAccWords + kWrapBits + 1) / 4 + 1; i += kPaintThreads)
+    for (int i = t; i < (kAccWords + kWrapBits + 1) / 4 + 1; i += NT)
       reinterpret_cast<uint4*>(accw)[i] = make_uint4(0, 0, 0, 0);
   } else {
-    for (int i = t; i < kAccWords; i += kPaintThreads) acc[i] = 0;
+    static_assert(kAccWords % 2 == 0, "whole 16-byte groups");
+    for (int i = t; i < NA * kAccWords / 2; i += NT) reinterpret_cast<uint4*>(accw)[i] = make_uint4(0, 0, 0, 0);
   }
   const int nt = 1 << ntl;
   const int tx = tile >> (2 * ntl), ty = (tile >> ntl) & (nt - 1), tz = tile & (nt - 1);
@@ -124,40 +150,41 @@ __device__ __forceinline__ void paint_tile(
   const uint32_t total = run_pre[14];
   // One particle per thread (coalesced loads in bucket order), its 8 corners added by
   // the same thread.
-  // carry form: 32-bit accumulators and conversions (GB300's FP64 pipe, which runs the
-  // 64-bit float <-> integer conversions, is narrow); w 2^24 < 2^31 needs mmax < 128
-  const bool carry = FAST || (wts == nullptr && mmax < 128.0f);
-  const float fix = wts ? kFixW : kFixM;
+  // masses below 128: w 2^24 < 2^31, so 32-bit conversions and a carry of at most 1
+  const bool narrow = FAST || (NW == 0 && mmax < 128.0f);
   const int ox = tx * kTile, oy = ty * kTile, oz = tz * kTile;
   bool bad = false, wrap = false;
   int r = 0;
-  // the particle of iteration v + kPaintThreads is loaded while v's corners are added
+  // the particle of iteration v + NT is loaded while v's corners are added
   auto locate = [&](uint32_t v) {
     while (v >= run_pre[r + 1]) ++r;  // v only grows, so the run index only grows
     return run_lo[r] + (v - run_pre[r]);
   };
-  uint32_t k = 0, qid = 0, qu0 = 0, qu1 = 0, qu2 = 0;
-  float qw = 0.0f;
-  if ((uint32_t)t < total) {
-    k = locate(t);
-    if (wts) qw = wts[k]; else qid = ids[k];
+  uint32_t qid = 0, qu0 = 0, qu1 = 0, qu2 = 0;
+  float qw[NA];
+  auto load = [&](uint32_t k) {
+    if constexpr (NW > 0) {
+#pragma unroll
+      for (int j = 0; j < NW; ++j) qw[j] = wts[(int64_t)j * n + k];
+    } else {
+      qid = ids[k];
+    }
     qu0 = us[k];
     qu1 = us[n + k];
     qu2 = us[2 * n + k];
-  }
-  for (uint32_t v = t; v < total; v += kPaintThreads) {
+  };
+  if ((uint32_t)t < total) load(locate(t));
+  for (uint32_t v = t; v < total; v += NT) {
     const uint32_t u0 = qu0, u1 = qu1, u2 = qu2, idv = qid;
-    const float wv = qw;
-    const uint32_t vn = v + kPaintThreads;
-    if (vn < total) {
-      const uint32_t kn = locate(vn);
-      if (wts) qw = wts[kn]; else qid = ids[kn];
-      qu0 = us[kn];
-      qu1 = us[n + kn];
-      qu2 = us[2 * n + kn];
+    float m[NA];  // mass, or the signed weights
+#pragma unroll
+    for (int j = 0; j < NA; ++j) m[j] = NW > 0 ? qw[j] : 0.0f;
+    const uint32_t vn = v + NT;
+    if (vn < total) load(locate(vn));
+    if constexpr (NW == 0) m[0] = id_mass(mt, idv, species, &bad);
+    if constexpr (NW <= 1) {
+      if (m[0] == 0.0f) continue;
     }
-    const float m = wts ? wv : id_mass(mt, idv, species, &bad);  // weights: signed, sorted order
-    if (m == 0.0f) continue;
     int l[3] = {(int)(u0 >> shift) - ox, (int)(u1 >> shift) - oy, (int)(u2 >> shift) - oz};
     int lo_ok = 0;  // bit d: lower corner inside along d; bit 3 + d: upper inside
 #pragma unroll
@@ -176,21 +203,23 @@ __device__ __forceinline__ void paint_tile(
       const bool inside = ((lo_ok >> (bx ? 3 : 0)) & 1) && ((lo_ok >> (by ? 4 : 1)) & 1) &&
                           ((lo_ok >> (bz ? 5 : 2)) & 1);
       if (inside) {
-        const float w = (bx ? fx : 1.0f - fx) * (by ? fy : 1.0f - fy) * (bz ? fz : 1.0f - fz) * m;
         const int ad = cell + bx * kSx + by * kSy + bz;
-        if (carry) {
-          const unsigned int q = __float2uint_rn(w * fix);  // < 2^31: masses below 128
+        const float wc = (bx ? fx : 1.0f - fx) * (by ? fy : 1.0f - fy) * (bz ? fz : 1.0f - fz);
+        if constexpr (FAST) {
+          const unsigned int q = __float2uint_rn(wc * m[0] * kFixM);  // < 2^31: masses below 128
           const unsigned int old = atomicAdd(&acc_lo[ad], q);
-          if (old + q < old) {  // the low word wrapped
-            if constexpr (FAST) {
-              if (!record_wrap(accw, ad)) wrap = true;  // the list is full: the tile is repainted
-            } else {
-              atomicAdd(&acc_hi[ad], 1u);
-            }
-          }
+          // the low word wrapped; a full list sends the tile to the redo pass
+          if (old + q < old && !record_wrap(accw, ad)) wrap = true;
+        } else if (narrow) {
+          const unsigned int q = __float2uint_rn(wc * m[0] * kFixM);
+          const unsigned int old = atomicAdd(&acc_lo[ad], q);
+          if (old + q < old) atomicAdd(&acc_lo[kAccWords + ad], 1u);
         } else {
-          const long long q = __float2ll_rn(w * fix);
-          atomicAdd((unsigned long long*)&acc[ad], (unsigned long long)q);
+#pragma unroll
+          for (int j = 0; j < NA; ++j) {
+            unsigned int* const w = acc_lo + j * 2 * kAccWords + ad;
+            add64(w, w + kAccWords, fixed64(wc * m[j] * (NW > 0 ? kFixW : kFixM)));
+          }
         }
       }
     }
@@ -210,44 +239,42 @@ __device__ __forceinline__ void paint_tile(
   bool any_wrap = false;
   if constexpr (FAST) any_wrap = *(volatile unsigned int*)wcount != 0u;
   // write the tile: 256 rows of 16 floats, as float4
-  for (int q = t; q < kTile * kTile * kTile / 4; q += kPaintThreads) {
-    int row = q >> 2, z4 = (q & 3) * 4;
-    int lx = row >> 4, ly = row & 15;
-    const int a0 = lx * kSx + ly * kSy + z4;
-    float fv[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if constexpr (FAST) {
-        const unsigned int ad = a0 + e, lo = acc_lo[ad];
-        if (any_wrap && ((wbits[ad >> 5] >> (ad & 31)) & 1u)) {  // the cell wrapped: count its events
-          const unsigned int ne = *(volatile unsigned int*)wcount;
-          unsigned int hi = 0;
-          for (unsigned int k = 0; k < ne; ++k) hi += wlist[k] == ad ? 1u : 0u;
-          fv[e] = __ull2float_rn(((unsigned long long)hi << 32) + (unsigned long long)lo);
+  for (int j = 0; j < NA; ++j) {
+    float* const mj = j == 0 ? mesh : (j == 1 ? mesh1 : mesh2);
+    for (int q = t; q < kTile * kTile * kTile / 4; q += NT) {
+      int row = q >> 2, z4 = (q & 3) * 4;
+      int lx = row >> 4, ly = row & 15;
+      const int a0 = lx * kSx + ly * kSy + z4;
+      float fv[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const unsigned int ad = a0 + e, lo = acc_lo[j * 2 * kAccWords + ad];
+        if constexpr (FAST) {
+          if (any_wrap && ((wbits[ad >> 5] >> (ad & 31)) & 1u)) {  // the cell wrapped: count its events
+            const unsigned int ne = *(volatile unsigned int*)wcount;
+            unsigned int hi = 0;
+            for (unsigned int k = 0; k < ne; ++k) hi += wlist[k] == ad ? 1u : 0u;
+            fv[e] = __ull2float_rn(((unsigned long long)hi << 32) + (unsigned long long)lo);
+          } else {
+            fv[e] = __uint2float_rn(lo);
+          }
         } else {
-          fv[e] = __uint2float_rn(lo);
+          fv[e] = float64w(acc_lo[(j * 2 + 1) * kAccWords + ad], lo);
         }
-      } else if (carry) {
-        // value = carry 2^32 + low word: without a carry the correctly rounded 32-bit
-        // conversion is that of the 64-bit sum
-        const unsigned int hi = acc_hi[a0 + e], lo = acc_lo[a0 + e];
-        fv[e] = hi == 0u ? __uint2float_rn(lo)
-                         : __ull2float_rn(((unsigned long long)hi << 32) + (unsigned long long)lo);
-      } else {
-        fv[e] = __ll2float_rn(acc[a0 + e]);
       }
+      const float un = NW > 0 ? kUnfixW : kUnfixM;
+      float4 v = make_float4(fv[0] * un, fv[1] * un, fv[2] * un, fv[3] * un);
+      size_t off = ((size_t)(ox + lx) * nm + (oy + ly)) * (size_t)row_pitch + oz + z4;
+      *reinterpret_cast<float4*>(mj + off) = v;
     }
-    const float un = wts ? kUnfixW : kUnfixM;
-    float4 v = make_float4(fv[0] * un, fv[1] * un, fv[2] * un, fv[3] * un);
-    size_t off = ((size_t)(ox + lx) * nm + (oy + ly)) * (size_t)row_pitch + oz + z4;
-    *reinterpret_cast<float4*>(mesh + off) = v;
   }
 }
 
 // One CTA per tile.  FAST: the 32-bit form with wrap events, tiles whose event list
-// overflows sent to the redo list (redo[0] = count, redo[1 ..] = tiles); else the carry or
-// 64-bit form.
-template <bool FAST>
+// overflows sent to the redo list (redo[0] = count, redo[1 ..] = tiles); else the two-word
+// form, with NW signed weights instead of masses when NW > 0.
+template <bool FAST, int NW>
 __global__ void __launch_bounds__(kPaintThreads, FAST ? 8 : 1) k_paint_tiles(
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
     const uint32_t* __restrict__ bstart, float* __restrict__ mesh, MassTable mt, int species,
@@ -255,11 +282,27 @@ __global__ void __launch_bounds__(kPaintThreads, FAST ? 8 : 1) k_paint_tiles(
     float mmax, uint32_t* __restrict__ redo) {
   __shared__ __align__(16) unsigned int accw[FAST ? kFastWords : 2 * kAccWords];
   __shared__ uint32_t run_lo[14], run_pre[15];
-  paint_tile<FAST>(blockIdx.x, accw, run_lo, run_pre, us, ids, n, bstart, mesh, mt, species, nm, shift, ntl,
-                   row_pitch, err, wts, mmax, redo);
+  paint_tile<FAST, NW, kPaintThreads>(blockIdx.x, accw, run_lo, run_pre, us, ids, n, bstart, mesh, mt, species, nm,
+                                      shift, ntl, row_pitch, err, wts, mmax, redo);
 }
 
-// The redo pass: the tiles the fast pass listed, painted with the 32-bit carry form
+// Three signed weights a particle onto three meshes in one pass over the particles: positions,
+// corners and weights of the corners once instead of three times.  The 109 KB of sums leave two
+// CTAs an SM, of 512 threads so that 32 warps hide the atomics' latency.
+constexpr int kPaint3Threads = 512;
+constexpr size_t kPaint3Smem = sizeof(unsigned int) * 3 * 2 * kAccWords;
+__global__ void __launch_bounds__(kPaint3Threads, 2) k_paint_weights3(
+    const uint32_t* __restrict__ us, int64_t n, const uint32_t* __restrict__ bstart, float* __restrict__ m0,
+    float* __restrict__ m1, float* __restrict__ m2, int nm, int shift, int ntl, int row_pitch, int* __restrict__ err,
+    const float* __restrict__ wts) {
+  extern __shared__ __align__(16) unsigned int accw3[];
+  __shared__ uint32_t run_lo[14], run_pre[15];
+  const MassTable none{};
+  paint_tile<false, 3, kPaint3Threads>(blockIdx.x, accw3, run_lo, run_pre, us, nullptr, n, bstart, m0, none, 0, nm,
+                                       shift, ntl, row_pitch, err, wts, 0.0f, nullptr, m1, m2);
+}
+
+// The redo pass: the tiles the fast pass listed, painted in the two-word form
 // (persistent CTAs walk the list; an empty list, the normal case, costs one launch).
 __global__ void __launch_bounds__(kPaintThreads) k_paint_redo(
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
@@ -270,8 +313,8 @@ __global__ void __launch_bounds__(kPaintThreads) k_paint_redo(
   __shared__ uint32_t run_lo[14], run_pre[15];
   const uint32_t count = redo[0];
   for (uint32_t q = blockIdx.x; q < count; q += gridDim.x) {
-    paint_tile<false>(redo[1 + q], accw, run_lo, run_pre, us, ids, n, bstart, mesh, mt, species, nm, shift, ntl,
-                      row_pitch, err, nullptr, mmax, nullptr);
+    paint_tile<false, 0, kPaintThreads>(redo[1 + q], accw, run_lo, run_pre, us, ids, n, bstart, mesh, mt, species, nm,
+                                        shift, ntl, row_pitch, err, nullptr, mmax, nullptr);
     __syncthreads();  // the shared accumulators are reused by the next tile
   }
 }
@@ -675,9 +718,9 @@ void paint_tiles(pm_ctx* c, const uint32_t* us, const uint32_t* ids, int64_t n, 
     cudaMemsetAsync(c->paint_redo, 0, sizeof(uint32_t), s);
     {
       LaunchScope L(c, s, K_PAINT);
-      k_paint_tiles<true><<<grid, kPaintThreads, 0, s>>>(us, ids, n, c->bstart, mesh, c->mt, species, c->g.n,
-                                                         32 - c->g.logn, c->ntl, row_pitch, c->err_dev, nullptr,
-                                                         mmax, c->paint_redo);
+      k_paint_tiles<true, 0><<<grid, kPaintThreads, 0, s>>>(us, ids, n, c->bstart, mesh, c->mt, species, c->g.n,
+                                                            32 - c->g.logn, c->ntl, row_pitch, c->err_dev, nullptr,
+                                                            mmax, c->paint_redo);
     }
     // persistent CTAs, as many as fit: the list is short, or empty, in most steps
     static int per_sm = 0, sms = 0;
@@ -693,9 +736,21 @@ void paint_tiles(pm_ctx* c, const uint32_t* us, const uint32_t* ids, int64_t n, 
     return;
   }
   LaunchScope L(c, s, K_PAINT);
-  k_paint_tiles<false><<<grid, kPaintThreads, 0, s>>>(us, ids, n, c->bstart, mesh, c->mt, species, c->g.n,
-                                                      32 - c->g.logn, c->ntl, row_pitch, c->err_dev, weights, mmax,
-                                                      nullptr);
+  auto kern = weights ? k_paint_tiles<false, 1> : k_paint_tiles<false, 0>;
+  kern<<<grid, kPaintThreads, 0, s>>>(us, ids, n, c->bstart, mesh, c->mt, species, c->g.n, 32 - c->g.logn, c->ntl,
+                                      row_pitch, c->err_dev, weights, mmax, nullptr);
+}
+
+void paint_weights3(pm_ctx* c, const uint32_t* us, int64_t n, const float* weights, float* m0, float* m1, float* m2,
+                    int row_pitch, cudaStream_t s) {
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_paint_weights3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPaint3Smem);
+    attr = true;
+  }
+  LaunchScope L(c, s, K_PAINT);
+  k_paint_weights3<<<(unsigned)(c->nt * c->nt * c->nt), kPaint3Threads, kPaint3Smem, s>>>(
+      us, n, c->bstart, m0, m1, m2, c->g.n, 32 - c->g.logn, c->ntl, row_pitch, c->err_dev, weights);
 }
 
 void readout_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint32_t* ids, int64_t n,

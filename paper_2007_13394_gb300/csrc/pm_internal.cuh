@@ -227,6 +227,9 @@ void gather_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint32_t*
 // weights (sorted order, signed) replace the species masses when non-null
 void paint_tiles(pm_ctx* c, const uint32_t* us, const uint32_t* ids, int64_t n, int species,
                  float* mesh, int row_pitch, cudaStream_t s, const float* weights = nullptr);
+// three signed weights a particle (w[3n], sorted order), one mesh each
+void paint_weights3(pm_ctx* c, const uint32_t* us, int64_t n, const float* weights, float* m0, float* m1, float* m2,
+                    int row_pitch, cudaStream_t s);
 void fft_forward(pm_ctx* c, const Geom& g, float2* buf, float2* dst, int green, cudaStream_t s);
 void fft_inverse_component(pm_ctx* c, const Geom& g, const float2* phi, float2* buf, int comp,
                            cudaStream_t s);
