@@ -229,8 +229,7 @@ int pm_step(pm_ctx* ctx, pm_state* st, double a0, double ah, double a1, void* st
  * that ends one step also applies the next step's first half kick and drift (FastPM's
  * KDK with the two half kicks of a step boundary in one pass over the particles), so
  * there is no separate kick/drift pass between steps and f is written by the last step
- * only.  On return: as pm_step after the last step.  Stream ordered, with one host
- * synchronisation per step (the sort's choice of method).  On an error status the
+ * only.  On return: as pm_step after the last step.  Stream ordered.  On an error status the
  * state is undefined (steps before the failing one have already applied the next
  * step's kick and drift). */
 int pm_run(pm_ctx* ctx, pm_state* st, const double* schedule, int64_t nsteps, void* stream);
@@ -440,7 +439,8 @@ const char* pm_kernel_name(int32_t kind);
  * used the near-sorted re-sort (the state in the order the context's last step left
  * it: most particles keep their key, only the others are radix-sorted), out[1] steps
  * that sorted from scratch, out[2] the particles the last near-sorted re-sort moved
- * between keys.  Both ways give the same stable permutation of the keys. */
+ * between keys.  Both ways give the same stable permutation of the keys.  The kernels choose
+ * and count, so this waits for the device. */
 int pm_sort_stats(pm_ctx* ctx, int64_t* out);
 
 #ifdef __cplusplus

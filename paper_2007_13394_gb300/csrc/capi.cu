@@ -122,14 +122,10 @@ void free_all(pm_ctx* c) {
   ctx_free(c, c->counts);
   ctx_free(c, c->bstart);
   ctx_free(c, c->bprev);
-  ctx_free(c, c->rs_low);
   ctx_free(c, c->rs_k2);
   ctx_free(c, c->rs_v2);
-  ctx_free(c, c->rs_dev);
-  if (c->rs_host) cudaFreeHost(c->rs_host);
+  ctx_free(c, c->rs_stats);
   ctx_free(c, c->hist);
-  ctx_free(c, c->hist_scan);
-  ctx_free(c, c->scan_tmp);
   ctx_free(c, c->pk_partial);
   ctx_free(c, c->pk_final);
   ctx_free(c, c->pk_w);
@@ -213,21 +209,13 @@ int check_state(pm_ctx* c, const pm_state* st) {
 }
 
 // Sort of the drifted state (keys and counts from kick_drift_keys or a drifting
-// readout) into the scratch copies: the near-sorted re-sort when the state is in the
-// order of the last sort, else from scratch.
+// readout) into the scratch copies: the near-sorted re-sort when the state may be in the
+// order of the last sort (the device checks), else from scratch.
 int sort_drifted(pm_ctx* c, pm_state* st, cudaStream_t s) {
   const int64_t n = st->n;
-  int done = 0;
-  if (n > 0 && c->rs_n == n) {
-    done = resort_near_sorted(c, st->u, st->p, st->id, n, s);
-    if (done < 0) return done;
-  }
-  if (done) {
-    ++c->rs_fast;
-    return PM_OK;
-  }
+  if (n > 0 && c->rs_n == n) return resort_near_sorted(c, st->u, st->p, st->id, n, s);
   ++c->rs_full;
-  const int rc = radix_and_buckets(c, n, s);
+  const int rc = n > 0 ? sort_by_keys(c, n, s) : sort_particles(c, nullptr, 0, s);
   if (rc != PM_OK) return rc;
   gather_sorted(c, st->u, st->p, st->id, n, c->vals[0], s);
   return PM_OK;
@@ -312,22 +300,20 @@ int run_impl(pm_ctx* c, pm_state* st, const double* sched, int64_t nsteps, cudaS
     if (rc != PM_OK) return rc;
   }
   kick_drift_keys(c, st->u, st->p, st->f, n, (float)k[0], dscale(0), s, c->rs_n == n);
-  const long long nb1 = c->nbuckets + 1;
   for (int64_t i = 0; i < nsteps; ++i) {
     rc = sort_drifted(c, st, s);
     if (rc != PM_OK) return rc;
     const float K2 = (float)k[3 * i + 2];
     if (i + 1 < nsteps) {
       // counts of the keys the drifting readout writes (the sort above has used its own)
-      PM_CUDA_TRY(cudaMemsetAsync(c->counts, 0, sizeof(uint32_t) * 3 * nb1, s));
-      PM_CUDA_TRY(cudaMemsetAsync(c->rs_low, 0, sizeof(uint32_t) * nb1, s));
-      PM_CUDA_TRY(cudaMemsetAsync(c->rs_dev, 0, sizeof(uint32_t), s));
+      rc = clear_resort(c, s);
+      if (rc != PM_OK) return rc;
       DriftNext dn;
       dn.K1 = (float)k[3 * (i + 1)];
       dn.dscale = dscale(i + 1);
       dn.keys = c->keys[0];
       dn.cnt3 = c->counts;
-      dn.nb1 = nb1;
+      dn.nb1 = c->nbuckets + 1;
       dn.low = c->rs_low;
       ForceOut o{c->ps, K2, st->p, nullptr, st->u, st->id, nullptr};
       o.drift = &dn;
@@ -431,9 +417,10 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
   c->nbuckets = (long long)c->nt * c->nt * c->nt * 8;
   int bits = 0;
   while ((1LL << bits) < c->nbuckets) ++bits;
-  // 18-bit keys or fewer: two 9-bit passes; else 8-bit passes
-  c->radix_bits = bits <= 18 ? 9 : 8;
-  c->radix_passes = std::max(1, (bits + c->radix_bits - 1) / c->radix_bits);
+  // as few passes as 9-bit digits allow, then the narrowest digits (7 to 9 bits) that take
+  // no more passes: fewer counters a tile
+  c->radix_passes = std::max(1, (bits + 8) / 9);
+  c->radix_bits = std::max(7, (bits + c->radix_passes - 1) / c->radix_passes);
   c->n_max = cfg->n_max;
   if (c->n_max >= (int64_t)0xffffffffLL) {
     delete c;
@@ -471,13 +458,10 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
   const size_t me = c->g.elems();
   const int64_t nm = std::max<int64_t>(c->n_max, 1);
   const long long hb = (nm + 4095) / 4096;
-  c->hist_blocks_max = hb;
-  const long long scan_n = std::max<long long>(512 * hb, 3 * (c->nbuckets + 1));
-  {  // every level of the recursive scan keeps 2 * blocks words
-    size_t need = 64;
-    for (long long m = scan_n; m > 1; m = (m + 4095) / 4096) need += 2 * (size_t)((m + 4095) / 4096);
-    c->scan_tmp_elems = need;
-  }
+  // zeroed words: counts, rs_low, rs_dev, the scan's tile counter, its status (8-byte aligned)
+  const size_t flag_at = 4 * (size_t)(c->nbuckets + 1), scan_at = (flag_at + 3) / 2 * 2;
+  const size_t clear_words = scan_at + 2 * ((3 * (size_t)(c->nbuckets + 1) + kScanTile - 1) / kScanTile);
+  const size_t hist_words = ((size_t)std::min<long long>(hb, kMaxChunks) + 1) << c->radix_bits;
   // flag bit 0, or a 2048^3 mesh: per-component force path with two meshes (at 2048^3 it is
   // also the faster one: reading three 34 GB meshes at once starves the readout)
   const bool two_mesh = (cfg->flags & PM_FLAG_TWO_MESH) != 0 || N >= 2048;
@@ -486,24 +470,29 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
       dalloc(c, &c->winv, N) || dalloc(c, &c->wforce, N) || dalloc(c, &c->kvec0, N) || dalloc(c, &c->keys[0], nm) ||
       dalloc(c, &c->keys[1], nm) || dalloc(c, &c->vals[0], nm) || dalloc(c, &c->vals[1], nm) ||
       dalloc(c, &c->us, 3 * nm) || dalloc(c, &c->ps, 3 * nm) || dalloc(c, &c->ids, nm) ||
-      dalloc(c, &c->counts, 3 * (c->nbuckets + 1)) || dalloc(c, &c->bstart, 3 * (c->nbuckets + 1)) ||
-      dalloc(c, &c->bprev, 3 * (c->nbuckets + 1)) || dalloc(c, &c->rs_low, c->nbuckets + 1) ||
-      dalloc(c, &c->rs_k2, nm) || dalloc(c, &c->rs_v2, nm) || dalloc(c, &c->rs_dev, 1) ||
-      dalloc(c, &c->hist, 512 * hb) || dalloc(c, &c->hist_scan, 512 * hb) ||
-      dalloc(c, &c->scan_tmp, c->scan_tmp_elems) || dalloc(c, &c->pk_partial, (size_t)N * 3 * 2048) ||
+      dalloc(c, &c->counts, clear_words) || dalloc(c, &c->bstart, 3 * (c->nbuckets + 1)) ||
+      dalloc(c, &c->bprev, 3 * (c->nbuckets + 1)) || dalloc(c, &c->rs_k2, nm) || dalloc(c, &c->rs_v2, nm) ||
+      dalloc(c, &c->rs_stats, 3) || dalloc(c, &c->hist, hist_words) ||
+      dalloc(c, &c->pk_partial, (size_t)N * 2 * 2048) ||
       dalloc(c, &c->pk_final, 3 * 2048) || dalloc(c, &c->err_dev, 1) ||
       dalloc(c, &c->paint_redo, (size_t)c->nt * c->nt * c->nt + 1)) {
     free_all(c);
     delete c;
     return PM_ENOMEM;
   }
-  if (cudaMallocHost(&c->err_host, sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&c->rs_host, 3 * sizeof(uint32_t)) != cudaSuccess) {
+  if (cudaMallocHost(&c->err_host, sizeof(int)) != cudaSuccess) {
     free_all(c);
     delete c;
     return PM_ENOMEM;
   }
   cudaMemset(c->err_dev, 0, sizeof(int));
+  c->rs_low = c->counts + 3 * (c->nbuckets + 1);
+  c->rs_dev = c->counts + flag_at;
+  c->scan_tile = c->rs_dev + 1;
+  c->scan_status = reinterpret_cast<unsigned long long*>(c->counts + scan_at);
+  c->clear_words = clear_words;
+  c->digit_totals = c->hist + (hist_words - ((size_t)1 << c->radix_bits));
+  cudaMemset(c->rs_stats, 0, 3 * sizeof(long long));
   // k tables of the force mesh (FP64 on the host, stored as float).  Force kernel:
   // phi_k = -1.5 Omega_m0 delta_k / N^3 / k^2 and the 4-point finite-difference gradient
   // D(k) = (8 sin kH - sin 2kH) / (6H); flags bit 1 selects the deconvolved spectral form
@@ -961,9 +950,12 @@ int pm_profile_read(pm_ctx* c, int32_t kind, double* ms, int64_t* launches, int3
 int pm_sort_stats(pm_ctx* c, int64_t* out) {
   if (!valid(c)) return PM_ENOTINIT;
   if (!out) return PM_EINVAL;
-  out[0] = c->rs_fast;
-  out[1] = c->rs_full;
-  out[2] = c->rs_last_movers;
+  long long d[3];
+  PM_CUDA_TRY(cudaDeviceSynchronize());  // the device counts the re-sorts
+  PM_CUDA_TRY(cudaMemcpy(d, c->rs_stats, sizeof(d), cudaMemcpyDeviceToHost));
+  out[0] = d[0];
+  out[1] = c->rs_full + d[1];
+  out[2] = d[2];
   return PM_OK;
 }
 

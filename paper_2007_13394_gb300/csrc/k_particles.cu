@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(kFd4Threads) k_readout_fd4_kick(
 // arrays of nbuckets + 1): cnt3[0][kn] all particles of new key kn, cnt3[1][kn]
 // stayers, cnt3[2][ko] movers out of old key ko; low[kn] movers from a lower old key.
 // Flag bit 1: a particle outside its old key's range [bprev[ko], bprev[ko + 1]) (the
-// state is not in bprev's order: the caller sorts from scratch).
+// state is not in bprev's order: every particle is then sorted as a mover).
 template <bool RESORT>
 __global__ void k_kick_drift_keys(uint32_t* __restrict__ u, float* __restrict__ p,
                                   const float* __restrict__ f, int64_t n, float K1, float dscale,
@@ -662,14 +662,13 @@ __global__ void k_kick_drift_keys(uint32_t* __restrict__ u, float* __restrict__ 
       }
     }
   }
-  unsigned act = __ballot_sync(0xffffffffu, ok);
-  if (ok) {
-    unsigned peers = __match_any_sync(act, key);
-    int leader = __ffs(peers) - 1;
-    if ((int)(threadIdx.x & 31) == leader) atomicAdd(cnt3 + key, (uint32_t)__popc(peers));
-  }
   if constexpr (RESORT) {
     const int lane = threadIdx.x & 31;
+    const unsigned act = __ballot_sync(0xffffffffu, ok);
+    if (ok) {
+      const unsigned peers = __match_any_sync(act, key);
+      if (lane == __ffs(peers) - 1) atomicAdd(cnt3 + key, (uint32_t)__popc(peers));
+    }
     const unsigned has = __ballot_sync(0xffffffffu, cat != 0xffffffffu);
     if (cat != 0xffffffffu) {
       const unsigned peers = __match_any_sync(has, cat);
@@ -797,11 +796,7 @@ void readout_fd4_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint
 void kick_drift_keys(pm_ctx* c, uint32_t* u, float* p, const float* f, int64_t n, float K1,
                      float dscale, cudaStream_t s, bool resort) {
   const long long nb1 = c->nbuckets + 1;
-  cudaMemsetAsync(c->counts, 0, sizeof(uint32_t) * (resort ? 3 * nb1 : nb1), s);
-  if (resort) {
-    cudaMemsetAsync(c->rs_low, 0, sizeof(uint32_t) * nb1, s);
-    cudaMemsetAsync(c->rs_dev, 0, sizeof(uint32_t), s);
-  }
+  if (resort) clear_resort(c, s);
   if (n == 0) return;
   LaunchScope L(c, s, K_KICK_DRIFT_KEYS);
   const unsigned grid = (unsigned)((n + 255) / 256);

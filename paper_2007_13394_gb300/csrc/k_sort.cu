@@ -1,15 +1,20 @@
 // Stable counting sort of particles into 16^3-cell tiles of the mesh.
 //
-// key = tile * 8 + face class (see pm.h, pm_sort).  The per-key counts (an
-// integer histogram, order independent) give every bucket's start by an
-// exclusive scan; the particle order inside the key space comes from a stable
-// least-significant-digit radix sort of (key, incoming index) with 8- or 9-bit
-// digits (two 9-bit passes cover the 18-bit keys of meshes up to 512^3):
-// per pass, an upsweep histogram per 4096-key block, a scan of the
-// digit-major histogram, and a downsweep that ranks each key stably inside
-// its block (warp match inside a round, warp-private digit counters across the
-// warp's contiguous 512 keys, one block scan over (digit, warp)) and writes it
-// through shared memory so that global writes stay coalesced.
+// key = tile * 8 + face class (see pm.h, pm_sort).  The order is a stable
+// least-significant-digit radix sort of (key, incoming index) with 7- to 9-bit digits (two
+// 9-bit passes cover the 18-bit keys of a 512^3 mesh).  Each CTA owns one contiguous chunk of
+// whole 4096-key tiles, at most three CTAs an SM, so a pass is: digit counts per chunk (made by
+// the key kernel for the first pass), a scan of them over the chunks, and a scatter in which the
+// CTA walks its tiles with its own running digit positions -- nothing waits for another CTA.
+// In a tile, warp w ranks 512 contiguous keys in 16 rounds of 32 (ballots for the rank inside
+// a round, warp-private digit counters across rounds), one block scan over (digit, warp) gives
+// staging offsets, and the keys go out through shared memory in coalesced runs.  A bucket's
+// start is a binary search in the sorted keys, done by the gather.
+//
+// Bound by latency inside a tile, then by DRAM (20 bytes a particle and pass).  us a pass (counts,
+// scan and scatter), 19 M particles, 9 bits: 28 + 3 + 137 (with a
+// warp match per round, 4096-key blocks and a three-launch scan: 42 + 15 + 215); the key kernel,
+// which no longer counts buckets with global atomics, 103 -> 56.
 //
 // Near-sorted re-sort (pm_step): the state is in the order of the last step's sort,
 // bucket starts bprev, and most particles keep their key.  A stayer (same key, inside
@@ -18,9 +23,13 @@
 // key B those with index below bprev[B] are exactly the movers from lower keys, those
 // inside B's old range are B's stayers, the rest came from higher keys: bucket B is
 // [lower movers | stayers | higher movers], which is the stable order.  The result is
-// the same permutation as the radix sort from scratch; a particle outside its old
-// key's range (a state not in bprev's order) sends the caller to that sort.
+// the same permutation as the radix sort from scratch.  A particle outside its old key's
+// range (a state not in bprev's order) makes every particle a mover, in index order: then it
+// is the radix sort from scratch.  That choice and the number of movers stay on the device:
+// the kernels take their ranges from there, and the host never waits.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "pm_internal.cuh"
 
@@ -28,32 +37,32 @@ namespace pmnu {
 
 namespace {
 
-constexpr int kScanThreads = 1024;
-constexpr int kScanItems = 4;
-constexpr int kScanTile = kScanThreads * kScanItems;  // 4096
-
 constexpr int kRadixThreads = 256;
 constexpr int kRadixRounds = 16;
-constexpr int kRadixTile = kRadixThreads * kRadixRounds;  // 4096 keys per block
+constexpr int kRadixTile = kRadixThreads * kRadixRounds;  // 4096 keys per tile
 constexpr int kRadixWarps = kRadixThreads / 32;
+constexpr int kCountThreads = 512;
+constexpr int kCountUnroll = 4;
+constexpr int kSpinLimit = 1 << 22;  // look-back polls of the scan before a CTA gives up (PM_ETIMEOUT)
 
-// ------------------------------------------------------------------ keys
-__global__ void k_keys(const uint32_t* __restrict__ u, int64_t n, int shift, int ntl,
-                       uint32_t* __restrict__ keys, uint32_t* __restrict__ counts) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool ok = i < n;
-  uint32_t key = 0xffffffffu;
-  if (ok) {
-    key = tile_key(u[i], u[n + i], u[2 * n + i], shift, ntl);
-    keys[i] = key;
-  }
-  // warp-aggregated histogram increment
-  unsigned act = __ballot_sync(0xffffffffu, ok);
-  if (ok) {
-    unsigned peers = __match_any_sync(act, key);
-    int leader = __ffs(peers) - 1;
-    if ((int)(threadIdx.x & 31) == leader) atomicAdd(counts + key, (uint32_t)__popc(peers));
-  }
+// look-back status word of the scan: state (1 the tile's own sum, 2 the sum up to it) above a
+// 32-bit value; one 64-bit access carries both, so no fence is needed
+__device__ __forceinline__ unsigned long long ld_status(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_status(unsigned long long* p, uint32_t flag, uint32_t value) {
+  const unsigned long long v = ((unsigned long long)flag << 32) | value;
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// Number of movers of a near-sorted re-sort (every particle when the state was not in
+// bprev's order), from the device: flags of k_kick_drift_keys<true>, scans in bstart3.
+__device__ __forceinline__ int64_t movers_of(const uint32_t* flags, const uint32_t* bstart3, long long nb1, int64_t n) {
+  if (*flags & 1u) return n;
+  const int64_t m = (int64_t)bstart3[3 * nb1 - 1] - (int64_t)bstart3[2 * nb1];
+  return m < 0 ? 0 : (m > n ? n : m);
 }
 
 // ------------------------------------------------------------------ scan
@@ -84,173 +93,334 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
   return before;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const uint32_t* __restrict__ in,
-                                                            long long n,
-                                                            uint32_t* __restrict__ sums) {
-  __shared__ uint32_t ws[32];
-  long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
-  uint32_t s = 0;
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k)
-    if (base + k < n) s += in[base + k];
-  uint32_t tot;
-  block_exclusive_scan(s, ws, &tot);
-  if (threadIdx.x == 0) sums[blockIdx.x] = tot;
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const uint32_t* __restrict__ in,
-                                                             long long n,
-                                                             const uint32_t* __restrict__ offs,
-                                                             uint32_t* __restrict__ out) {
-  __shared__ uint32_t ws[32];
-  long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
+// Exclusive scan in one launch: tiles of kScanTile words handed out in order, each adds up its
+// predecessors' sums by look-back (a warp reads 32 of them at a time).  status and the tile
+// counter start at 0.
+constexpr int kScanThreads = 512;
+constexpr int kScanItems = 8;
+__global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* __restrict__ in, long long n,
+                                                       uint32_t* __restrict__ out,
+                                                       unsigned long long* __restrict__ status,
+                                                       uint32_t* __restrict__ counter, int* __restrict__ err) {
+  __shared__ uint32_t ws[32], s_tile, s_before;
+  const int t = threadIdx.x;
+  if (t == 0) s_tile = atomicAdd(counter, 1u);
+  __syncthreads();
+  const uint32_t tile = s_tile;
+  const long long base = (long long)tile * kScanTile + (long long)t * kScanItems;
   uint32_t v[kScanItems], s = 0;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
     v[k] = (base + k < n) ? in[base + k] : 0u;
     s += v[k];
   }
-  uint32_t run = block_exclusive_scan(s, ws, nullptr) + (offs ? offs[blockIdx.x] : 0u);
+  uint32_t total;
+  uint32_t run = block_exclusive_scan(s, ws, &total);
+  if (t == 0) st_status(status + tile, tile == 0 ? 2u : 1u, total);
+  if (t < 32) {  // look-back
+    uint32_t before = 0;
+    int p = (int)tile - 1, spins = 0;
+    while (p >= 0) {
+      const unsigned long long w = p - t >= 0 ? ld_status(status + p - t) : (2ull << 32);
+      const uint32_t st = (uint32_t)(w >> 32);
+      const unsigned incl = __ballot_sync(0xffffffffu, st == 2u), ready = __ballot_sync(0xffffffffu, st != 0u);
+      const int first = incl ? __ffs(incl) - 1 : 31;
+      const unsigned need = first == 31 ? 0xffffffffu : (2u << first) - 1u;
+      if ((ready & need) != need) {
+        if (++spins > kSpinLimit) {
+          if (t == 0) atomicOr(err, 2);
+          break;
+        }
+        continue;
+      }
+      before += __reduce_add_sync(0xffffffffu, t <= first ? (uint32_t)w : 0u);
+      if (incl) break;
+      p -= 32;
+    }
+    if (t == 0) {
+      if (tile != 0) st_status(status + tile, 2u, before + total);
+      s_before = before;
+    }
+  }
+  __syncthreads();
+  run += s_before;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
     if (base + k < n) out[base + k] = run;
     run += v[k];
   }
 }
+static_assert(kScanThreads * kScanItems == kScanTile, "scan tile");
 
-// ------------------------------------------------------------------ radix
-// Digit width BITS (8 or 9): DIG digits, each of the 256 threads owns DIG / 256 of them.
-template <int BITS>
-__global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint32_t* __restrict__ keys,
-                                                              int64_t n, int shift,
-                                                              long long nblk,
-                                                              uint32_t* __restrict__ hist) {
-  constexpr int DIG = 1 << BITS, PER = DIG / kRadixThreads;
-  constexpr uint32_t MASK = DIG - 1;
-  __shared__ uint32_t cnt[DIG];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) cnt[threadIdx.x + q * kRadixThreads] = 0;
-  __syncthreads();
-  int64_t base = (int64_t)blockIdx.x * kRadixTile;
-#pragma unroll 4
-  for (int r = 0; r < kRadixRounds; ++r) {
-    int64_t i = base + r * kRadixThreads + threadIdx.x;
-    if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & MASK], 1u);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int d = threadIdx.x + q * kRadixThreads;
-    hist[(long long)d * nblk + blockIdx.x] = cnt[d];
+// ------------------------------------------------------------------ keys and digit counts
+// CTA c of C owns the particles [chunk_lo, chunk_hi): whole tiles, the same in every kernel of a pass.
+__device__ __forceinline__ void chunk_of(int64_t n, int64_t& lo, int64_t& hi) {
+  const int64_t tiles = (n + kRadixTile - 1) / kRadixTile, per = (tiles + gridDim.x - 1) / gridDim.x * kRadixTile;
+  lo = (int64_t)blockIdx.x * per;
+  if (lo > n) lo = n;
+  hi = lo + per < n ? lo + per : n;
+}
+
+// h[digit] += 1: neighbouring lanes often hold the same digit (nearly sorted particles), so
+// the first lane of a run adds its length.  Lanes without a particle pass 0xffffffff.
+__device__ __forceinline__ void count_digit(uint32_t d, uint32_t* h) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t prev = __shfl_up_sync(0xffffffffu, d, 1);
+  const bool head = lane == 0 || prev != d;
+  const unsigned heads = __ballot_sync(0xffffffffu, head);
+  if (head && d != 0xffffffffu) {
+    const unsigned next = heads & ~((2u << lane) - 1u);  // heads above this lane (lane 31: none)
+    atomicAdd(h + d, (uint32_t)((next ? __ffs(next) - 1 : 32) - lane));
   }
 }
 
-// Stable scatter of one 4096-key block: warp w ranks the contiguous keys [512 w, 512 w + 512)
-// of the block in 16 rounds of 32 (warp match for the rank inside a round, a warp-private
-// per-digit counter across rounds), so the order inside each digit is the index order;
-// one block-wide scan over (digit, warp) turns the counters into staging offsets; the
-// keys are staged in digit order in shared memory and written out in coalesced runs.
+// Keys of the particles and the chunk's counts of the first digit, hist[d C + c].
 template <int BITS>
-__global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
+__global__ void __launch_bounds__(kCountThreads) k_keys(const uint32_t* __restrict__ u, int64_t n, int shift, int ntl,
+                                                        uint32_t* __restrict__ keys, uint32_t* __restrict__ hist) {
+  constexpr int DIG = 1 << BITS;
+  __shared__ uint32_t h[DIG];
+  for (int i = threadIdx.x; i < DIG; i += kCountThreads) h[i] = 0;
+  __syncthreads();
+  int64_t lo, hi;
+  chunk_of(n, lo, hi);
+  for (int64_t base = lo; base < hi; base += kCountThreads * kCountUnroll) {
+    uint32_t ux[kCountUnroll], uy[kCountUnroll], uz[kCountUnroll];
+#pragma unroll
+    for (int k = 0; k < kCountUnroll; ++k) {
+      const int64_t i = base + k * kCountThreads + threadIdx.x;
+      if (i < hi) {
+        ux[k] = u[i];
+        uy[k] = u[n + i];
+        uz[k] = u[2 * n + i];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kCountUnroll; ++k) {
+      const int64_t i = base + k * kCountThreads + threadIdx.x;
+      uint32_t d = 0xffffffffu;
+      if (i < hi) {
+        const uint32_t key = tile_key(ux[k], uy[k], uz[k], shift, ntl);
+        keys[i] = key;
+        d = key & (DIG - 1);
+      }
+      count_digit(d, h);
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < DIG; i += kCountThreads) hist[(size_t)i * gridDim.x + blockIdx.x] = h[i];
+}
+
+// A digit's counts of existing keys: n of them, or (flags set) the movers of a re-sort.
+template <int BITS>
+__global__ void __launch_bounds__(kCountThreads) k_digits(const uint32_t* __restrict__ keys, int64_t n, int shift,
+                                                          uint32_t* __restrict__ hist,
+                                                          const uint32_t* __restrict__ flags,
+                                                          const uint32_t* __restrict__ bstart3, long long nb1) {
+  constexpr int DIG = 1 << BITS;
+  __shared__ uint32_t h[DIG];
+  for (int i = threadIdx.x; i < DIG; i += kCountThreads) h[i] = 0;
+  if (flags) n = movers_of(flags, bstart3, nb1, n);
+  __syncthreads();
+  int64_t lo, hi;
+  chunk_of(n, lo, hi);
+  for (int64_t base = lo; base < hi; base += kCountThreads * kCountUnroll) {
+    uint32_t key[kCountUnroll];
+#pragma unroll
+    for (int k = 0; k < kCountUnroll; ++k) {
+      const int64_t i = base + k * kCountThreads + threadIdx.x;
+      key[k] = i < hi ? keys[i] : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < kCountUnroll; ++k)
+      count_digit(base + k * kCountThreads + threadIdx.x < hi ? (key[k] >> shift) & (DIG - 1) : 0xffffffffu, h);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < DIG; i += kCountThreads) hist[(size_t)i * gridDim.x + blockIdx.x] = h[i];
+}
+
+// Exclusive scan of each digit's counts over the C chunks, in place; totals[d].  A warp a digit.
+__global__ void __launch_bounds__(256) k_chunk_scan(uint32_t* __restrict__ hist, int C, int digits,
+                                                    uint32_t* __restrict__ totals) {
+  const int d = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (d >= digits) return;
+  uint32_t* const h = hist + (size_t)d * C;
+  uint32_t run = 0;
+  for (int c0 = 0; c0 < C; c0 += 128) {  // four words a lane
+    uint32_t v[4], s = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = c0 + lane * 4 + k;
+      v[k] = c < C ? h[c] : 0u;
+      s += v[k];
+    }
+    uint32_t x = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    uint32_t at = run + x - s;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = c0 + lane * 4 + k;
+      if (c < C) h[c] = at;
+      at += v[k];
+    }
+    run += __shfl_sync(0xffffffffu, x, 31);
+  }
+  if (lane == 0) totals[d] = run;
+}
+
+// ------------------------------------------------------------------ radix scatter
+// One stable pass over (key, value) pairs (vin null: the value is the index), see the top of
+// the file: hist holds the chunk's exclusive counts per digit, totals every digit's count.
+template <int BITS>
+__global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift,
-    long long nblk, const uint32_t* __restrict__ hist, const uint32_t* __restrict__ hist_scan,
-    uint32_t* __restrict__ kout, uint32_t* __restrict__ vout) {
-  constexpr int DIG = 1 << BITS, PER = DIG / kRadixThreads;
+    const uint32_t* __restrict__ hist, const uint32_t* __restrict__ totals, uint32_t* __restrict__ kout,
+    uint32_t* __restrict__ vout, const uint32_t* __restrict__ flags, const uint32_t* __restrict__ bstart3,
+    long long nb1) {
+  constexpr int DIG = 1 << BITS, PER = DIG > kRadixThreads ? DIG / kRadixThreads : 1;
   constexpr uint32_t MASK = DIG - 1;
   constexpr int KPW = kRadixTile / kRadixWarps;  // keys per warp
   constexpr int RPW = KPW / 32;                  // rounds per warp
-  extern __shared__ uint32_t stage_kv[];  // keys then values of the block, in digit order
-  uint32_t* sk = stage_kv;
-  uint32_t* sv = stage_kv + kRadixTile;
+  extern __shared__ uint32_t stage_kv[];  // keys then values of the tile, in digit order
+  uint32_t* const sk = stage_kv;
+  uint32_t* const sv = stage_kv + kRadixTile;
   __shared__ uint32_t wcnt[kRadixWarps][DIG];  // per-warp digit counts, then staging offsets
-  __shared__ uint32_t dstart[DIG];             // block-local start of each digit
-  __shared__ uint32_t gbase[DIG];              // global start of this block's run of each digit
+  __shared__ uint32_t delta[DIG];              // global minus staging position of the tile's run of a digit
   __shared__ uint32_t ws[32];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-  for (int i = t; i < kRadixWarps * DIG; i += kRadixThreads) (&wcnt[0][0])[i] = 0;
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int d = t + q * kRadixThreads;
-    gbase[d] = hist_scan[(long long)d * nblk + blockIdx.x];
-  }
-  __syncthreads();
-  // 1. ranks inside the warp's digit runs
-  const unsigned lt = (1u << lane) - 1u;
-  uint32_t key[RPW], val[RPW], rk[RPW];
-#pragma unroll
-  for (int r = 0; r < RPW; ++r) {
-    const int64_t i = base + w * KPW + r * 32 + lane;
-    const bool ok = i < n;
-    key[r] = ok ? kin[i] : 0u;
-    val[r] = ok ? (vin ? vin[i] : (uint32_t)i) : 0u;
-    const uint32_t d = ok ? ((key[r] >> shift) & MASK) : (uint32_t)(DIG + lane);
-    const unsigned peers = __match_any_sync(0xffffffffu, d);
-    const uint32_t below = (uint32_t)__popc(peers & lt);
-    const uint32_t c0 = ok ? wcnt[w][d] : 0u;  // every peer reads the count before this round
-    rk[r] = c0 + below;
-    __syncwarp();
-    if (ok && below == 0) wcnt[w][d] = c0 + (uint32_t)__popc(peers);
-    __syncwarp();
-  }
-  __syncthreads();
-  // 2. digit totals -> block-exclusive digit starts -> per-warp staging offsets
+  if (flags) n = movers_of(flags, bstart3, nb1, n);
+  int64_t lo, hi;
+  chunk_of(n, lo, hi);
+  if (lo >= hi) return;
+  const bool owner = t * PER < DIG;  // this thread's digits: t PER + q
+  uint32_t next[PER];                // where the chunk's next key of a digit goes
   {
     uint32_t c[PER], sum = 0;
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-      const int d = t * PER + q;
-      uint32_t tot = 0;
-#pragma unroll
-      for (int ww = 0; ww < kRadixWarps; ++ww) tot += wcnt[ww][d];
-      c[q] = tot;
-      sum += tot;
+      c[q] = owner ? totals[t * PER + q] : 0u;
+      sum += c[q];
     }
     uint32_t ex = block_exclusive_scan(sum, ws, nullptr);
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-      const int d = t * PER + q;
-      dstart[d] = ex;
-      uint32_t run = ex;
-#pragma unroll
-      for (int ww = 0; ww < kRadixWarps; ++ww) {
-        const uint32_t cw = wcnt[ww][d];
-        wcnt[ww][d] = run;
-        run += cw;
-      }
+      next[q] = owner ? ex + hist[(size_t)(t * PER + q) * gridDim.x + blockIdx.x] : 0u;
       ex += c[q];
     }
   }
-  __syncthreads();
-  // 3. stage in digit order
+  const unsigned lt = (1u << lane) - 1u;
+  for (int64_t base = lo; base < hi; base += kRadixTile) {
+    // 1. ranks inside the warp's digit runs
+    uint32_t key[RPW], val[RPW], rk[RPW / 2];  // ranks are below 512: two to a word
 #pragma unroll
-  for (int r = 0; r < RPW; ++r) {
-    const int64_t i = base + w * KPW + r * 32 + lane;
-    if (i < n) {
-      const uint32_t d = (key[r] >> shift) & MASK;
-      const uint32_t pos = wcnt[w][d] + rk[r];
-      sk[pos] = key[r];
-      sv[pos] = val[r];
+    for (int r = 0; r < RPW; ++r) {
+      const int64_t i = base + w * KPW + r * 32 + lane;
+      key[r] = i < hi ? kin[i] : 0u;
+      val[r] = i < hi ? (vin ? vin[i] : (uint32_t)i) : 0u;
     }
-  }
-  __syncthreads();
-  // 4. coalesced runs to the digit's global position
-  const int64_t cnt = (n - base) < kRadixTile ? (n - base) : kRadixTile;
-  for (int j = t; j < cnt; j += kRadixThreads) {
-    uint32_t k = sk[j];
-    uint32_t d = (k >> shift) & MASK;
-    uint32_t dst = gbase[d] + (j - dstart[d]);
-    kout[dst] = k;
-    vout[dst] = sv[j];
+    __syncthreads();  // the previous tile's shared memory is read
+    for (int i = t; i < kRadixWarps * DIG; i += kRadixThreads) (&wcnt[0][0])[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) {
+      const bool ok = base + w * KPW + r * 32 + lane < hi;
+      const uint32_t d = (key[r] >> shift) & MASK;
+      unsigned peers = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+      for (int b = 0; b < BITS; ++b) {
+        const unsigned m = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+        peers &= ((d >> b) & 1u) ? m : ~m;
+      }
+      const uint32_t below = (uint32_t)__popc(peers & lt);
+      const uint32_t c0 = ok ? wcnt[w][d] : 0u;  // every peer reads the count before this round
+      if (r & 1) rk[r / 2] |= (c0 + below) << 16; else rk[r / 2] = c0 + below;
+      __syncwarp();
+      if (ok && below == 0) wcnt[w][d] = c0 + (uint32_t)__popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    // 2. digit totals -> tile-exclusive digit starts -> per-warp staging offsets
+    {
+      uint32_t c[PER], sum = 0;
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        uint32_t tot = 0;
+        if (owner) {
+#pragma unroll
+          for (int ww = 0; ww < kRadixWarps; ++ww) tot += wcnt[ww][t * PER + q];
+        }
+        c[q] = tot;
+        sum += tot;
+      }
+      uint32_t ex = block_exclusive_scan(sum, ws, nullptr);
+      if (owner) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+          const int d = t * PER + q;
+          uint32_t run = ex;
+#pragma unroll
+          for (int ww = 0; ww < kRadixWarps; ++ww) {
+            const uint32_t cw = wcnt[ww][d];
+            wcnt[ww][d] = run;
+            run += cw;
+          }
+          delta[d] = next[q] - ex;
+          next[q] += c[q];
+          ex += c[q];
+        }
+      }
+    }
+    __syncthreads();
+    // 3. stage in digit order
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) {
+      if (base + w * KPW + r * 32 + lane < hi) {
+        const uint32_t pos = wcnt[w][(key[r] >> shift) & MASK] + ((r & 1) ? rk[r / 2] >> 16 : rk[r / 2] & 0xffffu);
+        sk[pos] = key[r];
+        sv[pos] = val[r];
+      }
+    }
+    __syncthreads();
+    // 4. coalesced runs to the digit's global position
+    const int cnt = (int)((hi - base) < kRadixTile ? (hi - base) : kRadixTile);
+    for (int j = t; j < cnt; j += kRadixThreads) {
+      const uint32_t k = sk[j];
+      const uint32_t dst = delta[(k >> shift) & MASK] + (uint32_t)j;
+      kout[dst] = k;
+      vout[dst] = sv[j];
+    }
   }
 }
 
 // ------------------------------------------------------------------ gather
+// The first nbb CTAs find the bucket starts in the sorted keys (bstart[k] = number of keys
+// below k; nb1 of them), the others gather the particles.
 __global__ void k_gather(const uint32_t* __restrict__ u, const float* __restrict__ p,
                          const uint32_t* __restrict__ id, int64_t n,
                          const uint32_t* __restrict__ perm, uint32_t* __restrict__ us,
-                         float* __restrict__ ps, uint32_t* __restrict__ ids) {
-  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+                         float* __restrict__ ps, uint32_t* __restrict__ ids, const uint32_t* __restrict__ skeys,
+                         long long nb1, unsigned nbb, uint32_t* __restrict__ bstart) {
+  if (blockIdx.x < nbb) {
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= nb1) return;
+    uint32_t lo = 0, len = (uint32_t)n;
+    while (len > 0) {
+      const uint32_t h = len >> 1;
+      if ((long long)skeys[lo + h] < k) {
+        lo += h + 1;
+        len -= h + 1;
+      } else {
+        len = h;
+      }
+    }
+    bstart[k] = lo;
+    return;
+  }
+  int64_t k = (int64_t)(blockIdx.x - nbb) * blockDim.x + threadIdx.x;
   if (k >= n) return;
   uint32_t i = perm[k];
   us[k] = u[i];
@@ -286,21 +456,32 @@ __device__ __forceinline__ void copy_particle(const uint32_t* __restrict__ u, co
 // instead of seven scattered words), and mv holds that position.  A block scan of the mover flags gives every particle the
 // number of movers of its own old key before it (mrank); a stayer goes to
 // bstart[B] + low[B] + (i - bprev[B]) - mrank, a mover's (new key, index) to its old
-// key's slot of the mover list, mstart3[ko] - base3 + mrank (movers in index order).
+// key's slot of the mover list, mstart3[ko] - base3 + mrank (movers in index order).  With
+// flag bit 1 every particle is a mover at its own index.  stage_room: the movers' records
+// that the staging area holds (more movers: none is staged).
 constexpr int kResortThreads = 256;
 
 __global__ void __launch_bounds__(kResortThreads) k_resort_old_tiles(
     const uint32_t* __restrict__ u, const float* __restrict__ p, const uint32_t* __restrict__ id, int64_t n,
     const uint32_t* __restrict__ keys, const uint32_t* __restrict__ bprev, const uint32_t* __restrict__ bstart3,
     long long nb1, const uint32_t* __restrict__ low, uint32_t* __restrict__ us, float* __restrict__ ps,
-    uint32_t* __restrict__ ids, uint32_t* __restrict__ mk, uint32_t* __restrict__ mv, int64_t nm,
-    int* __restrict__ err, uint4* __restrict__ stage) {
+    uint32_t* __restrict__ ids, uint32_t* __restrict__ mk, uint32_t* __restrict__ mv,
+    const uint32_t* __restrict__ flags, int* __restrict__ err, uint4* __restrict__ stage, int64_t stage_room) {
   constexpr int W = kResortThreads / 32;
   __shared__ uint32_t cls_lo[9];   // bprev[8 O + c]
   __shared__ uint32_t cls_m0[8];   // movers of the tile before class c's first particle
   __shared__ uint32_t wsum[W];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const uint32_t O = blockIdx.x;
+  if (*flags & 1u) {
+    for (int64_t i = (int64_t)O * kResortThreads + t; i < n; i += (int64_t)gridDim.x * kResortThreads) {
+      mk[i] = keys[i];
+      mv[i] = (uint32_t)i;
+    }
+    return;
+  }
+  const int64_t nm = movers_of(flags, bstart3, nb1, n);
+  if (nm > stage_room) stage = nullptr;
   if (t < 9) cls_lo[t] = bprev[8 * O + t];
   __syncthreads();
   const uint32_t lo = cls_lo[0], hi = cls_lo[8];
@@ -381,17 +562,21 @@ __global__ void __launch_bounds__(kResortThreads) k_resort_old_tiles(
 // stayers when it came from a higher key (r >= low[B]).  The movers of keys below B
 // number bstart[B] - sstart[B], sstart = the stayers' scan (bstart3's second third
 // minus n).
-__global__ void k_place_movers(const uint32_t* __restrict__ mk, const uint32_t* __restrict__ mv, int64_t nm,
-                               const uint32_t* __restrict__ u, const float* __restrict__ p,
-                               const uint32_t* __restrict__ id, int64_t n, const uint32_t* __restrict__ bstart3,
-                               long long nb1, long long nbuckets, const uint32_t* __restrict__ low,
-                               uint32_t* __restrict__ us, float* __restrict__ ps, uint32_t* __restrict__ ids,
-                               int* __restrict__ err, const uint4* __restrict__ stage) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= nm) return;
+__device__ __forceinline__ void place_mover(int64_t j, bool all, const uint32_t* __restrict__ mk,
+                                            const uint32_t* __restrict__ mv, int64_t nm,
+                                            const uint32_t* __restrict__ u, const float* __restrict__ p,
+                                            const uint32_t* __restrict__ id, int64_t n,
+                                            const uint32_t* __restrict__ bstart3, long long nb1, long long nbuckets,
+                                            const uint32_t* __restrict__ low, uint32_t* __restrict__ us,
+                                            float* __restrict__ ps, uint32_t* __restrict__ ids,
+                                            int* __restrict__ err, const uint4* __restrict__ stage) {
   const uint32_t B = mk[j];
   if (B >= (uint64_t)nbuckets || mv[j] >= (uint64_t)(stage ? nm : n)) {
     atomicOr(err, 1);
+    return;
+  }
+  if (all) {
+    copy_particle(u, p, id, n, mv[j], (uint32_t)j, us, ps, ids);
     return;
   }
   const uint32_t s0 = bstart3[nb1 + B], s1 = bstart3[nb1 + B + 1];
@@ -417,152 +602,155 @@ __global__ void k_place_movers(const uint32_t* __restrict__ mk, const uint32_t* 
   }
 }
 
-}  // namespace
-
-namespace {
-// Reduce-then-scan; level k keeps its block sums and their scanned offsets in tmp,
-// the next level works further along tmp (total < 2.001 * ceil(n / 4096) words).
-void scan_rec(pm_ctx* c, const uint32_t* in, uint32_t* out, long long n, uint32_t* tmp,
-              cudaStream_t s) {
-  long long nb = (n + kScanTile - 1) / kScanTile;
-  if (nb == 1) {
-    LaunchScope L(c, s, K_SCAN);
-    k_scan_apply<<<1, kScanThreads, 0, s>>>(in, n, nullptr, out);
-    return;
+// With flag bit 1 the movers are all particles: mover j goes to slot j.  Counts the re-sort in
+// stats (near-sorted, from scratch, movers of the last near-sorted one).
+__global__ void k_place_movers(const uint32_t* __restrict__ mk, const uint32_t* __restrict__ mv,
+                               const uint32_t* __restrict__ u, const float* __restrict__ p,
+                               const uint32_t* __restrict__ id, int64_t n, const uint32_t* __restrict__ bstart3,
+                               long long nb1, long long nbuckets, const uint32_t* __restrict__ low,
+                               uint32_t* __restrict__ us, float* __restrict__ ps, uint32_t* __restrict__ ids,
+                               const uint32_t* __restrict__ flags, int* __restrict__ err,
+                               const uint4* __restrict__ stage, int64_t stage_room, long long* __restrict__ stats) {
+  const bool all = (*flags & 1u) != 0u;
+  const int64_t nm = movers_of(flags, bstart3, nb1, n);
+  if (all || nm > stage_room) stage = nullptr;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    stats[all ? 1 : 0] += 1;
+    if (!all) stats[2] = nm;
   }
-  uint32_t* sums = tmp;
-  uint32_t* offs = tmp + nb;
-  {
-    LaunchScope L(c, s, K_SCAN);
-    k_scan_sums<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, sums);
-  }
-  scan_rec(c, sums, offs, nb, tmp + 2 * nb, s);
-  {
-    LaunchScope L(c, s, K_SCAN);
-    k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, offs, out);
-  }
-}
-}  // namespace
-
-void scan_exclusive(pm_ctx* c, const uint32_t* in, uint32_t* out, long long n, cudaStream_t s) {
-  if (n <= 0) return;
-  scan_rec(c, in, out, n, c->scan_tmp, s);
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < nm; j += (int64_t)gridDim.x * blockDim.x)
+    place_mover(j, all, mk, mv, nm, u, p, id, n, bstart3, nb1, nbuckets, low, us, ps, ids, err, stage);
 }
 
-int build_keys(pm_ctx* c, const uint32_t* u, int64_t n, cudaStream_t s) {
-  if (cudaMemsetAsync(c->counts, 0, sizeof(uint32_t) * (c->nbuckets + 1), s) != cudaSuccess)
-    return PM_ECUDA;
-  if (n > 0) {
-    LaunchScope L(c, s, K_KEYS);
-    unsigned grid = (unsigned)((n + 255) / 256);
-    k_keys<<<grid, 256, 0, s>>>(u, n, 32 - c->g.logn, c->ntl, c->keys[0], c->counts);
-  }
-  return PM_OK;
+// the chunks of a sort of up to n keys: as many as tiles, at most kMaxChunks
+unsigned chunks_of(int64_t n) {
+  return (unsigned)std::min<int64_t>(kMaxChunks, std::max<int64_t>(1, (n + kRadixTile - 1) / kRadixTile));
 }
 
-namespace {
-// LSD radix passes of the context's digit width over n (key, value) pairs in buffer pair
-// 0 (values absent: the incoming index), pair 1 the other buffers.  Returns which pair
-// holds the result.
-int radix_passes(pm_ctx* c, uint32_t* const kb[2], uint32_t* const vb[2], bool index_vals, int64_t n,
-                 cudaStream_t s) {
-  const long long nblk = (n + kRadixTile - 1) / kRadixTile;
+template <int BITS>
+void launch_scatter(pm_ctx* c, const uint32_t* kin, const uint32_t* vin, int64_t n, int shift, uint32_t* kout,
+                    uint32_t* vout, const uint32_t* flags, cudaStream_t s) {
+  const size_t dyn = 2 * kRadixTile * sizeof(uint32_t);
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_radix_scatter<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    attr = true;
+  }
+  k_radix_scatter<BITS><<<chunks_of(n), kRadixThreads, dyn, s>>>(kin, vin, n, shift, c->hist, c->digit_totals, kout, vout,
+                                                                flags, c->bstart, c->nbuckets + 1);
+}
+
+// LSD radix passes over n (key, value) pairs in buffer pair 0 (values absent: the incoming
+// index), pair 1 the other buffers; flags: only the movers of a re-sort.  counted: hist holds
+// the first digit's chunk counts already.  Returns which pair holds the result.
+template <int BITS>
+int passes_of(pm_ctx* c, uint32_t* const kb[2], uint32_t* const vb[2], bool index_vals, bool counted, int64_t n,
+              const uint32_t* flags, cudaStream_t s) {
+  const unsigned C = chunks_of(n);
   int cur = 0;
-  const int bits = c->radix_bits;
   for (int pass = 0; pass < c->radix_passes; ++pass) {
-    int shift = bits * pass;
-    {
+    const int shift = BITS * pass;
+    if (!counted || pass > 0) {
       LaunchScope L(c, s, K_RADIX_HIST);
-      if (bits == 9)
-        k_radix_hist<9><<<(unsigned)nblk, kRadixThreads, 0, s>>>(kb[cur], n, shift, nblk, c->hist);
-      else
-        k_radix_hist<8><<<(unsigned)nblk, kRadixThreads, 0, s>>>(kb[cur], n, shift, nblk, c->hist);
+      k_digits<BITS><<<C, kCountThreads, 0, s>>>(kb[cur], n, shift, c->hist, flags, c->bstart, c->nbuckets + 1);
     }
-    scan_exclusive(c, c->hist, c->hist_scan, (1LL << bits) * nblk, s);
     {
-      LaunchScope L(c, s, K_RADIX_SCATTER);
-      const uint32_t* vin = (pass == 0 && index_vals) ? nullptr : vb[cur];
-      const int dyn = 2 * kRadixTile * (int)sizeof(uint32_t);
-      static bool attr = false;
-      if (!attr) {
-        cudaFuncSetAttribute(k_radix_scatter<9>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-        cudaFuncSetAttribute(k_radix_scatter<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-        attr = true;
-      }
-      if (bits == 9)
-        k_radix_scatter<9><<<(unsigned)nblk, kRadixThreads, dyn, s>>>(kb[cur], vin, n, shift, nblk, c->hist,
-                                                                      c->hist_scan, kb[cur ^ 1], vb[cur ^ 1]);
-      else
-        k_radix_scatter<8><<<(unsigned)nblk, kRadixThreads, dyn, s>>>(kb[cur], vin, n, shift, nblk, c->hist,
-                                                                      c->hist_scan, kb[cur ^ 1], vb[cur ^ 1]);
+      LaunchScope L(c, s, K_SCAN);
+      k_chunk_scan<<<(1 << BITS) / 8, 256, 0, s>>>(c->hist, (int)C, 1 << BITS, c->digit_totals);
     }
+    LaunchScope L(c, s, K_RADIX_SCATTER);
+    launch_scatter<BITS>(c, kb[cur], (pass == 0 && index_vals) ? nullptr : vb[cur], n, shift, kb[cur ^ 1], vb[cur ^ 1],
+                         flags, s);
     cur ^= 1;
   }
   return cur;
 }
-}  // namespace
 
-int radix_and_buckets(pm_ctx* c, int64_t n, cudaStream_t s) {
-  // bucket starts: exclusive scan of the nbuckets + 1 counts (last count is 0 -> total)
-  scan_exclusive(c, c->counts, c->bstart, c->nbuckets + 1, s);
-  if (n == 0) return PM_OK;
-  if ((n + kRadixTile - 1) / kRadixTile > c->hist_blocks_max) return PM_EINVAL;
+int radix_passes(pm_ctx* c, uint32_t* const kb[2], uint32_t* const vb[2], bool index_vals, bool counted, int64_t n,
+                 const uint32_t* flags, cudaStream_t s) {
+  if (c->radix_bits == 9) return passes_of<9>(c, kb, vb, index_vals, counted, n, flags, s);
+  if (c->radix_bits == 8) return passes_of<8>(c, kb, vb, index_vals, counted, n, flags, s);
+  return passes_of<7>(c, kb, vb, index_vals, counted, n, flags, s);
+}
+
+void sort_keys0(pm_ctx* c, bool counted, int64_t n, cudaStream_t s) {  // keys[0] -> keys[0], vals[0]
   uint32_t* const kb[2] = {c->keys[0], c->keys[1]};
   uint32_t* const vb[2] = {c->vals[0], c->vals[1]};
-  if (radix_passes(c, kb, vb, true, n, s) != 0) {  // keep the result in keys[0] / vals[0]
+  if (radix_passes(c, kb, vb, true, counted, n, nullptr, s) != 0) {  // keep the result in keys[0] / vals[0]
     std::swap(c->keys[0], c->keys[1]);
     std::swap(c->vals[0], c->vals[1]);
   }
+}
+
+}  // namespace
+
+int sort_by_keys(pm_ctx* c, int64_t n, cudaStream_t s) {
+  if (n > 0) sort_keys0(c, false, n, s);
   return PM_OK;
 }
 
 int sort_particles(pm_ctx* c, const uint32_t* u, int64_t n, cudaStream_t s) {
-  int st = build_keys(c, u, n, s);
-  if (st != PM_OK) return st;
-  return radix_and_buckets(c, n, s);
+  if (n == 0) {  // no gather will run: every bucket is empty
+    PM_CUDA_TRY(cudaMemsetAsync(c->bstart, 0, sizeof(uint32_t) * (c->nbuckets + 1), s));
+    return PM_OK;
+  }
+  {
+    LaunchScope L(c, s, K_KEYS);
+    const int shift = 32 - c->g.logn;
+    auto kern = c->radix_bits == 9 ? k_keys<9> : (c->radix_bits == 8 ? k_keys<8> : k_keys<7>);
+    kern<<<chunks_of(n), kCountThreads, 0, s>>>(u, n, shift, c->ntl, c->keys[0], c->hist);
+  }
+  sort_keys0(c, true, n, s);
+  return PM_OK;
 }
 
 void gather_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint32_t* id, int64_t n,
                    const uint32_t* perm, cudaStream_t s) {
   if (n == 0) return;
   LaunchScope L(c, s, K_GATHER);
-  k_gather<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(u, p, id, n, perm, c->us, c->ps, c->ids);
+  const unsigned nbb = (unsigned)((c->nbuckets + 1 + 255) / 256);
+  k_gather<<<nbb + (unsigned)((n + 255) / 256), 256, 0, s>>>(u, p, id, n, perm, c->us, c->ps, c->ids, c->keys[0],
+                                                            c->nbuckets + 1, nbb, c->bstart);
+}
+
+int clear_resort(pm_ctx* c, cudaStream_t s) {
+  PM_CUDA_TRY(cudaMemsetAsync(c->counts, 0, sizeof(uint32_t) * c->clear_words, s));
+  return PM_OK;
 }
 
 int resort_near_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint32_t* id, int64_t n,
                        cudaStream_t s) {
   const long long nb1 = c->nbuckets + 1;
-  // bucket starts, stayers' and old keys' movers' starts in one scan
-  scan_exclusive(c, c->counts, c->bstart, 3 * nb1, s);
-  if (n == 0) return 1;
-  PM_CUDA_TRY(cudaMemcpyAsync(c->rs_host, c->rs_dev, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  PM_CUDA_TRY(cudaMemcpyAsync(c->rs_host + 1, c->bstart + 2 * nb1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  PM_CUDA_TRY(cudaMemcpyAsync(c->rs_host + 2, c->bstart + 3 * nb1 - 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  PM_CUDA_TRY(cudaStreamSynchronize(s));
-  if (c->rs_host[0] & 1u) return 0;  // not the order of bprev: sort from scratch
-  const int64_t nm = (int64_t)c->rs_host[2] - (int64_t)c->rs_host[1];
-  if (nm < 0 || nm > n || (nm + kRadixTile - 1) / kRadixTile > c->hist_blocks_max) return PM_EINVAL;
-  c->rs_last_movers = nm;
+  {  // bucket starts, stayers' and old keys' movers' starts in one scan
+    LaunchScope L(c, s, K_SCAN);
+    k_scan<<<(unsigned)((3 * nb1 + kScanTile - 1) / kScanTile), kScanThreads, 0, s>>>(
+        c->counts, 3 * nb1, c->bstart, c->scan_status, c->scan_tile, c->err_dev);
+  }
   // the movers' records go to the second mesh, free during a step, when they fit (32 bytes a
   // mover: up to 2^30 movers at 2048^3); else the placement gathers from the state itself
-  uint4* stage = nullptr;
-  if (c->meshB && (size_t)nm * 32 <= c->g.elems() * sizeof(float2)) stage = reinterpret_cast<uint4*>(c->meshB);
+  uint4* const stage = reinterpret_cast<uint4*>(c->meshB);
+  const int64_t room = (int64_t)(c->g.elems() * sizeof(float2) / 32);
   {
     LaunchScope L(c, s, K_RESORT_PLACE);
     k_resort_old_tiles<<<(unsigned)((long long)c->nt * c->nt * c->nt), kResortThreads, 0, s>>>(
         u, p, id, n, c->keys[0], c->bprev, c->bstart, nb1, c->rs_low, c->us, c->ps, c->ids, c->keys[1], c->vals[1],
-        nm, c->err_dev, stage);
+        c->rs_dev, c->err_dev, stage, room);
   }
-  if (nm > 0) {
-    uint32_t* const kb[2] = {c->keys[1], c->rs_k2};
-    uint32_t* const vb[2] = {c->vals[1], c->rs_v2};
-    const int r = radix_passes(c, kb, vb, false, nm, s);
-    LaunchScope L(c, s, K_RESORT_MISC);
-    k_place_movers<<<(unsigned)((nm + 255) / 256), 256, 0, s>>>(kb[r], vb[r], nm, u, p, id, n, c->bstart, nb1,
-                                                                 c->nbuckets, c->rs_low, c->us, c->ps, c->ids,
-                                                                 c->err_dev, stage);
+  uint32_t* const kb[2] = {c->keys[1], c->rs_k2};
+  uint32_t* const vb[2] = {c->vals[1], c->rs_v2};
+  const int r = radix_passes(c, kb, vb, false, false, n, c->rs_dev, s);
+  LaunchScope L(c, s, K_RESORT_MISC);
+  static int full = 0;  // grid-stride: the CTAs that fill the GPU once
+  if (full == 0) {
+    int per_sm = 0, sms = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_place_movers, 256, 0);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    full = std::max(per_sm, 1) * std::max(sms, 1);
   }
-  return 1;
+  k_place_movers<<<(unsigned)std::min<int64_t>(full, (n + 255) / 256), 256, 0, s>>>(
+      kb[r], vb[r], u, p, id, n, c->bstart, nb1, c->nbuckets, c->rs_low, c->us, c->ps, c->ids, c->rs_dev, c->err_dev,
+      stage, room, c->rs_stats);
+  return PM_OK;
 }
 
 }  // namespace pmnu

@@ -52,6 +52,9 @@ enum Kind {
 constexpr int kTile = 16;        // tile edge in cells (the sort contract)
 constexpr int kMaxShell = 64;    // largest N_shell the mass table carries
 
+constexpr int kMaxChunks = 3 * 152;  // CTAs of the radix kernels (k_sort.cu): three an SM
+constexpr int kScanTile = 4096;  // words a CTA of the scan takes
+
 // Particle-mass lookup from the canonical id (passed by value to kernels).
 struct MassTable {
   int64_t n_cdm;   // ids below are CDM
@@ -122,8 +125,7 @@ struct pm_ctx {
   uint32_t* us = nullptr;
   float* ps = nullptr;
   uint32_t* ids = nullptr;
-  uint32_t* counts = nullptr;   // 3 (nbuckets + 1), see below
-  uint32_t* bstart = nullptr;   // 3 (nbuckets + 1)
+  uint32_t* bstart = nullptr;   // 3 (nbuckets + 1), see below
   // near-sorted re-sort of pm_step (k_sort.cu).  counts, bstart and bprev hold three
   // arrays of nbuckets + 1 words each: counts = [per new key | stayers per new key |
   // movers per old key], scanned as one array into bstart (bucket starts, then the two
@@ -131,18 +133,20 @@ struct pm_ctx {
   // step left its state in (valid for rs_n particles, -1: none).
   uint32_t* bprev = nullptr;
   int64_t rs_n = -1;
+  // one allocation, zeroed (clear_words) before each drift that counts: counts, rs_low,
+  // rs_dev, the scan's tile counter and status words
+  uint32_t* counts = nullptr;     // 3 (nbuckets + 1)
+  size_t clear_words = 0;
   uint32_t* rs_low = nullptr;     // movers from a lower old key, per new key (nbuckets + 1)
+  uint32_t* rs_dev = nullptr;     // flag bits of k_kick_drift_keys<true>
+  unsigned long long* scan_status = nullptr;
+  uint32_t* scan_tile = nullptr;
   uint32_t* rs_k2 = nullptr;      // second (key, index) buffer pair of the movers' radix
   uint32_t* rs_v2 = nullptr;
-  uint32_t* rs_dev = nullptr;     // flag bits of k_kick_drift_keys<true>
-  uint32_t* rs_host = nullptr;    // pinned: flags, first word of the third scan, last word
-  int64_t rs_fast = 0, rs_full = 0;  // re-sorts done the near-sorted way / from scratch
-  int64_t rs_last_movers = 0;        // movers of the last near-sorted re-sort
-  uint32_t* hist = nullptr;     // 256 * radix blocks, raw
-  uint32_t* hist_scan = nullptr;
-  uint32_t* scan_tmp = nullptr;
-  size_t scan_tmp_elems = 0;
-  long long hist_blocks_max = 0;
+  long long* rs_stats = nullptr;  // device: re-sorts near-sorted, from scratch, movers of the last near-sorted one
+  int64_t rs_full = 0;            // re-sorts that the host sent to the sort from scratch
+  uint32_t* hist = nullptr;       // digit counts per chunk of a radix pass, then the digits' totals
+  uint32_t* digit_totals = nullptr;
   // masses
   pmnu::MassTable mt{};
   double m_cdm = 0.0;
@@ -218,10 +222,10 @@ int ctx_alloc_n(pm_ctx* c, T** p, size_t count) {
 }
 
 // host launch helpers implemented in the .cu files
-int sort_particles(pm_ctx* c, const uint32_t* u, int64_t n, cudaStream_t s);  // keys + radix -> vals
-int build_keys(pm_ctx* c, const uint32_t* u, int64_t n, cudaStream_t s);
-int radix_and_buckets(pm_ctx* c, int64_t n, cudaStream_t s);                 // after keys
-void scan_exclusive(pm_ctx* c, const uint32_t* in, uint32_t* out, long long n, cudaStream_t s);
+// stable sort by key: sorted keys in keys[0], permutation in vals[0]
+int sort_particles(pm_ctx* c, const uint32_t* u, int64_t n, cudaStream_t s);
+int sort_by_keys(pm_ctx* c, int64_t n, cudaStream_t s);  // keys[0] given
+// after either sort: the sorted copies and the bucket starts (nothing for n = 0)
 void gather_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint32_t* id, int64_t n,
                    const uint32_t* perm, cudaStream_t s);
 // weights (sorted order, signed) replace the species masses when non-null
@@ -257,10 +261,10 @@ void readout_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint32_t
 // resort: also classify the particles against bprev for resort_near_sorted
 void kick_drift_keys(pm_ctx* c, uint32_t* u, float* p, const float* f, int64_t n, float K1,
                      float dscale, cudaStream_t s, bool resort);
-// After kick_drift_keys(resort = true): bucket starts, and if the state was in bprev's
-// order, the sorted copies us / ps / ids of (u, p, id) with the stable order of keys[0]
-// (returns 1); returns 0 (nothing written but bstart) when the caller must sort from
-// scratch, a negative status on error.  Synchronises the stream once.
+// zeroes what a counting drift and the re-sort after it add to
+int clear_resort(pm_ctx* c, cudaStream_t s);
+// After kick_drift_keys(resort = true) or a drifting readout: bucket starts and the sorted
+// copies us / ps / ids of (u, p, id) with the stable order of keys[0] (n > 0)
 int resort_near_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint32_t* id, int64_t n,
                        cudaStream_t s);
 void repack_real(pm_ctx* c, const Geom& g, const float* src, int src_pitch, float* dst,
