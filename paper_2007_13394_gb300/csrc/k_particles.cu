@@ -89,22 +89,75 @@ __device__ __forceinline__ float float64w(unsigned int hi, unsigned int lo) {
   return __ll2float_rn((long long)(((unsigned long long)hi << 32) | (unsigned long long)lo));
 }
 
-// Paint of one tile.  FAST: 32-bit low words only (half the shared memory of the carry form:
+// A tile whose list of wraps overflowed, painted again by its CTA: half of its x planes at a
+// time in two words a cell, which fit where the low words of the whole tile were.  Out of line:
+// rare, and the main form keeps its 32 registers.  Every thread of the CTA calls it.
+__device__ __noinline__ void paint_halves(uint32_t tile, unsigned int* __restrict__ accw,
+                                          const uint32_t* __restrict__ run_lo, const uint32_t* __restrict__ run_pre,
+                                          const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
+                                          float* __restrict__ mesh, const MassTable& mt, int species, int nm, int shift,
+                                          int ntl, int row_pitch) {
+  constexpr int HX = kTile / 2, WORDS = HX * kSx;
+  const int t = threadIdx.x, nt = 1 << ntl;
+  const int ox = (int)(tile >> (2 * ntl)) * kTile, oy = (int)((tile >> ntl) & (nt - 1)) * kTile,
+            oz = (int)(tile & (nt - 1)) * kTile;
+  const float fscale = 1.0f / (float)(1u << shift);
+  const uint32_t fmask = (1u << shift) - 1u, total = run_pre[14];
+  for (int x0 = 0; x0 < kTile; x0 += HX) {
+    __syncthreads();  // the accumulators are free
+    for (int i = t; i < 2 * WORDS; i += kPaintThreads) accw[i] = 0;
+    __syncthreads();
+    int r = 0;
+    for (uint32_t v = t; v < total; v += kPaintThreads) {
+      while (v >= run_pre[r + 1]) ++r;
+      const uint32_t k = run_lo[r] + (v - run_pre[r]);
+      const uint32_t q[3] = {us[k], us[n + k], us[2 * n + k]};
+      bool bad = false;  // reported by the first pass
+      const float m = id_mass(mt, ids[k], species, &bad);
+      if (m == 0.0f) continue;
+      int l[3] = {(int)(q[0] >> shift) - ox, (int)(q[1] >> shift) - oy, (int)(q[2] >> shift) - oz};
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {  // periodic wrap relative to the tile origin
+        if (l[d] > nm / 2) l[d] -= nm;
+        if (l[d] < -nm / 2) l[d] += nm;
+      }
+      const float fx = (float)(q[0] & fmask) * fscale, fy = (float)(q[1] & fmask) * fscale,
+                  fz = (float)(q[2] & fmask) * fscale;
+      for (int corner = 0; corner < 8; ++corner) {
+        const int bx = corner >> 2, by = (corner >> 1) & 1, bz = corner & 1;
+        const int x = l[0] + bx - x0, y = l[1] + by, z = l[2] + bz;
+        if ((unsigned)x >= (unsigned)HX || (unsigned)y >= (unsigned)kTile || (unsigned)z >= (unsigned)kTile) continue;
+        const float wc = (bx ? fx : 1.0f - fx) * (by ? fy : 1.0f - fy) * (bz ? fz : 1.0f - fz);
+        const unsigned int qv = __float2uint_rn(wc * m * kFixM);  // < 2^31: masses below 128
+        unsigned int* const lo = accw + x * kSx + y * kSy + z;
+        const unsigned int old = atomicAdd(lo, qv);
+        if (old + qv < old) atomicAdd(lo + WORDS, 1u);
+      }
+    }
+    __syncthreads();
+    for (int q = t; q < HX * kTile * kTile; q += kPaintThreads) {
+      const int x = q / (kTile * kTile), y = (q / kTile) % kTile, z = q % kTile;
+      const int a = x * kSx + y * kSy + z;
+      mesh[((size_t)(ox + x0 + x) * nm + (oy + y)) * (size_t)row_pitch + oz + z] = float64w(accw[WORDS + a], accw[a]) * kUnfixM;
+    }
+  }
+}
+
+// Paint of one tile.  FAST: 32-bit low words only (half the shared memory of the two-word form:
 // zeroed, and read at the write-out, once per cell).  A low word that wraps past 2^32 (the
 // cell passes another 256 mean cell masses) is recorded as an event -- the cell's bit in a
 // bitmap, its index in a list of up to kWraps events -- and at the write-out a cell whose
 // bit is set counts its events in the list: value = events 2^32 + low word.  A tile with
-// more events than the list holds is written to the redo list and left unwritten; the redo
-// pass paints it in full in the two-word form.  Every form sums the same exact integers, so
-// all give the same floats.  Else two words a cell and NW = 0 (masses), or NW = 1 or 3 signed
+// more events than the list holds is painted again (paint_halves).  Every form sums the same
+// exact integers, so all give the same floats.  Else two words a cell and NW = 0 (masses), or NW = 1 or 3 signed
 // weights a particle (wts[j n + k]), weight j painted onto mesh j (mesh, mesh1, mesh2).
 template <bool FAST, int NW, int NT>
 __device__ __forceinline__ void paint_tile(
     uint32_t tile, unsigned int* __restrict__ accw, uint32_t* __restrict__ run_lo, uint32_t* __restrict__ run_pre,
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
     const uint32_t* __restrict__ bstart, float* __restrict__ mesh, const MassTable& mt, int species, int nm,
-    int shift, int ntl, int row_pitch, int* __restrict__ err, const float* __restrict__ wts, float mmax,
-    uint32_t* __restrict__ redo, float* __restrict__ mesh1 = nullptr, float* __restrict__ mesh2 = nullptr) {
+    int shift, int ntl, int row_pitch, int* __restrict__ err, const float* __restrict__ wts,
+    float* __restrict__ mesh1 = nullptr, float* __restrict__ mesh2 = nullptr) {
   constexpr int NA = NW > 1 ? NW : 1;  // meshes painted
   // FAST: low words, then the wrap bitmap, the event count and the event list.  Else per
   // mesh the low words, then the high words.
@@ -150,8 +203,6 @@ __device__ __forceinline__ void paint_tile(
   const uint32_t total = run_pre[14];
   // One particle per thread (coalesced loads in bucket order), its 8 corners added by
   // the same thread.
-  // masses below 128: w 2^24 < 2^31, so 32-bit conversions and a carry of at most 1
-  const bool narrow = FAST || (NW == 0 && mmax < 128.0f);
   const int ox = tx * kTile, oy = ty * kTile, oz = tz * kTile;
   bool bad = false, wrap = false;
   int r = 0;
@@ -208,12 +259,7 @@ __device__ __forceinline__ void paint_tile(
         if constexpr (FAST) {
           const unsigned int q = __float2uint_rn(wc * m[0] * kFixM);  // < 2^31: masses below 128
           const unsigned int old = atomicAdd(&acc_lo[ad], q);
-          // the low word wrapped; a full list sends the tile to the redo pass
-          if (old + q < old && !record_wrap(accw, ad)) wrap = true;
-        } else if (narrow) {
-          const unsigned int q = __float2uint_rn(wc * m[0] * kFixM);
-          const unsigned int old = atomicAdd(&acc_lo[ad], q);
-          if (old + q < old) atomicAdd(&acc_lo[kAccWords + ad], 1u);
+          if (old + q < old && !record_wrap(accw, ad)) wrap = true;  // the low word wrapped; a full list
         } else {
 #pragma unroll
           for (int j = 0; j < NA; ++j) {
@@ -226,10 +272,9 @@ __device__ __forceinline__ void paint_tile(
   }
   if (bad) atomicOr(err, 1);
   if constexpr (FAST) {
-    // the barrier's vote tells every thread whether the event list overflowed (the redo pass
-    // then paints this tile)
+    // the barrier's vote tells every thread whether the event list overflowed
     if (__syncthreads_or(wrap ? 1 : 0)) {
-      if (t == 0) redo[1 + atomicAdd(redo, 1u)] = tile;
+      paint_halves(tile, accw, run_lo, run_pre, us, ids, n, mesh, mt, species, nm, shift, ntl, row_pitch);
       return;
     }
   } else {
@@ -271,19 +316,17 @@ __device__ __forceinline__ void paint_tile(
   }
 }
 
-// One CTA per tile.  FAST: the 32-bit form with wrap events, tiles whose event list
-// overflows sent to the redo list (redo[0] = count, redo[1 ..] = tiles); else the two-word
-// form, with NW signed weights instead of masses when NW > 0.
+// One CTA per tile.  FAST: the 32-bit form with wrap events (masses below 128); else the
+// two-word form, with NW signed weights instead of masses when NW > 0.
 template <bool FAST, int NW>
 __global__ void __launch_bounds__(kPaintThreads, FAST ? 8 : 1) k_paint_tiles(
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
-    const uint32_t* __restrict__ bstart, float* __restrict__ mesh, MassTable mt, int species,
-    int nm, int shift, int ntl, int row_pitch, int* __restrict__ err, const float* __restrict__ wts,
-    float mmax, uint32_t* __restrict__ redo) {
+    const uint32_t* __restrict__ bstart, float* __restrict__ mesh, const __grid_constant__ MassTable mt, int species,
+    int nm, int shift, int ntl, int row_pitch, int* __restrict__ err, const float* __restrict__ wts) {
   __shared__ __align__(16) unsigned int accw[FAST ? kFastWords : 2 * kAccWords];
   __shared__ uint32_t run_lo[14], run_pre[15];
   paint_tile<FAST, NW, kPaintThreads>(blockIdx.x, accw, run_lo, run_pre, us, ids, n, bstart, mesh, mt, species, nm,
-                                      shift, ntl, row_pitch, err, wts, mmax, redo);
+                                      shift, ntl, row_pitch, err, wts);
 }
 
 // Three signed weights a particle onto three meshes in one pass over the particles: positions,
@@ -299,24 +342,7 @@ __global__ void __launch_bounds__(kPaint3Threads, 2) k_paint_weights3(
   __shared__ uint32_t run_lo[14], run_pre[15];
   const MassTable none{};
   paint_tile<false, 3, kPaint3Threads>(blockIdx.x, accw3, run_lo, run_pre, us, nullptr, n, bstart, m0, none, 0, nm,
-                                       shift, ntl, row_pitch, err, wts, 0.0f, nullptr, m1, m2);
-}
-
-// The redo pass: the tiles the fast pass listed, painted in the two-word form
-// (persistent CTAs walk the list; an empty list, the normal case, costs one launch).
-__global__ void __launch_bounds__(kPaintThreads) k_paint_redo(
-    const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
-    const uint32_t* __restrict__ bstart, float* __restrict__ mesh, MassTable mt, int species,
-    int nm, int shift, int ntl, int row_pitch, int* __restrict__ err, float mmax,
-    const uint32_t* __restrict__ redo) {
-  __shared__ __align__(16) unsigned int accw[2 * kAccWords];
-  __shared__ uint32_t run_lo[14], run_pre[15];
-  const uint32_t count = redo[0];
-  for (uint32_t q = blockIdx.x; q < count; q += gridDim.x) {
-    paint_tile<false, 0, kPaintThreads>(redo[1 + q], accw, run_lo, run_pre, us, ids, n, bstart, mesh, mt, species, nm,
-                                        shift, ntl, row_pitch, err, nullptr, mmax, nullptr);
-    __syncthreads();  // the shared accumulators are reused by the next tile
-  }
+                                       shift, ntl, row_pitch, err, wts, m1, m2);
 }
 
 // CIC readout of one real mesh component fused with the kick p_j += K F_j.
@@ -712,32 +738,11 @@ void paint_tiles(pm_ctx* c, const uint32_t* us, const uint32_t* ids, int64_t n, 
   if (species & PM_SPECIES_CDM) mmax = std::max(mmax, c->mt.m_cdm);
   if (species & PM_SPECIES_NU)
     for (int i = 0; i < c->mt.nshell && i < kMaxShell; ++i) mmax = std::max(mmax, c->mt.m_nu[i]);
-  if (weights == nullptr && mmax < 128.0f && c->paint_redo) {
-    // 32-bit pass, then the tiles whose words wrapped, in the carry form
-    cudaMemsetAsync(c->paint_redo, 0, sizeof(uint32_t), s);
-    {
-      LaunchScope L(c, s, K_PAINT);
-      k_paint_tiles<true, 0><<<grid, kPaintThreads, 0, s>>>(us, ids, n, c->bstart, mesh, c->mt, species, c->g.n,
-                                                            32 - c->g.logn, c->ntl, row_pitch, c->err_dev, nullptr,
-                                                            mmax, c->paint_redo);
-    }
-    // persistent CTAs, as many as fit: the list is short, or empty, in most steps
-    static int per_sm = 0, sms = 0;
-    if (per_sm == 0) {
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_paint_redo, kPaintThreads, 0);
-      if (per_sm < 1) per_sm = 1;
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    }
-    LaunchScope L(c, s, K_PAINT_REDO);
-    k_paint_redo<<<(unsigned)std::min<long long>((long long)per_sm * sms, grid), kPaintThreads, 0, s>>>(
-        us, ids, n, c->bstart, mesh, c->mt, species, c->g.n, 32 - c->g.logn, c->ntl, row_pitch, c->err_dev, mmax,
-        c->paint_redo);
-    return;
-  }
   LaunchScope L(c, s, K_PAINT);
-  auto kern = weights ? k_paint_tiles<false, 1> : k_paint_tiles<false, 0>;
+  // masses below 128: w 2^24 < 2^31, so every contribution fits the 32-bit form
+  auto kern = weights ? k_paint_tiles<false, 1> : (mmax < 128.0f ? k_paint_tiles<true, 0> : k_paint_tiles<false, 0>);
   kern<<<grid, kPaintThreads, 0, s>>>(us, ids, n, c->bstart, mesh, c->mt, species, c->g.n, 32 - c->g.logn, c->ntl,
-                                      row_pitch, c->err_dev, weights, mmax, nullptr);
+                                      row_pitch, c->err_dev, weights);
 }
 
 void paint_weights3(pm_ctx* c, const uint32_t* us, int64_t n, const float* weights, float* m0, float* m1, float* m2,

@@ -274,8 +274,9 @@ __global__ void __launch_bounds__(256) k_chunk_scan(uint32_t* __restrict__ hist,
 
 // ------------------------------------------------------------------ radix scatter
 // One stable pass over (key, value) pairs (vin null: the value is the index), see the top of
-// the file: hist holds the chunk's exclusive counts per digit, totals every digit's count.
-template <int BITS>
+// the file: hist holds the chunks' exclusive counts per digit and totals every digit's count, or
+// (RAW, few chunks: a launch costs more than the sums) the counts themselves.
+template <int BITS, bool RAW>
 __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift,
     const uint32_t* __restrict__ hist, const uint32_t* __restrict__ totals, uint32_t* __restrict__ kout,
@@ -302,13 +303,28 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
     uint32_t c[PER], sum = 0;
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-      c[q] = owner ? totals[t * PER + q] : 0u;
+      c[q] = 0u;
+      next[q] = 0u;
+      if (owner) {
+        const uint32_t* const h = hist + (size_t)(t * PER + q) * gridDim.x;
+        if constexpr (RAW) {
+#pragma unroll 8
+          for (int k = 0; k < (int)gridDim.x; ++k) {
+            const uint32_t v = h[k];
+            c[q] += v;
+            if (k < (int)blockIdx.x) next[q] += v;
+          }
+        } else {
+          c[q] = totals[t * PER + q];
+          next[q] = h[blockIdx.x];
+        }
+      }
       sum += c[q];
     }
     uint32_t ex = block_exclusive_scan(sum, ws, nullptr);
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-      next[q] = owner ? ex + hist[(size_t)(t * PER + q) * gridDim.x + blockIdx.x] : 0u;
+      next[q] += ex;
       ex += c[q];
     }
   }
@@ -627,17 +643,22 @@ unsigned chunks_of(int64_t n) {
   return (unsigned)std::min<int64_t>(kMaxChunks, std::max<int64_t>(1, (n + kRadixTile - 1) / kRadixTile));
 }
 
+// up to 32 chunks (131 k keys) the scatter adds up the counts itself
+bool raw_counts(int64_t n) { return chunks_of(n) <= 32; }
+
 template <int BITS>
 void launch_scatter(pm_ctx* c, const uint32_t* kin, const uint32_t* vin, int64_t n, int shift, uint32_t* kout,
                     uint32_t* vout, const uint32_t* flags, cudaStream_t s) {
   const size_t dyn = 2 * kRadixTile * sizeof(uint32_t);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_radix_scatter<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    attr = true;
+  const bool raw = raw_counts(n);
+  auto kern = raw ? k_radix_scatter<BITS, true> : k_radix_scatter<BITS, false>;
+  static bool attr[2] = {false, false};
+  if (!attr[raw]) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    attr[raw] = true;
   }
-  k_radix_scatter<BITS><<<chunks_of(n), kRadixThreads, dyn, s>>>(kin, vin, n, shift, c->hist, c->digit_totals, kout, vout,
-                                                                flags, c->bstart, c->nbuckets + 1);
+  kern<<<chunks_of(n), kRadixThreads, dyn, s>>>(kin, vin, n, shift, c->hist, c->digit_totals, kout, vout, flags,
+                                                c->bstart, c->nbuckets + 1);
 }
 
 // LSD radix passes over n (key, value) pairs in buffer pair 0 (values absent: the incoming
@@ -654,7 +675,7 @@ int passes_of(pm_ctx* c, uint32_t* const kb[2], uint32_t* const vb[2], bool inde
       LaunchScope L(c, s, K_RADIX_HIST);
       k_digits<BITS><<<C, kCountThreads, 0, s>>>(kb[cur], n, shift, c->hist, flags, c->bstart, c->nbuckets + 1);
     }
-    {
+    if (!raw_counts(n)) {
       LaunchScope L(c, s, K_SCAN);
       k_chunk_scan<<<(1 << BITS) / 8, 256, 0, s>>>(c->hist, (int)C, 1 << BITS, c->digit_totals);
     }
