@@ -112,18 +112,13 @@ void free_all(pm_ctx* c) {
   ctx_free(c, c->winv);
   ctx_free(c, c->wforce);
   ctx_free(c, c->kvec0);
-  for (int i = 0; i < 2; ++i) {
-    ctx_free(c, c->keys[i]);
-    ctx_free(c, c->vals[i]);
-  }
+  ctx_free(c, c->sortbuf);
   ctx_free(c, c->us);
   ctx_free(c, c->ps);
   ctx_free(c, c->ids);
   ctx_free(c, c->counts);
   ctx_free(c, c->bstart);
   ctx_free(c, c->bprev);
-  ctx_free(c, c->rs_k2);
-  ctx_free(c, c->rs_v2);
   ctx_free(c, c->rs_stats);
   ctx_free(c, c->hist);
   ctx_free(c, c->pk_partial);
@@ -466,11 +461,10 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
   const bool two_mesh = (cfg->flags & PM_FLAG_TWO_MESH) != 0 || N >= 2048;
   if ((!two_mesh && dalloc(c, &c->meshC, me)) || dalloc(c, &c->meshA, me) || dalloc(c, &c->meshB, me) ||
       dalloc(c, &c->ksq, N) ||
-      dalloc(c, &c->winv, N) || dalloc(c, &c->wforce, N) || dalloc(c, &c->kvec0, N) || dalloc(c, &c->keys[0], nm) ||
-      dalloc(c, &c->keys[1], nm) || dalloc(c, &c->vals[0], nm) || dalloc(c, &c->vals[1], nm) ||
+      dalloc(c, &c->winv, N) || dalloc(c, &c->wforce, N) || dalloc(c, &c->kvec0, N) || dalloc(c, &c->sortbuf, 6 * nm) ||
       dalloc(c, &c->us, 3 * nm) || dalloc(c, &c->ps, 3 * nm) || dalloc(c, &c->ids, nm) ||
       dalloc(c, &c->counts, clear_words) || dalloc(c, &c->bstart, 3 * (c->nbuckets + 1)) ||
-      dalloc(c, &c->bprev, 3 * (c->nbuckets + 1)) || dalloc(c, &c->rs_k2, nm) || dalloc(c, &c->rs_v2, nm) ||
+      dalloc(c, &c->bprev, 3 * (c->nbuckets + 1)) ||
       dalloc(c, &c->rs_stats, 3) || dalloc(c, &c->hist, hist_words) ||
       dalloc(c, &c->pk_partial, (size_t)N * 2 * 2048) ||
       dalloc(c, &c->pk_final, 3 * 2048) || dalloc(c, &c->err_dev, 1)) {
@@ -484,6 +478,8 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
     return PM_ENOMEM;
   }
   cudaMemset(c->err_dev, 0, sizeof(int));
+  uint32_t** const sorted[6] = {&c->keys[0], &c->vals[0], &c->rs_k2, &c->rs_v2, &c->keys[1], &c->vals[1]};
+  for (int i = 0; i < 6; ++i) *sorted[i] = c->sortbuf + i * nm;
   c->rs_low = c->counts + 3 * (c->nbuckets + 1);
   c->rs_dev = c->counts + flag_at;
   c->scan_tile = c->rs_dev + 1;

@@ -119,6 +119,9 @@ struct pm_ctx {
   float* wforce = nullptr;
   float* kvec0 = nullptr;
   // sort / particle scratch
+  // one allocation of six arrays of n_max words: keys[0], vals[0], rs_k2, rs_v2, keys[1],
+  // vals[1]; the pairs 0 and 1 may be exchanged, so four adjoining arrays are free after a sort
+  uint32_t* sortbuf = nullptr;
   uint32_t* keys[2] = {nullptr, nullptr};
   uint32_t* vals[2] = {nullptr, nullptr};
   uint32_t* us = nullptr;
