@@ -464,6 +464,44 @@ __device__ __forceinline__ uint32_t drift_fixed(uint32_t u, float dscale, float 
   return u + step;
 }
 
+// Counts for the near-sorted re-sort, by the lanes of act: all particles by new key kn, stayers
+// (new key = old key) by new key, movers by old key, movers from a lower key by new key.  The
+// lanes hold consecutive particles of the state; those in range of their old key ko (in) have
+// old keys that never decrease from lane to lane, so stayers and movers are counted per run
+// of equal old keys with ballots, and only the movers' new keys need a match over the lanes.
+__device__ __forceinline__ void count_resort(unsigned act, uint32_t kn, uint32_t ko, bool in, uint32_t* __restrict__ cnt3,
+                                             long long nb1, uint32_t* __restrict__ low) {
+  const int lane = threadIdx.x & 31;
+  const bool stay = in && kn == ko;
+  const unsigned below = act & ((1u << lane) - 1u);
+  const int prev = below ? 31 - __clz(below) : lane;  // the nearest active lane below
+  const uint32_t run_key = in ? ko : 0xffffffffu;
+  const uint32_t prev_key = __shfl_sync(act, run_key, prev);
+  const bool head = prev == lane || prev_key != run_key;
+  const unsigned heads = __ballot_sync(act, head);
+  const unsigned stays = __ballot_sync(act, stay);
+  const unsigned lows = __ballot_sync(act, in && ko < kn);
+  if (head && in) {
+    const unsigned after = heads & ~((2u << lane) - 1u);  // heads above this lane (lane 31: none)
+    const unsigned upto = after ? (1u << (__ffs(after) - 1)) - 1u : 0xffffffffu;
+    const unsigned run = act & upto & ~((1u << lane) - 1u);
+    const uint32_t ns = (uint32_t)__popc(run & stays), nmv = (uint32_t)__popc(run & ~stays);
+    if (ns) {
+      atomicAdd(cnt3 + ko, ns);
+      atomicAdd(cnt3 + nb1 + ko, ns);
+    }
+    if (nmv) atomicAdd(cnt3 + 2 * nb1 + ko, nmv);
+  }
+  if (!stay) {
+    const unsigned peers = __match_any_sync(act & ~stays, kn);
+    if (lane == __ffs(peers) - 1) {
+      atomicAdd(cnt3 + kn, (uint32_t)__popc(peers));
+      const uint32_t nl = (uint32_t)__popc(peers & lows);
+      if (nl) atomicAdd(low + kn, nl);
+    }
+  }
+}
+
 __device__ __forceinline__ void drift_next(const DriftNext& dn, const float (&F)[3], const float (&pv)[3],
                                            float K2, int64_t n, uint32_t i, uint32_t ux, uint32_t uy, uint32_t uz,
                                            int shift, int ntl, float* __restrict__ p_out, float* __restrict__ f_out,
@@ -481,40 +519,7 @@ __device__ __forceinline__ void drift_next(const DriftNext& dn, const float (&F)
   const uint32_t kn = tile_key(uu[0], uu[1], uu[2], shift, ntl);
   const uint32_t ko = tile_key(ux, uy, uz, shift, ntl);
   dn.keys[i] = kn;
-  // counts: all particles by new key, stayers by new key, movers by old key, movers from a
-  // lower key by new key.  The lanes here hold consecutive particles of the tile's sorted
-  // range, so their old keys never decrease from lane to lane: stayers (new key = old key)
-  // and movers are counted per run of equal old keys with ballots, and only the movers'
-  // new keys need a match over the lanes.
-  const unsigned act = __activemask();
-  const int lane = threadIdx.x & 31;
-  const bool stay = kn == ko;
-  const unsigned below = act & ((1u << lane) - 1u);
-  const int prev = below ? 31 - __clz(below) : lane;  // the nearest active lane below
-  const uint32_t ko_prev = __shfl_sync(act, ko, prev);
-  const bool head = prev == lane || ko_prev != ko;
-  const unsigned heads = __ballot_sync(act, head);
-  const unsigned stays = __ballot_sync(act, stay);
-  const unsigned lows = __ballot_sync(act, !stay && ko < kn);
-  if (head) {
-    const unsigned after = heads & ~((2u << lane) - 1u);  // heads above this lane (lane 31: none)
-    const unsigned upto = after ? (1u << (__ffs(after) - 1)) - 1u : 0xffffffffu;
-    const unsigned run = act & upto & ~((1u << lane) - 1u);
-    const uint32_t ns = (uint32_t)__popc(run & stays), nmv = (uint32_t)__popc(run & ~stays);
-    if (ns) {
-      atomicAdd(dn.cnt3 + ko, ns);
-      atomicAdd(dn.cnt3 + dn.nb1 + ko, ns);
-    }
-    if (nmv) atomicAdd(dn.cnt3 + 2 * dn.nb1 + ko, nmv);
-  }
-  if (!stay) {
-    const unsigned peers = __match_any_sync(act & ~stays, kn);
-    if (lane == __ffs(peers) - 1) {
-      atomicAdd(dn.cnt3 + kn, (uint32_t)__popc(peers));
-      const uint32_t nl = (uint32_t)__popc(peers & lows);
-      if (nl) atomicAdd(dn.low + kn, nl);
-    }
-  }
+  count_resort(__activemask(), kn, ko, true, dn.cnt3, dn.nb1, dn.low);
 }
 
 constexpr int kFd4Threads = 256;
@@ -523,6 +528,11 @@ constexpr int kSpanZ = kTile + 8;                  // cells -4 .. 19 along z
 constexpr int kChunksZ = kSpanZ / 4;               // 16-byte chunks per staged z row
 constexpr int kStageChunks = kSpanXY * kSpanXY * kChunksZ;
 constexpr int kFd4SY = kSpanZ, kFd4SX = kSpanXY * kSpanZ;
+constexpr int kNodeThreads = 512;
+constexpr int kNodesMin = 1500;    // mean particles a tile from which the node form is taken
+constexpr int kNodes = kTile + 1;  // corner nodes of a tile per axis
+constexpr size_t kFd4Smem = sizeof(float) * kSpanXY * kFd4SX;
+constexpr size_t kNodeSmem = kFd4Smem + sizeof(float) * 3 * kNodes * kNodes * kNodes;
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)),
@@ -530,14 +540,40 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
                : "memory");
 }
 
-template <bool DRIFT>
-__global__ void __launch_bounds__(kFd4Threads) k_readout_fd4_kick(
+// The tile's potential with its halo into sp, by asynchronous copies of one group.  Chunk k of
+// staged row (x, y) holds cells oz - 4 + 4k .. oz - 1 + 4k (mod N): contiguous and 16-byte aligned
+// because N, oz and the row pitch are multiples of 4 floats.
+template <int NT>
+__device__ __forceinline__ void stage_potential(float* sp, const float* __restrict__ phi, int ox, int oy, int oz, int nm,
+                                                int row_pitch) {
+  const int wrap = nm - 1;
+  for (int c = threadIdx.x; c < kStageChunks; c += NT) {
+    const int x = c / (kSpanXY * kChunksZ), r = c - x * (kSpanXY * kChunksZ);
+    const int y = r / kChunksZ, k = r - y * kChunksZ;
+    const int gx = (ox + x - 2) & wrap, gy = (oy + y - 2) & wrap, gz = (oz - 4 + 4 * k) & wrap;
+    cp_async16(sp + x * kFd4SX + y * kFd4SY + 4 * k, phi + ((size_t)gx * nm + gy) * (size_t)row_pitch + gz);
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// NODES = false: each particle gathers the 56 potential values of its 8 corners' stencils
+// (207 shared-memory wavefronts a warp: random cells, about 3.7 conflicts a gather).  NODES =
+// true: the CTA first computes the force at the tile's 17^3 corner nodes (2500 wavefronts, free
+// of conflicts), then each particle gathers 8 x 3 values (89 wavefronts a warp).  us a launch of
+// 4096 tiles, gathering / nodes, by mean particles a tile: 500 63 / 104, 1000 113 / 131, 1500
+// 162 / 157, 2000 211 / 184, 4000 411 / 292, 8000 806 / 494.
+// The gathering form runs five CTAs an SM (48 registers; at 60 to 104 it holds four to two: 4.65
+// to 6.2 ms against 4.1 on the late steps of 152 M particles at 1024^3).
+template <bool DRIFT, bool NODES>
+__global__ void __launch_bounds__(NODES ? kNodeThreads : kFd4Threads, NODES ? 2 : 5) k_readout_fd4_kick(
     const uint32_t* __restrict__ us, const float* __restrict__ ps, const uint32_t* __restrict__ ids,
     int64_t n, const uint32_t* __restrict__ bstart, const float* __restrict__ phi, int nm, int shift,
     int ntl, int row_pitch, float inv12h, float K, float* __restrict__ p_out, float* __restrict__ f_out,
     uint32_t* __restrict__ u_out, uint32_t* __restrict__ id_out, const uint32_t* __restrict__ perm,
     int* __restrict__ err, DriftNext dn) {
-  __shared__ __align__(16) float sp[kSpanXY * kSpanXY * kSpanZ];
+  constexpr int NT = NODES ? kNodeThreads : kFd4Threads;
+  extern __shared__ __align__(16) float sp[];  // the potential, then (NODES) the nodes' forces
+  float* const nodes = sp + kSpanXY * kFd4SX;
   const int t = threadIdx.x;
   const uint32_t tile = blockIdx.x;
   const uint32_t lo = bstart[8 * tile], hi = bstart[8 * tile + 8];
@@ -545,16 +581,7 @@ __global__ void __launch_bounds__(kFd4Threads) k_readout_fd4_kick(
   const int nt = 1 << ntl;
   const int ox = (int)(tile >> (2 * ntl)) * kTile, oy = (int)((tile >> ntl) & (nt - 1)) * kTile,
             oz = (int)(tile & (nt - 1)) * kTile;
-  const int wrap = nm - 1;
-  // chunk k of staged row (x, y) holds cells oz - 4 + 4k .. oz - 1 + 4k (mod N): contiguous
-  // and 16-byte aligned because N, oz and the row pitch are multiples of 4 floats
-  for (int c = t; c < kStageChunks; c += kFd4Threads) {
-    const int x = c / (kSpanXY * kChunksZ), r = c - x * (kSpanXY * kChunksZ);
-    const int y = r / kChunksZ, k = r - y * kChunksZ;
-    const int gx = (ox + x - 2) & wrap, gy = (oy + y - 2) & wrap, gz = (oz - 4 + 4 * k) & wrap;
-    cp_async16(sp + x * kFd4SX + y * kFd4SY + 4 * k, phi + ((size_t)gx * nm + gy) * (size_t)row_pitch + gz);
-  }
-  asm volatile("cp.async.commit_group;" ::: "memory");
+  stage_potential<NT>(sp, phi, ox, oy, oz, nm, row_pitch);
   // a particle's position, momentum and id are loaded one iteration ahead
   const bool kick = ps != nullptr && perm == nullptr;
   auto load = [&](uint32_t j, uint32_t (&uq)[3], float (&pq)[3], uint32_t& idq) {
@@ -571,11 +598,22 @@ __global__ void __launch_bounds__(kFd4Threads) k_readout_fd4_kick(
   if (i < hi) load(i, cu, cp, cid);
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
+  if constexpr (NODES) {
+    for (int c = t; c < kNodes * kNodes * kNodes; c += NT) {
+      const int x = c / (kNodes * kNodes), r = c - x * (kNodes * kNodes), y = r / kNodes, z = r - y * kNodes;
+      const float* const q = sp + (x + 2) * kFd4SX + (y + 2) * kFd4SY + (z + 4);
+      auto st = [q](int S) { return 8.0f * (q[S] - q[-S]) - (q[2 * S] - q[-2 * S]); };
+      nodes[3 * c] = -inv12h * st(kFd4SX);
+      nodes[3 * c + 1] = -inv12h * st(kFd4SY);
+      nodes[3 * c + 2] = -inv12h * st(1);
+    }
+    __syncthreads();
+  }
   const float fscale = 1.0f / (float)(1u << shift);
   const uint32_t fmask = (1u << shift) - 1u;
   bool bad = false, nonfinite = false;
-  for (; i < hi; i += kFd4Threads) {
-    const uint32_t inext = i + kFd4Threads;
+  for (; i < hi; i += NT) {
+    const uint32_t inext = i + NT;
     uint32_t nu[3] = {0u, 0u, 0u}, nid = 0u;
     float np[3] = {0.f, 0.f, 0.f};
     if (inext < hi) load(inext, nu, np, nid);
@@ -585,25 +623,39 @@ __global__ void __launch_bounds__(kFd4Threads) k_readout_fd4_kick(
       const float fx = (float)(ux & fmask) * fscale, fy = (float)(uy & fmask) * fscale,
                   fz = (float)(uz & fmask) * fscale;
       const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
-      const float* q = sp + (lx + 2) * kFd4SX + (ly + 2) * kFd4SY + (lz + 4);  // phi at the particle's cell
-      // stencil sum of one axis at the two corners 0 (weight g) and 1 (weight f) of a
-      // line through q0 with stride S: g (8 (p1 - m1) - (p2 - m2)) + f (8 (p2 - p0) - (p3 - m1))
-      auto axis_sum = [](const float* q0, int S, float g, float f) {
-        const float m2 = q0[-2 * S], m1 = q0[-S], p0 = q0[0], p1 = q0[S], p2 = q0[2 * S], p3 = q0[3 * S];
-        return g * (8.0f * (p1 - m1) - (p2 - m2)) + f * (8.0f * (p2 - p0) - (p3 - m1));
-      };
-      float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f;
+      float F[3];
+      if constexpr (NODES) {
+        const float* const q = nodes + 3 * ((lx * kNodes + ly) * kNodes + lz);
+        constexpr int Y = 3 * kNodes, X = 3 * kNodes * kNodes;
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          // x lines at (y, z) = (b, a); y lines at (x, z) = (b, a); z lines at (x, y) = (b, a)
-          Fx = fmaf((b ? fy : gy) * (a ? fz : gz), axis_sum(q + b * kFd4SY + a, kFd4SX, gx, fx), Fx);
-          Fy = fmaf((b ? fx : gx) * (a ? fz : gz), axis_sum(q + b * kFd4SX + a, kFd4SY, gy, fy), Fy);
-          Fz = fmaf((b ? fx : gx) * (a ? fy : gy), axis_sum(q + b * kFd4SX + a * kFd4SY, 1, gz, fz), Fz);
+        for (int d = 0; d < 3; ++d) {
+          const float* const v = q + d;
+          F[d] = gx * (gy * (gz * v[0] + fz * v[3]) + fy * (gz * v[Y] + fz * v[Y + 3])) +
+                 fx * (gy * (gz * v[X] + fz * v[X + 3]) + fy * (gz * v[X + Y] + fz * v[X + Y + 3]));
         }
+      } else {
+        const float* q = sp + (lx + 2) * kFd4SX + (ly + 2) * kFd4SY + (lz + 4);  // phi at the particle's cell
+        // stencil sum of one axis at the two corners 0 (weight g) and 1 (weight f) of a
+        // line through q0 with stride S: g (8 (p1 - m1) - (p2 - m2)) + f (8 (p2 - p0) - (p3 - m1))
+        auto axis_sum = [](const float* q0, int S, float g, float f) {
+          const float m2 = q0[-2 * S], m1 = q0[-S], p0 = q0[0], p1 = q0[S], p2 = q0[2 * S], p3 = q0[3 * S];
+          return g * (8.0f * (p1 - m1) - (p2 - m2)) + f * (8.0f * (p2 - p0) - (p3 - m1));
+        };
+        float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+#pragma unroll
+          for (int b = 0; b < 2; ++b) {
+            // x lines at (y, z) = (b, a); y lines at (x, z) = (b, a); z lines at (x, y) = (b, a)
+            Fx = fmaf((b ? fy : gy) * (a ? fz : gz), axis_sum(q + b * kFd4SY + a, kFd4SX, gx, fx), Fx);
+            Fy = fmaf((b ? fx : gx) * (a ? fz : gz), axis_sum(q + b * kFd4SX + a, kFd4SY, gy, fy), Fy);
+            Fz = fmaf((b ? fx : gx) * (a ? fy : gy), axis_sum(q + b * kFd4SX + a * kFd4SY, 1, gz, fz), Fz);
+          }
+        }
+        F[0] = -inv12h * Fx;
+        F[1] = -inv12h * Fy;
+        F[2] = -inv12h * Fz;
       }
-      const float F[3] = {-inv12h * Fx, -inv12h * Fy, -inv12h * Fz};
       // a NaN or infinity in the force or the incoming momentum poisons the sum
       if (!isfinite(F[0] + F[1] + F[2] + cp[0] + cp[1] + cp[2])) nonfinite = true;
       if (perm) {  // force in the caller's order
@@ -655,65 +707,30 @@ __global__ void k_kick_drift_keys(uint32_t* __restrict__ u, float* __restrict__ 
                                   uint32_t* __restrict__ cnt3, long long nb1, const uint32_t* __restrict__ bprev,
                                   uint32_t* __restrict__ low, uint32_t* __restrict__ flags, int* __restrict__ err) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool ok = i < n;
-  uint32_t key = 0xffffffffu, cat = 0xffffffffu, ko = 0xffffffffu;
-  uint32_t flag = 0u;
-  if (ok) {
-    uint32_t uu[3], u0[3];
-    float chk = 0.0f;  // a NaN or infinity in p or f poisons the sum
+  const unsigned act = __ballot_sync(0xffffffffu, i < n);
+  if (i >= n) return;
+  uint32_t uu[3], u0[3];
+  float chk = 0.0f;  // a NaN or infinity in p or f poisons the sum
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const float pv = __fmaf_rn(K1, f[d * n + i], p[d * n + i]);
-      chk += pv;
-      p[d * n + i] = pv;
-      // u += rne(Delta p 2^32 / L), modulo 2^32; the 32-bit conversion (same rounding)
-      // whenever the step fits, the 64-bit one (FP64 pipe) only for steps of 2^31 or more
-      u0[d] = u[d * n + i];
-      uu[d] = drift_fixed(u0[d], dscale, pv);
-      u[d * n + i] = uu[d];
-    }
-    key = tile_key(uu[0], uu[1], uu[2], shift, ntl);
-    keys[i] = key;
-    if (!isfinite(chk)) atomicOr(err, 4);
-    if constexpr (RESORT) {
-      const uint32_t k0 = tile_key(u0[0], u0[1], u0[2], shift, ntl);
-      const bool in_range = (uint32_t)i >= bprev[k0] && (uint32_t)i < bprev[k0 + 1];
-      if (!in_range) {
-        flag = 1u;
-      } else if (k0 == key) {
-        cat = key << 1;  // stayer
-      } else {
-        ko = k0;
-        if (k0 < key) cat = (key << 1) | 1u;  // mover from a lower key
-      }
-    }
+  for (int d = 0; d < 3; ++d) {
+    const float pv = __fmaf_rn(K1, f[d * n + i], p[d * n + i]);
+    chk += pv;
+    p[d * n + i] = pv;
+    // u += rne(Delta p 2^32 / L), modulo 2^32; the 32-bit conversion (same rounding)
+    // whenever the step fits, the 64-bit one (FP64 pipe) only for steps of 2^31 or more
+    u0[d] = u[d * n + i];
+    uu[d] = drift_fixed(u0[d], dscale, pv);
+    u[d * n + i] = uu[d];
   }
+  const uint32_t key = tile_key(uu[0], uu[1], uu[2], shift, ntl);
+  keys[i] = key;
+  if (!isfinite(chk)) atomicOr(err, 4);
   if constexpr (RESORT) {
-    const int lane = threadIdx.x & 31;
-    const unsigned act = __ballot_sync(0xffffffffu, ok);
-    if (ok) {
-      const unsigned peers = __match_any_sync(act, key);
-      if (lane == __ffs(peers) - 1) atomicAdd(cnt3 + key, (uint32_t)__popc(peers));
-    }
-    const unsigned has = __ballot_sync(0xffffffffu, cat != 0xffffffffu);
-    if (cat != 0xffffffffu) {
-      const unsigned peers = __match_any_sync(has, cat);
-      if (lane == __ffs(peers) - 1) {
-        if (cat & 1u)
-          atomicAdd(low + (cat >> 1), (uint32_t)__popc(peers));
-        else
-          atomicAdd(cnt3 + nb1 + (cat >> 1), (uint32_t)__popc(peers));
-      }
-    }
-    const unsigned hasm = __ballot_sync(0xffffffffu, ko != 0xffffffffu);
-    if (ko != 0xffffffffu) {
-      const unsigned peers = __match_any_sync(hasm, ko);
-      if (lane == __ffs(peers) - 1) atomicAdd(cnt3 + 2 * nb1 + ko, (uint32_t)__popc(peers));
-    }
-    unsigned fl = flag;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) fl |= __shfl_xor_sync(0xffffffffu, fl, o);
-    if (fl && lane == 0) atomicOr(flags, fl);
+    const uint32_t k0 = tile_key(u0[0], u0[1], u0[2], shift, ntl);
+    const bool in = (uint32_t)i >= bprev[k0] && (uint32_t)i < bprev[k0 + 1];
+    count_resort(act, key, k0, in, cnt3, nb1, low);
+    const unsigned out = __ballot_sync(act, !in);
+    if (out && (int)(threadIdx.x & 31) == __ffs(out) - 1) atomicOr(flags, 1u);
   }
 }
 
@@ -787,15 +804,21 @@ void readout_fd4_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint
   LaunchScope L(c, s, K_READOUT_FD4_KICK);
   const float inv12h = (float)((double)c->g.n / (12.0 * c->cfg.box));
   const unsigned grid = (unsigned)(c->nt * c->nt * c->nt);
-  if (dn)
-    k_readout_fd4_kick<true><<<grid, kFd4Threads, 0, s>>>(us, ps, ids, n, c->bstart, phi, c->g.n, 32 - c->g.logn,
-                                                          c->ntl, row_pitch, inv12h, K, p_out, f_out, u_out,
-                                                          id_out, nullptr, c->err_dev, *dn);
-  else
-    k_readout_fd4_kick<false><<<grid, kFd4Threads, 0, s>>>(us, ps, ids, n, c->bstart, phi, c->g.n,
-                                                           32 - c->g.logn, c->ntl, row_pitch, inv12h, K, p_out,
-                                                           f_out, u_out, id_out, perm_scatter, c->err_dev,
-                                                           DriftNext{});
+  // Forces at the nodes first where tiles are full: see the kernel for both sides.  Meshes below
+  // 256^3 keep the gathering form, and with it their bits.
+  const bool nodes = c->g.n >= 256 && n >= (int64_t)kNodesMin * grid;
+  auto kern = dn ? (nodes ? k_readout_fd4_kick<true, true> : k_readout_fd4_kick<true, false>)
+                 : (nodes ? k_readout_fd4_kick<false, true> : k_readout_fd4_kick<false, false>);
+  const size_t smem = nodes ? kNodeSmem : kFd4Smem;
+  static bool attr[2][2] = {};
+  if (!attr[dn != nullptr][nodes]) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    attr[dn != nullptr][nodes] = true;
+  }
+  kern<<<grid, nodes ? kNodeThreads : kFd4Threads, smem, s>>>(us, ps, ids, n, c->bstart, phi, c->g.n, 32 - c->g.logn,
+                                                             c->ntl, row_pitch, inv12h, K, p_out, f_out, u_out, id_out,
+                                                             dn ? nullptr : perm_scatter, c->err_dev,
+                                                             dn ? *dn : DriftNext{});
 }
 
 void kick_drift_keys(pm_ctx* c, uint32_t* u, float* p, const float* f, int64_t n, float K1,
