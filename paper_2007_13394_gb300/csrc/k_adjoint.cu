@@ -124,7 +124,6 @@ __global__ void k_adj_combine(const float2* __restrict__ a, float2* __restrict__
 // the 4-point stencil along axis j (transfer function i D(k_j)), so
 //   term 1: sum_j lambda_j grad R[F_j] from the potential staged per tile, and
 //   term 2: B = G * (sum_j S_j paint(lambda_j)) (IFFT[g sum_j i D(k_j) FFT(paint_j)]).
-constexpr int kVjpThreads = 256;
 constexpr int kVjpSpanXY = kTile + 5;  // cells -2 .. 18 along x and y
 constexpr int kVjpSpanZ = kTile + 8;   // cells -4 .. 19 along z (16-byte aligned rows)
 constexpr int kVjpChunksZ = kVjpSpanZ / 4;
@@ -150,7 +149,8 @@ constexpr int kVjpStageB = kVjpSpanB * kVjpSpanB * (kVjpSpanBZ / 4);
 constexpr int kVjpBSY = kVjpSpanBZ, kVjpBSX = kVjpSpanB * kVjpSpanBZ;
 constexpr size_t kVjpSmem = sizeof(float) * (kVjpSpanXY * kVjpSX + kVjpSpanB * kVjpBSX);
 
-__global__ void __launch_bounds__(kVjpThreads) k_force_vjp_readout(
+template <int NT>
+__global__ void __launch_bounds__(NT) k_force_vjp_readout(
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n, const uint32_t* __restrict__ bstart,
     const float* __restrict__ phi, const float* __restrict__ B, int nm, int shift, int ntl, int row_pitch,
     float inv12h, float inv_h, const float* __restrict__ lam, MassTable mt, const uint32_t* __restrict__ perm,
@@ -165,13 +165,13 @@ __global__ void __launch_bounds__(kVjpThreads) k_force_vjp_readout(
   const int ox = (int)(tile >> (2 * ntl)) * kTile, oy = (int)((tile >> ntl) & (nt - 1)) * kTile,
             oz = (int)(tile & (nt - 1)) * kTile;
   const int wrap = nm - 1;
-  for (int c = t; c < kVjpStage; c += kVjpThreads) {
+  for (int c = t; c < kVjpStage; c += NT) {
     const int x = c / (kVjpSpanXY * kVjpChunksZ), r = c - x * (kVjpSpanXY * kVjpChunksZ);
     const int y = r / kVjpChunksZ, k = r - y * kVjpChunksZ;
     const int gx = (ox + x - 2) & wrap, gy = (oy + y - 2) & wrap, gz = (oz - 4 + 4 * k) & wrap;
     vjp_cp_async16(sp + x * kVjpSX + y * kVjpSY + 4 * k, phi + ((size_t)gx * nm + gy) * (size_t)row_pitch + gz);
   }
-  for (int c = t; c < kVjpStageB; c += kVjpThreads) {
+  for (int c = t; c < kVjpStageB; c += NT) {
     const int x = c / (kVjpSpanB * (kVjpSpanBZ / 4)), r = c - x * (kVjpSpanB * (kVjpSpanBZ / 4));
     const int y = r / (kVjpSpanBZ / 4), k = r - y * (kVjpSpanBZ / 4);
     const int gx = (ox + x) & wrap, gy = (oy + y) & wrap, gz = (oz + 4 * k) & wrap;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kVjpThreads) k_force_vjp_readout(
   const float fscale = 1.0f / (float)(1u << shift);
   const uint32_t fmask = (1u << shift) - 1u;
   bool bad = false;
-  for (uint32_t i = lo + t; i < hi; i += kVjpThreads) {
+  for (uint32_t i = lo + t; i < hi; i += NT) {
     const uint32_t ux = us[i], uy = us[n + i], uz = us[2 * n + i];
     const int lx = (int)(ux >> shift) - ox, ly = (int)(uy >> shift) - oy, lz = (int)(uz >> shift) - oz;
     if ((unsigned)lx >= (unsigned)kTile || (unsigned)ly >= (unsigned)kTile || (unsigned)lz >= (unsigned)kTile) {
@@ -252,8 +252,8 @@ __global__ void __launch_bounds__(kVjpThreads) k_force_vjp_readout(
 // One mesh's or three meshes' worth of the VJP, staged per tile like B above (the learned path):
 // NM = 1: tmp[d][i] = m_i d/dx_d R[B](x_i) in sorted order; NM = 3: out[d][perm[i]] = tmp[d][i] +
 // sum_j lambda_j(i) d/dx_d R[F_j](x_i).  Staging replaces 8 NM scattered global reads a particle.
-template <int NM>
-__global__ void __launch_bounds__(kVjpThreads) k_vjp_readout(
+template <int NM, int NT>
+__global__ void __launch_bounds__(NT) k_vjp_readout(
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n, const uint32_t* __restrict__ bstart,
     const float* __restrict__ m0, const float* __restrict__ m1, const float* __restrict__ m2, int nm, int shift,
     int ntl, int row_pitch, float inv_h, const float* __restrict__ lam, MassTable mt,
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kVjpThreads) k_vjp_readout(
   for (int j = 0; j < NM; ++j) {
     const float* const M = j == 0 ? m0 : (j == 1 ? m1 : m2);
     float* const dst = sb + j * kVjpSpanB * kVjpBSX;
-    for (int c = t; c < kVjpStageB; c += kVjpThreads) {
+    for (int c = t; c < kVjpStageB; c += NT) {
       const int x = c / (kVjpSpanB * (kVjpSpanBZ / 4)), r = c - x * (kVjpSpanB * (kVjpSpanBZ / 4));
       const int y = r / (kVjpSpanBZ / 4), k = r - y * (kVjpSpanBZ / 4);
       const int gx = (ox + x) & wrap, gy = (oy + y) & wrap, gz = (oz + 4 * k) & wrap;
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(kVjpThreads) k_vjp_readout(
   const float fscale = 1.0f / (float)(1u << shift);
   const uint32_t fmask = (1u << shift) - 1u;
   bool bad = false;
-  for (uint32_t i = lo + t; i < hi; i += kVjpThreads) {
+  for (uint32_t i = lo + t; i < hi; i += NT) {
     const uint32_t ux = us[i], uy = us[n + i], uz = us[2 * n + i];
     const int lx = (int)(ux >> shift) - ox, ly = (int)(uy >> shift) - oy, lz = (int)(uz >> shift) - oz;
     if ((unsigned)lx >= (unsigned)kTile || (unsigned)ly >= (unsigned)kTile || (unsigned)lz >= (unsigned)kTile) {
@@ -651,18 +651,20 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
       }
       fft_inverse_plain(c, c->g, pot, s);  // B
       const size_t sm1 = sizeof(float) * kVjpSpanB * kVjpBSX;
-      static bool attr3 = false;
-      if (!attr3) {
-        cudaFuncSetAttribute(k_vjp_readout<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(3 * sm1));
-        attr3 = true;
+      const int threads = std::min(tile_threads(c), 512);
+      auto read1 = threads == 512 ? k_vjp_readout<1, 512> : k_vjp_readout<1, 256>;
+      auto read3 = threads == 512 ? k_vjp_readout<3, 512> : k_vjp_readout<3, 256>;
+      static bool attr3[2] = {false, false};
+      if (!attr3[threads == 512]) {
+        cudaFuncSetAttribute(read3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(3 * sm1));
+        attr3[threads == 512] = true;
       }
       const unsigned tiles = (unsigned)(c->nt * c->nt * c->nt);
       float* const tmp = c->adj + 7 * 3 * n;  // the second term, sorted order
       {
         LaunchScope L(c, s, K_ADJOINT);
-        k_vjp_readout<1><<<tiles, kVjpThreads, sm1, s>>>(c->us, c->ids, n, c->bstart, realP, nullptr, nullptr, c->g.n,
-                                                        32 - c->g.logn, c->ntl, rp, inv_h, nullptr, c->mt, nullptr, tmp,
-                                                        nullptr, c->err_dev);
+        read1<<<tiles, threads, sm1, s>>>(c->us, c->ids, n, c->bstart, realP, nullptr, nullptr, c->g.n, 32 - c->g.logn,
+                                          c->ntl, rp, inv_h, nullptr, c->mt, nullptr, tmp, nullptr, c->err_dev);
       }
       // F_y, F_z into the other meshes, F_x in place over phi_k
       fft_inverse_component(c, c->g, c->meshA, c->meshB, 1, s);
@@ -670,23 +672,24 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
       fft_inverse_component(c, c->g, c->meshA, c->meshA, 0, s);
       {
         LaunchScope L(c, s, K_ADJOINT);
-        k_vjp_readout<3><<<tiles, kVjpThreads, 3 * sm1, s>>>(c->us, c->ids, n, c->bstart, realA, realB, realP, c->g.n,
-                                                            32 - c->g.logn, c->ntl, rp, inv_h, lam_s, c->mt,
-                                                            c->vals[0], tmp, grad, c->err_dev);
+        read3<<<tiles, threads, 3 * sm1, s>>>(c->us, c->ids, n, c->bstart, realA, realB, realP, c->g.n, 32 - c->g.logn,
+                                              c->ntl, rp, inv_h, lam_s, c->mt, c->vals[0], tmp, grad, c->err_dev);
       }
       mlp_backward(c, a, s);
       return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ECUDA;
     }
     fft_potential(c, c->g, c->meshA, s);
     fft_potential(c, c->g, pot, s);
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_force_vjp_readout, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVjpSmem);
-      attr = true;
+    const int threads = std::min(tile_threads(c), 512);
+    auto kern = threads == 512 ? k_force_vjp_readout<512> : k_force_vjp_readout<256>;
+    static bool attr[2] = {false, false};
+    if (!attr[threads == 512]) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVjpSmem);
+      attr[threads == 512] = true;
     }
     {
       LaunchScope L(c, s, K_ADJOINT);
-      k_force_vjp_readout<<<(unsigned)(c->nt * c->nt * c->nt), kVjpThreads, kVjpSmem, s>>>(
+      kern<<<(unsigned)(c->nt * c->nt * c->nt), threads, kVjpSmem, s>>>(
           c->us, c->ids, n, c->bstart, realA, realP, c->g.n, 32 - c->g.logn, c->ntl, rp, inv12h, inv_h, lam_s, c->mt,
           c->vals[0], grad, c->err_dev);
     }

@@ -92,6 +92,7 @@ __device__ __forceinline__ float float64w(unsigned int hi, unsigned int lo) {
 // A tile whose list of wraps overflowed, painted again by its CTA: half of its x planes at a
 // time in two words a cell, which fit where the low words of the whole tile were.  Out of line:
 // rare, and the main form keeps its 32 registers.  Every thread of the CTA calls it.
+template <int NT>
 __device__ __noinline__ void paint_halves(uint32_t tile, unsigned int* __restrict__ accw,
                                           const uint32_t* __restrict__ run_lo, const uint32_t* __restrict__ run_pre,
                                           const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
@@ -105,10 +106,10 @@ __device__ __noinline__ void paint_halves(uint32_t tile, unsigned int* __restric
   const uint32_t fmask = (1u << shift) - 1u, total = run_pre[14];
   for (int x0 = 0; x0 < kTile; x0 += HX) {
     __syncthreads();  // the accumulators are free
-    for (int i = t; i < 2 * WORDS; i += kPaintThreads) accw[i] = 0;
+    for (int i = t; i < 2 * WORDS; i += NT) accw[i] = 0;
     __syncthreads();
     int r = 0;
-    for (uint32_t v = t; v < total; v += kPaintThreads) {
+    for (uint32_t v = t; v < total; v += NT) {
       while (v >= run_pre[r + 1]) ++r;
       const uint32_t k = run_lo[r] + (v - run_pre[r]);
       const uint32_t q[3] = {us[k], us[n + k], us[2 * n + k]};
@@ -135,7 +136,7 @@ __device__ __noinline__ void paint_halves(uint32_t tile, unsigned int* __restric
       }
     }
     __syncthreads();
-    for (int q = t; q < HX * kTile * kTile; q += kPaintThreads) {
+    for (int q = t; q < HX * kTile * kTile; q += NT) {
       const int x = q / (kTile * kTile), y = (q / kTile) % kTile, z = q % kTile;
       const int a = x * kSx + y * kSy + z;
       mesh[((size_t)(ox + x0 + x) * nm + (oy + y)) * (size_t)row_pitch + oz + z] = float64w(accw[WORDS + a], accw[a]) * kUnfixM;
@@ -274,7 +275,7 @@ __device__ __forceinline__ void paint_tile(
   if constexpr (FAST) {
     // the barrier's vote tells every thread whether the event list overflowed
     if (__syncthreads_or(wrap ? 1 : 0)) {
-      paint_halves(tile, accw, run_lo, run_pre, us, ids, n, mesh, mt, species, nm, shift, ntl, row_pitch);
+      paint_halves<NT>(tile, accw, run_lo, run_pre, us, ids, n, mesh, mt, species, nm, shift, ntl, row_pitch);
       return;
     }
   } else {
@@ -318,14 +319,14 @@ __device__ __forceinline__ void paint_tile(
 
 // One CTA per tile.  FAST: the 32-bit form with wrap events (masses below 128); else the
 // two-word form, with NW signed weights instead of masses when NW > 0.
-template <bool FAST, int NW>
-__global__ void __launch_bounds__(kPaintThreads, FAST ? 8 : 1) k_paint_tiles(
+template <bool FAST, int NW, int NT>
+__global__ void __launch_bounds__(NT, FAST ? 2048 / NT : 1) k_paint_tiles(
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
     const uint32_t* __restrict__ bstart, float* __restrict__ mesh, const __grid_constant__ MassTable mt, int species,
     int nm, int shift, int ntl, int row_pitch, int* __restrict__ err, const float* __restrict__ wts) {
   __shared__ __align__(16) unsigned int accw[FAST ? kFastWords : 2 * kAccWords];
   __shared__ uint32_t run_lo[14], run_pre[15];
-  paint_tile<FAST, NW, kPaintThreads>(blockIdx.x, accw, run_lo, run_pre, us, ids, n, bstart, mesh, mt, species, nm,
+  paint_tile<FAST, NW, NT>(blockIdx.x, accw, run_lo, run_pre, us, ids, n, bstart, mesh, mt, species, nm,
                                       shift, ntl, row_pitch, err, wts);
 }
 
@@ -522,7 +523,6 @@ __device__ __forceinline__ void drift_next(const DriftNext& dn, const float (&F)
   count_resort(__activemask(), kn, ko, true, dn.cnt3, dn.nb1, dn.low);
 }
 
-constexpr int kFd4Threads = 256;
 constexpr int kSpanXY = kTile + 5;                 // cells -2 .. 18 along x and y
 constexpr int kSpanZ = kTile + 8;                  // cells -4 .. 19 along z
 constexpr int kChunksZ = kSpanZ / 4;               // 16-byte chunks per staged z row
@@ -564,14 +564,13 @@ __device__ __forceinline__ void stage_potential(float* sp, const float* __restri
 // 162 / 157, 2000 211 / 184, 4000 411 / 292, 8000 806 / 494.
 // The gathering form runs five CTAs an SM (48 registers; at 60 to 104 it holds four to two: 4.65
 // to 6.2 ms against 4.1 on the late steps of 152 M particles at 1024^3).
-template <bool DRIFT, bool NODES>
-__global__ void __launch_bounds__(NODES ? kNodeThreads : kFd4Threads, NODES ? 2 : 5) k_readout_fd4_kick(
+template <bool DRIFT, bool NODES, int NT>
+__global__ void __launch_bounds__(NT, NODES ? 2 : (NT == 256 ? 5 : 1024 / NT)) k_readout_fd4_kick(
     const uint32_t* __restrict__ us, const float* __restrict__ ps, const uint32_t* __restrict__ ids,
     int64_t n, const uint32_t* __restrict__ bstart, const float* __restrict__ phi, int nm, int shift,
     int ntl, int row_pitch, float inv12h, float K, float* __restrict__ p_out, float* __restrict__ f_out,
     uint32_t* __restrict__ u_out, uint32_t* __restrict__ id_out, const uint32_t* __restrict__ perm,
     int* __restrict__ err, DriftNext dn) {
-  constexpr int NT = NODES ? kNodeThreads : kFd4Threads;
   extern __shared__ __align__(16) float sp[];  // the potential, then (NODES) the nodes' forces
   float* const nodes = sp + kSpanXY * kFd4SX;
   const int t = threadIdx.x;
@@ -757,8 +756,17 @@ void paint_tiles(pm_ctx* c, const uint32_t* us, const uint32_t* ids, int64_t n, 
     for (int i = 0; i < c->mt.nshell && i < kMaxShell; ++i) mmax = std::max(mmax, c->mt.m_nu[i]);
   LaunchScope L(c, s, K_PAINT);
   // masses below 128: w 2^24 < 2^31, so every contribution fits the 32-bit form
-  auto kern = weights ? k_paint_tiles<false, 1> : (mmax < 128.0f ? k_paint_tiles<true, 0> : k_paint_tiles<false, 0>);
-  kern<<<grid, kPaintThreads, 0, s>>>(us, ids, n, c->bstart, mesh, c->mt, species, c->g.n, 32 - c->g.logn, c->ntl,
+  int threads = kPaintThreads;
+  auto kern = k_paint_tiles<false, 1, kPaintThreads>;
+  if (!weights) {
+    kern = k_paint_tiles<false, 0, kPaintThreads>;
+    if (mmax < 128.0f) {
+      threads = tile_threads(c);
+      kern = threads == 1024 ? k_paint_tiles<true, 0, 1024>
+                             : (threads == 512 ? k_paint_tiles<true, 0, 512> : k_paint_tiles<true, 0, 256>);
+    }
+  }
+  kern<<<grid, threads, 0, s>>>(us, ids, n, c->bstart, mesh, c->mt, species, c->g.n, 32 - c->g.logn, c->ntl,
                                       row_pitch, c->err_dev, weights);
 }
 
@@ -807,15 +815,22 @@ void readout_fd4_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint
   // Forces at the nodes first where tiles are full: see the kernel for both sides.  Meshes below
   // 256^3 keep the gathering form, and with it their bits.
   const bool nodes = c->g.n >= 256 && n >= (int64_t)kNodesMin * grid;
-  auto kern = dn ? (nodes ? k_readout_fd4_kick<true, true> : k_readout_fd4_kick<true, false>)
-                 : (nodes ? k_readout_fd4_kick<false, true> : k_readout_fd4_kick<false, false>);
+  const bool few = !nodes && tile_threads(c) == 1024;  // (at 128^3 five CTAs of 256 hold more warps than two of 512)
+  const int threads = nodes ? kNodeThreads : (few ? 1024 : 256);
+  const int v = nodes ? 2 : (few ? 1 : 0);
+  decltype(&k_readout_fd4_kick<false, false, 256>) const kerns[2][3] = {
+      {k_readout_fd4_kick<false, false, 256>, k_readout_fd4_kick<false, false, 1024>,
+       k_readout_fd4_kick<false, true, kNodeThreads>},
+      {k_readout_fd4_kick<true, false, 256>, k_readout_fd4_kick<true, false, 1024>,
+       k_readout_fd4_kick<true, true, kNodeThreads>}};
+  const auto kern = kerns[dn != nullptr][v];
   const size_t smem = nodes ? kNodeSmem : kFd4Smem;
-  static bool attr[2][2] = {};
-  if (!attr[dn != nullptr][nodes]) {
+  static bool attr[2][3] = {};
+  if (!attr[dn != nullptr][v]) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr[dn != nullptr][nodes] = true;
+    attr[dn != nullptr][v] = true;
   }
-  kern<<<grid, nodes ? kNodeThreads : kFd4Threads, smem, s>>>(us, ps, ids, n, c->bstart, phi, c->g.n, 32 - c->g.logn,
+  kern<<<grid, threads, smem, s>>>(us, ps, ids, n, c->bstart, phi, c->g.n, 32 - c->g.logn,
                                                              c->ntl, row_pitch, inv12h, K, p_out, f_out, u_out, id_out,
                                                              dn ? nullptr : perm_scatter, c->err_dev,
                                                              dn ? *dn : DriftNext{});

@@ -516,22 +516,21 @@ __device__ __forceinline__ void copy_particle(const uint32_t* __restrict__ u, co
 // key's slot of the mover list, mstart3[ko] - base3 + mrank (movers in index order).  With
 // flag bit 1 every particle is a mover at its own index.  stage_room: the movers' records
 // that the staging area holds (more movers: none is staged).
-constexpr int kResortThreads = 256;
-
-__global__ void __launch_bounds__(kResortThreads) k_resort_old_tiles(
+template <int NT>
+__global__ void __launch_bounds__(NT) k_resort_old_tiles(
     const uint32_t* __restrict__ u, const float* __restrict__ p, const uint32_t* __restrict__ id, int64_t n,
     const uint32_t* __restrict__ keys, const uint32_t* __restrict__ bprev, const uint32_t* __restrict__ bstart3,
     long long nb1, const uint32_t* __restrict__ low, uint32_t* __restrict__ us, float* __restrict__ ps,
     uint32_t* __restrict__ ids, uint32_t* __restrict__ mk, uint32_t* __restrict__ mv,
     const uint32_t* __restrict__ flags, int* __restrict__ err, uint4* __restrict__ stage, int64_t stage_room) {
-  constexpr int W = kResortThreads / 32;
+  constexpr int W = NT / 32;
   __shared__ uint32_t cls_lo[9];   // bprev[8 O + c]
   __shared__ uint32_t cls_m0[8];   // movers of the tile before class c's first particle
   __shared__ uint32_t wsum[W];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const uint32_t O = blockIdx.x;
   if (*flags & 1u) {
-    for (int64_t i = (int64_t)O * kResortThreads + t; i < n; i += (int64_t)gridDim.x * kResortThreads) {
+    for (int64_t i = (int64_t)O * NT + t; i < n; i += (int64_t)gridDim.x * NT) {
       mk[i] = keys[i];
       mv[i] = (uint32_t)i;
     }
@@ -546,7 +545,7 @@ __global__ void __launch_bounds__(kResortThreads) k_resort_old_tiles(
   const uint32_t base3 = bstart3[2 * nb1];  // n + all stayers: offset of the third scan
   const unsigned lt = (1u << lane) - 1u;
   uint32_t run = 0;  // movers of the tile before this chunk
-  for (uint32_t chunk = lo; chunk < hi; chunk += kResortThreads) {
+  for (uint32_t chunk = lo; chunk < hi; chunk += NT) {
     const uint32_t i = chunk + t;
     const bool ok = i < hi;
     uint32_t kn = 0, c = 0;
@@ -807,7 +806,9 @@ int resort_near_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint3
   const int64_t room = (int64_t)(c->g.elems() * sizeof(float2) / 32);
   {
     LaunchScope L(c, s, K_RESORT_PLACE);
-    k_resort_old_tiles<<<(unsigned)((long long)c->nt * c->nt * c->nt), kResortThreads, 0, s>>>(
+    const int threads = tile_threads(c);
+    auto kern = threads == 1024 ? k_resort_old_tiles<1024> : (threads == 512 ? k_resort_old_tiles<512> : k_resort_old_tiles<256>);
+    kern<<<(unsigned)((long long)c->nt * c->nt * c->nt), threads, 0, s>>>(
         u, p, id, n, c->keys[0], c->bprev, c->bstart, nb1, c->rs_low, c->us, c->ps, c->ids, c->keys[1], c->vals[1],
         c->rs_dev, c->err_dev, stage, room);
   }
