@@ -38,6 +38,7 @@ __global__ void k_readout_grad(const uint32_t* __restrict__ us, const uint32_t* 
                                int row_pitch, float inv_h, const float* __restrict__ wts, MassTable mt,
                                const uint32_t* __restrict__ perm, float* __restrict__ out,
                                int accumulate, int species) {
+  pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t ux = us[i], uy = us[n + i], uz = us[2 * n + i];
@@ -93,6 +94,7 @@ __global__ void k_adj_combine(const float2* __restrict__ a, float2* __restrict__
                               const float* __restrict__ kvec0, float gcoef, int comp, int accumulate,
                               const float* __restrict__ mtab, const float2* __restrict__ rho,
                               double* __restrict__ gbin) {
+  pdl_begin();
   const int x = blockIdx.x / nm, y = blockIdx.x % nm;
   const int nx = x < nm / 2 ? x : x - nm, ny = y < nm / 2 ? y : y - nm;
   for (int kz = threadIdx.x; kz <= nm / 2; kz += blockDim.x) {
@@ -155,6 +157,7 @@ __global__ void __launch_bounds__(NT) k_force_vjp_readout(
     const float* __restrict__ phi, const float* __restrict__ B, int nm, int shift, int ntl, int row_pitch,
     float inv12h, float inv_h, const float* __restrict__ lam, MassTable mt, const uint32_t* __restrict__ perm,
     float* __restrict__ out, int* __restrict__ err) {
+  pdl_begin();
   extern __shared__ __align__(16) float sp[];
   float* const sb = sp + kVjpSpanXY * kVjpSX;
   const int t = threadIdx.x;
@@ -258,6 +261,7 @@ __global__ void __launch_bounds__(NT) k_vjp_readout(
     const float* __restrict__ m0, const float* __restrict__ m1, const float* __restrict__ m2, int nm, int shift,
     int ntl, int row_pitch, float inv_h, const float* __restrict__ lam, MassTable mt,
     const uint32_t* __restrict__ perm, float* __restrict__ tmp, float* __restrict__ out, int* __restrict__ err) {
+  pdl_begin();
   extern __shared__ __align__(16) float sb[];
   const int t = threadIdx.x;
   const uint32_t tile = blockIdx.x;
@@ -334,6 +338,7 @@ constexpr int kDivThreads = 256;
 constexpr int kDivSteps = 8;
 __global__ void __launch_bounds__(kDivThreads) k_stencil_div(const float* __restrict__ A, const float* __restrict__ B,
                                                              float* C, int nm, int rp, float inv12h) {
+  pdl_begin();
   const int quads = nm / 4, rows = kDivThreads / quads;  // rows of z quads a CTA (nm <= 1024)
   const int q = threadIdx.x % quads, z = 4 * q, w = nm - 1;
   const int y = (blockIdx.x % (nm / rows)) * rows + threadIdx.x / quads;
@@ -369,6 +374,7 @@ __global__ void __launch_bounds__(kDivThreads) k_stencil_div(const float* __rest
 __global__ void __launch_bounds__(256) k_spectrum_div(const float2* __restrict__ A, const float2* __restrict__ B,
                                                       float2* __restrict__ C, int nm, int pc,
                                                       const float* __restrict__ kvec0) {
+  pdl_begin();
   const long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);  // x N + y: a warp a row
   const float kx = __ldg(kvec0 + row / nm), ky = __ldg(kvec0 + row % nm);
   for (int kz = threadIdx.x & 31; kz <= nm / 2; kz += 32) {
@@ -389,6 +395,7 @@ __global__ void __launch_bounds__(256) k_vjp_combine(float2* __restrict__ rho, f
                                                      int units, const float* __restrict__ ksq,
                                                      const float* __restrict__ winv, float gcoef,
                                                      const float* __restrict__ mtab, double* __restrict__ gbin) {
+  pdl_begin();
   const int wu = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31, half = nm / 2;
   if (wu >= units) return;
   int a = (int)((sqrtf(8.0f * (float)wu + 1.0f) - 1.0f) * 0.5f);  // (a, b), 0 <= b <= a <= N/2
@@ -424,6 +431,7 @@ __global__ void __launch_bounds__(256) k_vjp_combine(float2* __restrict__ rho, f
 // B (+)= S_j A on real meshes (row pitch rp): the 4-point stencil along axis j, periodic.
 __global__ void k_stencil_axis(const float* __restrict__ A, float* __restrict__ B, int nm, int rp, int axis,
                                float inv12h, int accumulate) {
+  pdl_begin();
   const int x = blockIdx.x / nm, y = blockIdx.x % nm;
   const int w = nm - 1;
   const size_t row = ((size_t)x * nm + y) * rp;
@@ -445,6 +453,7 @@ __global__ void k_vjp_begin(const float* __restrict__ lx1, const float* __restri
                             const float* __restrict__ p0, const float* __restrict__ f0, int64_t n, float K1,
                             float dscale, float K2, float* __restrict__ Lx, float* __restrict__ Lp,
                             float* __restrict__ lamF, uint32_t* __restrict__ u1) {
+  pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t j = (int64_t)id[i];
@@ -462,6 +471,7 @@ __global__ void k_vjp_begin(const float* __restrict__ lx1, const float* __restri
 // Between the two force VJPs, over 3n: Lx += g, Lp += Delta Lx, lamF = K1 Lp.
 __global__ void k_vjp_middle(const float* __restrict__ g, int64_t m, float delta, float K1, float* __restrict__ Lx,
                              float* __restrict__ Lp, float* __restrict__ lamF) {
+  pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
   const float x = Lx[i] + g[i], p = fmaf(delta, x, Lp[i]);
@@ -474,6 +484,7 @@ __global__ void k_vjp_middle(const float* __restrict__ g, int64_t m, float delta
 __global__ void k_vjp_end(const float* __restrict__ g, const float* __restrict__ Lx, const float* __restrict__ Lp,
                           const uint32_t* __restrict__ id, int64_t n, float* __restrict__ lx0,
                           float* __restrict__ lp0) {
+  pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t j = (int64_t)id[i];
@@ -487,6 +498,7 @@ __global__ void k_vjp_end(const float* __restrict__ g, const float* __restrict__
 // gather per-component weights into the sorted order: ws[j][k] = w[j][perm[k]]
 __global__ void k_gather3(const float* __restrict__ w, const uint32_t* __restrict__ perm, int64_t n,
                           int ncomp, float* __restrict__ ws) {
+  pdl_begin();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const uint32_t i = perm[k];
@@ -497,6 +509,7 @@ __global__ void k_gather3(const float* __restrict__ w, const uint32_t* __restric
 __global__ void k_icadj_cdm(const float* __restrict__ lx, const float* __restrict__ lp, int nc,
                             int rp, int comp, float D0, float gp0, int64_t n_total,
                             float* __restrict__ mesh) {
+  pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t ncell = (int64_t)nc * nc * nc;
   if (i >= ncell) return;
@@ -509,6 +522,7 @@ __global__ void k_icadj_cdm(const float* __restrict__ lx, const float* __restric
 __global__ void k_icadj_nu(const float* __restrict__ lx, const float* __restrict__ lp, int nc,
                            int rp, int comp, float D0, float gp0, int nsites, int stride, int j0,
                            int per_site, int64_t n_offset, int64_t n_total, float* __restrict__ mesh) {
+  pdl_begin();
   const int64_t site = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nsite3 = (int64_t)nsites * nsites * nsites;
   if (site >= nsite3) return;
@@ -528,6 +542,7 @@ __global__ void k_icadj_nu(const float* __restrict__ lx, const float* __restrict
 __global__ void k_icadj_kspace(const float2* __restrict__ a, float2* __restrict__ kacc, int nc, int pc,
                                const float* __restrict__ amp, int comp, int phase_shift,
                                int accumulate) {
+  pdl_begin();
   const int x = blockIdx.x / nc, y = blockIdx.x % nc;
   const int nx = x < nc / 2 ? x : x - nc, ny = y < nc / 2 ? y : y - nc;
   for (int kz = threadIdx.x; kz <= nc / 2; kz += blockDim.x) {
@@ -572,7 +587,7 @@ unsigned blocks(int64_t n) { return (unsigned)((n + 255) / 256); }
 int gather_weights(pm_ctx* c, const float* w, int64_t n, float* w_sorted, cudaStream_t s) {
   if (n == 0) return PM_OK;
   LaunchScope L(c, s, K_ADJOINT);
-  k_gather3<<<blocks(n), 256, 0, s>>>(w, c->vals[0], n, 1, w_sorted);
+  pdl_launch(k_gather3, blocks(n), 256, 0, s, w, c->vals[0], n, 1, w_sorted);
   return PM_OK;
 }
 
@@ -583,7 +598,7 @@ void readout_grad(pm_ctx* c, int64_t n, const float* const* meshes, int nmeshes,
   if (n == 0) return;
   LaunchScope L(c, s, K_ADJOINT);
   const float inv_h = (float)(c->g.n / c->cfg.box);
-  k_readout_grad<<<blocks(n), 256, 0, s>>>(c->us, c->ids, n, meshes[0], nmeshes > 1 ? meshes[1] : nullptr,
+  pdl_launch(k_readout_grad, blocks(n), 256, 0, s, c->us, c->ids, n, meshes[0], nmeshes > 1 ? meshes[1] : nullptr,
                                            nmeshes > 2 ? meshes[2] : nullptr, nmeshes, c->g.n,
                                            32 - c->g.logn, row_pitch, inv_h, wts_sorted, c->mt, perm,
                                            out, accumulate ? 1 : 0, species);
@@ -605,7 +620,7 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
   float* lam_s = c->adj + 6 * 3 * n;  // sorted cotangent, 3n
   {
     LaunchScope L(c, s, K_ADJOINT);
-    k_gather3<<<blocks(n), 256, 0, s>>>(lam_f, c->vals[0], n, 3, lam_s);
+    pdl_launch(k_gather3, blocks(n), 256, 0, s, lam_f, c->vals[0], n, 3, lam_s);
   }
   float* realA = reinterpret_cast<float*>(c->meshA);
   float* realB = reinterpret_cast<float*>(c->meshB);
@@ -626,15 +641,15 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
       LaunchScope L(c, s, K_ADJOINT);
       const int rows = kDivThreads / (c->g.n / 4);
       if (learned)
-        k_spectrum_div<<<(unsigned)(c->g.rows() / 8), 256, 0, s>>>(c->meshA, c->meshB, pot, c->g.n, c->g.pc, c->kvec0);
+        pdl_launch(k_spectrum_div, (unsigned)(c->g.rows() / 8), 256, 0, s, c->meshA, c->meshB, pot, c->g.n, c->g.pc, c->kvec0);
       else
-        k_stencil_div<<<(unsigned)(c->g.n / rows * (c->g.n / kDivSteps)), kDivThreads, 0, s>>>(
+        pdl_launch(k_stencil_div, (unsigned)(c->g.n / rows * (c->g.n / kDivSteps)), kDivThreads, 0, s, 
             realA, realB, realP, c->g.n, rp, inv12h);
     } else {  // two meshes: one component at a time
       for (int j = 0; j < 3; ++j) {
         paint_tiles(c, c->us, c->ids, n, PM_SPECIES_ALL, realA, rp, s, lam_s + (int64_t)j * n);
         LaunchScope L(c, s, K_ADJOINT);
-        k_stencil_axis<<<(unsigned)(c->g.n * c->g.n), 256, 0, s>>>(realA, realP, c->g.n, rp, j, inv12h, j > 0);
+        pdl_launch(k_stencil_axis, (unsigned)(c->g.n * c->g.n), 256, 0, s, realA, realP, c->g.n, rp, j, inv12h, j > 0);
       }
     }
     paint_tiles(c, c->us, c->ids, n, PM_SPECIES_ALL, realA, rp, s);
@@ -645,7 +660,7 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
         LaunchScope L(c, s, K_ADJOINT);
         const double nn = (double)c->g.n;
         const int units = (c->g.n / 2 + 1) * (c->g.n / 2 + 2) / 2;
-        k_vjp_combine<<<(units + 7) / 8, 256, 0, s>>>(c->meshA, pot, c->g.n, c->g.pc, units, c->ksq, c->wforce,
+        pdl_launch(k_vjp_combine, (units + 7) / 8, 256, 0, s, c->meshA, pot, c->g.n, c->g.pc, units, c->ksq, c->wforce,
                                                       (float)(-1.5 * c->cosmo.omega_m0 / (nn * nn * nn)), c->mlp_tab,
                                                       c->mlp_gbin);
       }
@@ -663,7 +678,7 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
       float* const tmp = c->adj + 7 * 3 * n;  // the second term, sorted order
       {
         LaunchScope L(c, s, K_ADJOINT);
-        read1<<<tiles, threads, sm1, s>>>(c->us, c->ids, n, c->bstart, realP, nullptr, nullptr, c->g.n, 32 - c->g.logn,
+        pdl_launch(read1, tiles, threads, sm1, s, c->us, c->ids, n, c->bstart, realP, nullptr, nullptr, c->g.n, 32 - c->g.logn,
                                           c->ntl, rp, inv_h, nullptr, c->mt, nullptr, tmp, nullptr, c->err_dev);
       }
       // F_y, F_z into the other meshes, F_x in place over phi_k
@@ -672,7 +687,7 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
       fft_inverse_component(c, c->g, c->meshA, c->meshA, 0, s);
       {
         LaunchScope L(c, s, K_ADJOINT);
-        read3<<<tiles, threads, 3 * sm1, s>>>(c->us, c->ids, n, c->bstart, realA, realB, realP, c->g.n, 32 - c->g.logn,
+        pdl_launch(read3, tiles, threads, 3 * sm1, s, c->us, c->ids, n, c->bstart, realA, realB, realP, c->g.n, 32 - c->g.logn,
                                               c->ntl, rp, inv_h, lam_s, c->mt, c->vals[0], tmp, grad, c->err_dev);
       }
       mlp_backward(c, a, s);
@@ -689,7 +704,7 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
     }
     {
       LaunchScope L(c, s, K_ADJOINT);
-      kern<<<(unsigned)(c->nt * c->nt * c->nt), threads, kVjpSmem, s>>>(
+      pdl_launch(kern, (unsigned)(c->nt * c->nt * c->nt), threads, kVjpSmem, s, 
           c->us, c->ids, n, c->bstart, realA, realP, c->g.n, 32 - c->g.logn, c->ntl, rp, inv12h, inv_h, lam_s, c->mt,
           c->vals[0], grad, c->err_dev);
     }
@@ -716,7 +731,7 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
     paint_tiles(c, c->us, c->ids, n, PM_SPECIES_ALL, realA, rp, s, lam_s + (int64_t)j * n);
     fft_forward(c, c->g, c->meshA, c->meshA, 0, s);
     LaunchScope L(c, s, K_ADJOINT);
-    k_adj_combine<<<(unsigned)(c->g.n * c->g.n), 128, 0, s>>>(
+    pdl_launch(k_adj_combine, (unsigned)(c->g.n * c->g.n), 128, 0, s, 
         c->meshA, c->meshB, c->g.n, c->g.pc, c->ksq, c->wforce, c->kvec0, gcoef, j, j > 0,
         learned ? c->mlp_tab : nullptr, learned ? c->meshC : nullptr, c->mlp_gbin);
   }
@@ -743,20 +758,20 @@ int step_vjp(pm_ctx* c, const pm_state* st, double a0, double ah, double a1, con
   uint32_t* u1 = reinterpret_cast<uint32_t*>(c->adj + 4 * m3);
   {  // lambda_F of x1: K2 lambda_p1
     LaunchScope L(c, s, K_ADJOINT);
-    k_vjp_begin<<<blocks(n), 256, 0, s>>>(lx1, lp1, st->id, st->u, st->p, st->f, n, (float)k[0],
+    pdl_launch(k_vjp_begin, blocks(n), 256, 0, s, lx1, lp1, st->id, st->u, st->p, st->f, n, (float)k[0],
                                           (float)(k[1] * 4294967296.0 / c->cfg.box), (float)k[2], Lx, Lp, lamF, u1);
   }
   rc = force_vjp(c, u1, st->id, n, lamF, a1, g, s);
   if (rc != PM_OK) return rc;
   {  // lambda_x1' = lambda_x1 + F_vjp(x1), lambda_ph = lambda_p1 + Delta lambda_x1', lambda_F of x0: K1 lambda_ph
     LaunchScope L(c, s, K_ADJOINT);
-    k_vjp_middle<<<blocks(m3), 256, 0, s>>>(g, m3, (float)k[1], (float)k[0], Lx, Lp, lamF);
+    pdl_launch(k_vjp_middle, blocks(m3), 256, 0, s, g, m3, (float)k[1], (float)k[0], Lx, Lp, lamF);
   }
   rc = force_vjp(c, st->u, st->id, n, lamF, a0, g, s);
   if (rc != PM_OK) return rc;
   {  // lambda_x0 = lambda_x1' + F_vjp(x0)
     LaunchScope L(c, s, K_ADJOINT);
-    k_vjp_end<<<blocks(n), 256, 0, s>>>(g, Lx, Lp, st->id, n, lx0, lp0);
+    pdl_launch(k_vjp_end, blocks(n), 256, 0, s, g, Lx, Lp, st->id, n, lx0, lp0);
   }
   return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ECUDA;
 }
@@ -790,14 +805,14 @@ int ic_vjp(pm_ctx* c, const float* lx, const float* lp, double a0, double k_fs, 
       {
         LaunchScope L(c, s, K_ADJOINT);
         if (species == 0)
-          k_icadj_cdm<<<blocks(n_cdm), 256, 0, s>>>(lx, lp, nc, rp, comp, D0, gp0, n, realA);
+          pdl_launch(k_icadj_cdm, blocks(n_cdm), 256, 0, s, lx, lp, nc, rp, comp, D0, gp0, n, realA);
         else
-          k_icadj_nu<<<blocks((int64_t)cf.nsites * cf.nsites * cf.nsites), 256, 0, s>>>(
+          pdl_launch(k_icadj_nu, blocks((int64_t)cf.nsites * cf.nsites * cf.nsites), 256, 0, s, 
               lx, lp, nc, rp, comp, D0, gp0, cf.nsites, stride, j0, cf.nshell * ndir, n_cdm, n, realA);
       }
       fft_forward(c, gi, c->meshA, c->meshA, 0, s);
       LaunchScope L(c, s, K_ADJOINT);
-      k_icadj_kspace<<<(unsigned)(nc * nc), 128, 0, s>>>(c->meshA, c->meshB, nc, gi.pc,
+      pdl_launch(k_icadj_kspace, (unsigned)(nc * nc), 128, 0, s, c->meshA, c->meshB, nc, gi.pc,
                                                          species == 0 ? c->ic_amp : c->ic_amp_nu, comp,
                                                          species == 1 && even ? 1 : 0, first ? 0 : 1);
       first = false;

@@ -21,6 +21,7 @@ namespace {
 
 __global__ void k_ic_za(const float2* __restrict__ wk, float2* __restrict__ sk, int nc, int pc,
                         const float* __restrict__ amp, int comp, int phase_shift) {
+  pdl_begin();
   const int x = blockIdx.x / nc, y = blockIdx.x % nc;
   const int nx = x < nc / 2 ? x : x - nc, ny = y < nc / 2 ? y : y - nc;
   for (int kz = threadIdx.x; kz <= nc / 2; kz += blockDim.x) {
@@ -47,6 +48,7 @@ __global__ void k_ic_za(const float2* __restrict__ wk, float2* __restrict__ sk, 
 __global__ void k_ic_cdm(const float* __restrict__ s, int nc, int rp, int comp, double cell,
                          double D0, double gp0, double to_fix, int64_t n_offset,
                          uint32_t* __restrict__ u, float* __restrict__ p, int64_t n_total) {
+  pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t ncell = (int64_t)nc * nc * nc;
   if (i >= ncell) return;
@@ -64,6 +66,7 @@ __global__ void k_ic_nu(const float* __restrict__ s, int nc, int rp, int comp, i
                         double to_fix, int nshell, int ndir, const double* __restrict__ tab,
                         int64_t n_offset, int64_t n_nu, uint32_t* __restrict__ u,
                         float* __restrict__ p, int64_t n_total) {
+  pdl_begin();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n_nu) return;
   const int dir = (int)(k % ndir);
@@ -92,6 +95,7 @@ __global__ void k_ic_nu_pseudo(const float* __restrict__ s, int nc, int rp, int 
                                int nF, double dq, const float* __restrict__ uni, int64_t n_offset,
                                int64_t n_nu, uint32_t* __restrict__ u, float* __restrict__ p,
                                int64_t n_total) {
+  pdl_begin();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n_nu) return;
   const int sx = (int)(k / ((int64_t)nsites * nsites)), sy = (int)((k / nsites) % nsites),
@@ -117,6 +121,7 @@ __global__ void k_ic_nu_pseudo(const float* __restrict__ s, int nc, int rp, int 
 }
 
 __global__ void k_iota(uint32_t* __restrict__ id, int64_t n) {
+  pdl_begin();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) id[i] = (uint32_t)i;
 }
@@ -221,7 +226,7 @@ int ic_build(pm_ctx* c, const float* noise, double a0, double k_fs, pm_state* st
     for (int comp = 0; comp < 3; ++comp) {
       {
         LaunchScope Lz(c, s, K_IC_ZA);
-        k_ic_za<<<(unsigned)(nc * nc), 128, 0, s>>>(A, B, nc, gi.pc,
+        pdl_launch(k_ic_za, (unsigned)(nc * nc), 128, 0, s, A, B, nc, gi.pc,
                                                     species == 0 ? c->ic_amp : c->ic_amp_nu, comp,
                                                     species == 1 && even ? 1 : 0);
       }
@@ -229,14 +234,14 @@ int ic_build(pm_ctx* c, const float* noise, double a0, double k_fs, pm_state* st
       const float* sr = reinterpret_cast<const float*>(B);
       LaunchScope La(c, s, K_IC_ASSEMBLE);
       if (species == 0) {
-        k_ic_cdm<<<(unsigned)((n_cdm + 255) / 256), 256, 0, s>>>(
+        pdl_launch(k_ic_cdm, (unsigned)((n_cdm + 255) / 256), 256, 0, s, 
             sr, nc, 2 * gi.pc, comp, L / nc, D0, gp0, to_fix, 0, st->u, st->p, st->n);
       } else if (uniforms) {
-        k_ic_nu_pseudo<<<(unsigned)((n_nu + 255) / 256), 256, 0, s>>>(
+        pdl_launch(k_ic_nu_pseudo, (unsigned)((n_nu + 255) / 256), 256, 0, s, 
             sr, nc, 2 * gi.pc, comp, cf.nsites, stride, j0, L / cf.nsites, 0.5 * L / nc, D0, gp0,
             to_fix, pscale_ps, tab, kNF, kQmax / (kNF - 1), uniforms, n_cdm, n_nu, st->u, st->p, st->n);
       } else {
-        k_ic_nu<<<(unsigned)((n_nu + 255) / 256), 256, 0, s>>>(
+        pdl_launch(k_ic_nu, (unsigned)((n_nu + 255) / 256), 256, 0, s, 
             sr, nc, 2 * gi.pc, comp, cf.nsites, stride, j0, L / cf.nsites, 0.5 * L / nc, D0, gp0,
             to_fix, cf.nshell, ndir, tab, n_cdm, n_nu, st->u, st->p, st->n);
       }
@@ -244,7 +249,7 @@ int ic_build(pm_ctx* c, const float* noise, double a0, double k_fs, pm_state* st
   }
   {
     LaunchScope Li(c, s, K_IC_ASSEMBLE);
-    k_iota<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(st->id, n);
+    pdl_launch(k_iota, (unsigned)((n + 255) / 256), 256, 0, s, st->id, n);
   }
   if (tab) cudaFreeAsync(tab, s);
   if (cudaGetLastError() != cudaSuccess) return PM_ECUDA;

@@ -65,6 +65,7 @@ __device__ __forceinline__ void load_theta(const float* __restrict__ theta, floa
 // tab[s] = m(sqrt(s) / (N/2), a)
 __global__ void __launch_bounds__(256) k_mlp_table(const float* __restrict__ theta, float a, float inv_half,
                                                    int64_t ntab, float* __restrict__ tab) {
+  pdl_begin();
   __shared__ __align__(16) float th[NP + 3];
   load_theta(theta, th);
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < ntab;
@@ -75,6 +76,7 @@ __global__ void __launch_bounds__(256) k_mlp_table(const float* __restrict__ the
 // out[i] = m(kappa[i], a[i])
 __global__ void __launch_bounds__(256) k_mlp_eval(const float* __restrict__ theta, const float* __restrict__ kappa,
                                                   const float* __restrict__ av, int64_t n, float* __restrict__ out) {
+  pdl_begin();
   __shared__ __align__(16) float th[NP + 3];
   load_theta(theta, th);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -85,6 +87,7 @@ __global__ void __launch_bounds__(256) k_mlp_eval(const float* __restrict__ thet
 __global__ void k_green_apply(const float2* __restrict__ rho, float2* __restrict__ phi, int nm, int pc,
                               const float* __restrict__ ksq, const float* __restrict__ winv, float gcoef,
                               const float* __restrict__ mtab) {
+  pdl_begin();
   const int x = blockIdx.x / nm, y = blockIdx.x % nm;
   const int nx = x < nm / 2 ? x : x - nm, ny = y < nm / 2 ? y : y - nm;
   for (int kz = threadIdx.x; kz <= nm / 2; kz += blockDim.x) {
@@ -111,6 +114,7 @@ __global__ void __launch_bounds__(BW_THREADS) k_mlp_backward(const float* __rest
                                                              float inv_half, int64_t ntab,
                                                              double* __restrict__ gbin,
                                                              double* __restrict__ dtheta) {
+  pdl_begin();
   extern __shared__ __align__(16) float sm[];
   float* th = sm;
   float* H1 = th + NP + 3;
@@ -203,6 +207,7 @@ __global__ void __launch_bounds__(BW_THREADS) k_mlp_backward(const float* __rest
 __global__ void k_adam(float* __restrict__ theta, const float* __restrict__ grad, float* __restrict__ m,
                        float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float bc1,
                        float bc2) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float g = grad[i];
@@ -215,6 +220,7 @@ __global__ void k_adam(float* __restrict__ theta, const float* __restrict__ grad
 
 __global__ void k_grad_out(const double* __restrict__ acc, float* __restrict__ out, int n, int reset,
                            double* __restrict__ acc_w) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   out[i] = (float)acc[i];
@@ -224,6 +230,7 @@ __global__ void k_grad_out(const double* __restrict__ acc, float* __restrict__ o
 // ref_c[d][id_ref[i]] = u_ref[d][i]
 __global__ void k_ref_canonical(const uint32_t* __restrict__ u_ref, const uint32_t* __restrict__ id_ref,
                                 int64_t n, uint32_t* __restrict__ ref_c, int* __restrict__ err) {
+  pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t j = id_ref ? (int64_t)id_ref[i] : i;
@@ -250,6 +257,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // sum of the particle masses
 __global__ void k_mass_sum(const uint32_t* __restrict__ id, int64_t n, MassTable mt, int species,
                            double* __restrict__ out, int* __restrict__ err) {
+  pdl_begin();
   __shared__ double red[32];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double m = 0.0;
@@ -267,6 +275,7 @@ __global__ void k_disp_loss(const uint32_t* __restrict__ u, const uint32_t* __re
                             const uint32_t* __restrict__ ref_c, MassTable mt, int species, float scale,
                             const double* __restrict__ wsum, float* __restrict__ lam,
                             double* __restrict__ loss) {
+  pdl_begin();
   __shared__ double red[32];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double l = 0.0;
@@ -338,13 +347,13 @@ void mlp_table(pm_ctx* c, double a, cudaStream_t s) {
   }
   LaunchScope L(c, s, K_MLP_TABLE);
   const unsigned grid = (unsigned)std::min<int64_t>(nblocks(c->mlp_ntab), 4 * 152);
-  k_mlp_table<<<grid, 256, 0, s>>>(c->mlp_theta, (float)a, 2.0f / (float)c->g.n, c->mlp_ntab, c->mlp_tab);
+  pdl_launch(k_mlp_table, grid, 256, 0, s, c->mlp_theta, (float)a, 2.0f / (float)c->g.n, c->mlp_ntab, c->mlp_tab);
 }
 
 void mlp_green_apply(pm_ctx* c, const float2* rho_k, float2* phi_k, cudaStream_t s) {
   LaunchScope L(c, s, K_MLP_MISC);
   const double nn = (double)c->g.n;
-  k_green_apply<<<(unsigned)(c->g.n * c->g.n), 128, 0, s>>>(rho_k, phi_k, c->g.n, c->g.pc, c->ksq, c->wforce,
+  pdl_launch(k_green_apply, (unsigned)(c->g.n * c->g.n), 128, 0, s, rho_k, phi_k, c->g.n, c->g.pc, c->ksq, c->wforce,
                                                            (float)(-1.5 * c->cosmo.omega_m0 / (nn * nn * nn)),
                                                            c->mlp_tab);
 }
@@ -357,7 +366,7 @@ void mlp_backward(pm_ctx* c, double a, cudaStream_t s) {
     attr = true;
   }
   LaunchScope L(c, s, K_MLP_BACKWARD);
-  k_mlp_backward<<<nblocks(c->mlp_ntab, CH), BW_THREADS, BW_SMEM, s>>>(
+  pdl_launch(k_mlp_backward, nblocks(c->mlp_ntab, CH), BW_THREADS, BW_SMEM, s, 
       c->mlp_theta, (float)a, 2.0f / (float)c->g.n, c->mlp_ntab, c->mlp_gbin, c->mlp_dtheta);
 }
 
@@ -395,7 +404,7 @@ int pm_mlp_eval(pm_ctx* c, const float* kappa, const float* a, int64_t n, float*
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   LaunchScope L(c, s, K_MLP_MISC);
   const unsigned grid = (unsigned)std::min<int64_t>(nblocks(n), 4 * 152);
-  k_mlp_eval<<<grid, 256, 0, s>>>(c->mlp_theta, kappa, a, n, m_out);
+  pdl_launch(k_mlp_eval, grid, 256, 0, s, c->mlp_theta, kappa, a, n, m_out);
   return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ECUDA;
 }
 
@@ -416,7 +425,7 @@ int pm_mlp_grad(pm_ctx* c, float* grad_out, int64_t nparam, int32_t reset, void*
   if (!c->mlp_theta || nparam != NP || !grad_out) return PM_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   LaunchScope L(c, s, K_MLP_MISC);
-  k_grad_out<<<nblocks(NP), 256, 0, s>>>(c->mlp_dtheta, grad_out, NP, reset ? 1 : 0, c->mlp_dtheta);
+  pdl_launch(k_grad_out, nblocks(NP), 256, 0, s, c->mlp_dtheta, grad_out, NP, reset ? 1 : 0, c->mlp_dtheta);
   return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ECUDA;
 }
 
@@ -429,7 +438,7 @@ int pm_mlp_adam(pm_ctx* c, const float* grad, int64_t nparam, double lr, double 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const double bc1 = 1.0 - std::pow(beta1, (double)t), bc2 = 1.0 - std::pow(beta2, (double)t);
   LaunchScope L(c, s, K_MLP_MISC);
-  k_adam<<<nblocks(NP), 256, 0, s>>>(c->mlp_theta, grad, c->mlp_adam, c->mlp_adam + NP, NP, (float)lr,
+  pdl_launch(k_adam, nblocks(NP), 256, 0, s, c->mlp_theta, grad, c->mlp_adam, c->mlp_adam + NP, NP, (float)lr,
                                      (float)beta1, (float)beta2, (float)eps, (float)bc1, (float)bc2);
   return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ECUDA;
 }
@@ -454,15 +463,15 @@ int pm_displacement_loss(pm_ctx* c, const uint32_t* u, const uint32_t* id, const
   PM_CUDA_TRY(cudaMemsetAsync(c->mlp_red, 0, sizeof(double) * 2, s));
   {
     LaunchScope L(c, s, K_MLP_MISC);
-    k_ref_canonical<<<nblocks(n), 256, 0, s>>>(u_ref, id_ref, n, ref_c, c->err_dev);
+    pdl_launch(k_ref_canonical, nblocks(n), 256, 0, s, u_ref, id_ref, n, ref_c, c->err_dev);
   }
   {
     LaunchScope L(c, s, K_MLP_MISC);
-    k_mass_sum<<<nblocks(n), 256, 0, s>>>(id, n, c->mt, species, c->mlp_red, c->err_dev);
+    pdl_launch(k_mass_sum, nblocks(n), 256, 0, s, id, n, c->mt, species, c->mlp_red, c->err_dev);
   }
   {
     LaunchScope L(c, s, K_MLP_MISC);
-    k_disp_loss<<<nblocks(n), 256, 0, s>>>(u, id, n, ref_c, c->mt, species, (float)(c->cfg.box / 4294967296.0),
+    pdl_launch(k_disp_loss, nblocks(n), 256, 0, s, u, id, n, ref_c, c->mt, species, (float)(c->cfg.box / 4294967296.0),
                                            c->mlp_red, lam_x, c->mlp_red + 1);
   }
   double h[2];

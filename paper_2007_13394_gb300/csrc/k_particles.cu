@@ -324,6 +324,7 @@ __global__ void __launch_bounds__(NT, FAST ? 2048 / NT : 1) k_paint_tiles(
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
     const uint32_t* __restrict__ bstart, float* __restrict__ mesh, const __grid_constant__ MassTable mt, int species,
     int nm, int shift, int ntl, int row_pitch, int* __restrict__ err, const float* __restrict__ wts) {
+  pdl_begin();
   __shared__ __align__(16) unsigned int accw[FAST ? kFastWords : 2 * kAccWords];
   __shared__ uint32_t run_lo[14], run_pre[15];
   paint_tile<FAST, NW, NT>(blockIdx.x, accw, run_lo, run_pre, us, ids, n, bstart, mesh, mt, species, nm,
@@ -339,6 +340,7 @@ __global__ void __launch_bounds__(kPaint3Threads, 2) k_paint_weights3(
     const uint32_t* __restrict__ us, int64_t n, const uint32_t* __restrict__ bstart, float* __restrict__ m0,
     float* __restrict__ m1, float* __restrict__ m2, int nm, int shift, int ntl, int row_pitch, int* __restrict__ err,
     const float* __restrict__ wts) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned int accw3[];
   __shared__ uint32_t run_lo[14], run_pre[15];
   const MassTable none{};
@@ -353,6 +355,7 @@ __global__ void k_readout_kick(const uint32_t* __restrict__ us, const float* __r
                                int comp, float K, float* __restrict__ p_out,
                                float* __restrict__ f_out, uint32_t* __restrict__ u_out,
                                uint32_t* __restrict__ id_out, const uint32_t* __restrict__ perm) {
+  pdl_begin();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t ux = us[i], uy = us[n + i], uz = us[2 * n + i];
@@ -394,6 +397,7 @@ __global__ void k_readout3_kick(const uint32_t* __restrict__ us, const float* __
                                 float K, float* __restrict__ p_out, float* __restrict__ f_out,
                                 uint32_t* __restrict__ u_out, uint32_t* __restrict__ id_out,
                                 const uint32_t* __restrict__ perm) {
+  pdl_begin();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t ux = us[i], uy = us[n + i], uz = us[2 * n + i];
@@ -571,6 +575,7 @@ __global__ void __launch_bounds__(NT, NODES ? 2 : (NT == 256 ? 5 : 1024 / NT)) k
     int ntl, int row_pitch, float inv12h, float K, float* __restrict__ p_out, float* __restrict__ f_out,
     uint32_t* __restrict__ u_out, uint32_t* __restrict__ id_out, const uint32_t* __restrict__ perm,
     int* __restrict__ err, DriftNext dn) {
+  pdl_begin();
   extern __shared__ __align__(16) float sp[];  // the potential, then (NODES) the nodes' forces
   float* const nodes = sp + kSpanXY * kFd4SX;
   const int t = threadIdx.x;
@@ -705,6 +710,7 @@ __global__ void k_kick_drift_keys(uint32_t* __restrict__ u, float* __restrict__ 
                                   int shift, int ntl, uint32_t* __restrict__ keys,
                                   uint32_t* __restrict__ cnt3, long long nb1, const uint32_t* __restrict__ bprev,
                                   uint32_t* __restrict__ low, uint32_t* __restrict__ flags, int* __restrict__ err) {
+  pdl_begin();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned act = __ballot_sync(0xffffffffu, i < n);
   if (i >= n) return;
@@ -735,12 +741,14 @@ __global__ void k_kick_drift_keys(uint32_t* __restrict__ u, float* __restrict__ 
 
 __global__ void k_repack_real(const float* __restrict__ src, int sp, float* __restrict__ dst,
                               int dp, int nm) {
+  pdl_begin();
   long long row = blockIdx.x;
   for (int z = threadIdx.x; z < nm; z += blockDim.x) dst[row * dp + z] = src[row * sp + z];
 }
 
 __global__ void k_repack_complex(const float2* __restrict__ src, int sp, float2* __restrict__ dst,
                                  int dp, int ncols) {
+  pdl_begin();
   long long row = blockIdx.x;
   for (int z = threadIdx.x; z < ncols; z += blockDim.x) dst[row * dp + z] = src[row * sp + z];
 }
@@ -766,7 +774,7 @@ void paint_tiles(pm_ctx* c, const uint32_t* us, const uint32_t* ids, int64_t n, 
                              : (threads == 512 ? k_paint_tiles<true, 0, 512> : k_paint_tiles<true, 0, 256>);
     }
   }
-  kern<<<grid, threads, 0, s>>>(us, ids, n, c->bstart, mesh, c->mt, species, c->g.n, 32 - c->g.logn, c->ntl,
+  pdl_launch(kern, grid, threads, 0, s, us, ids, n, c->bstart, mesh, c->mt, species, c->g.n, 32 - c->g.logn, c->ntl,
                                       row_pitch, c->err_dev, weights);
 }
 
@@ -778,7 +786,7 @@ void paint_weights3(pm_ctx* c, const uint32_t* us, int64_t n, const float* weigh
     attr = true;
   }
   LaunchScope L(c, s, K_PAINT);
-  k_paint_weights3<<<(unsigned)(c->nt * c->nt * c->nt), kPaint3Threads, kPaint3Smem, s>>>(
+  pdl_launch(k_paint_weights3, (unsigned)(c->nt * c->nt * c->nt), kPaint3Threads, kPaint3Smem, s, 
       us, n, c->bstart, m0, m1, m2, c->g.n, 32 - c->g.logn, c->ntl, row_pitch, c->err_dev, weights);
 }
 
@@ -788,7 +796,7 @@ void readout_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint32_t
                   cudaStream_t s) {
   if (n == 0) return;
   LaunchScope L(c, s, K_READOUT_KICK);
-  k_readout_kick<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
+  pdl_launch(k_readout_kick, (unsigned)((n + 255) / 256), 256, 0, s, 
       us, ps, ids, n, mesh, c->g.n, 32 - c->g.logn, row_pitch, comp, K, p_out, f_out, u_out,
       id_out, perm_scatter);
 }
@@ -799,7 +807,7 @@ void readout3_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint32_
                    const uint32_t* perm_scatter, cudaStream_t s) {
   if (n == 0) return;
   LaunchScope L(c, s, K_READOUT3_KICK);
-  k_readout3_kick<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
+  pdl_launch(k_readout3_kick, (unsigned)((n + 255) / 256), 256, 0, s, 
       us, ps, ids, n, mx, my, mz, c->g.n, 32 - c->g.logn, row_pitch, K, p_out, f_out, u_out, id_out,
       perm_scatter);
 }
@@ -830,7 +838,7 @@ void readout_fd4_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr[dn != nullptr][v] = true;
   }
-  kern<<<grid, threads, smem, s>>>(us, ps, ids, n, c->bstart, phi, c->g.n, 32 - c->g.logn,
+  pdl_launch(kern, grid, threads, smem, s, us, ps, ids, n, c->bstart, phi, c->g.n, 32 - c->g.logn,
                                                              c->ntl, row_pitch, inv12h, K, p_out, f_out, u_out, id_out,
                                                              dn ? nullptr : perm_scatter, c->err_dev,
                                                              dn ? *dn : DriftNext{});
@@ -844,23 +852,23 @@ void kick_drift_keys(pm_ctx* c, uint32_t* u, float* p, const float* f, int64_t n
   LaunchScope L(c, s, K_KICK_DRIFT_KEYS);
   const unsigned grid = (unsigned)((n + 255) / 256);
   if (resort)
-    k_kick_drift_keys<true><<<grid, 256, 0, s>>>(u, p, f, n, K1, dscale, 32 - c->g.logn, c->ntl, c->keys[0],
+    pdl_launch(k_kick_drift_keys<true>, grid, 256, 0, s, u, p, f, n, K1, dscale, 32 - c->g.logn, c->ntl, c->keys[0],
                                                   c->counts, nb1, c->bprev, c->rs_low, c->rs_dev, c->err_dev);
   else
-    k_kick_drift_keys<false><<<grid, 256, 0, s>>>(u, p, f, n, K1, dscale, 32 - c->g.logn, c->ntl, c->keys[0],
+    pdl_launch(k_kick_drift_keys<false>, grid, 256, 0, s, u, p, f, n, K1, dscale, 32 - c->g.logn, c->ntl, c->keys[0],
                                                    c->counts, nb1, nullptr, nullptr, nullptr, c->err_dev);
 }
 
 void repack_real(pm_ctx* c, const Geom& g, const float* src, int sp, float* dst, int dp,
                  cudaStream_t s) {
   LaunchScope L(c, s, K_REPACK);
-  k_repack_real<<<(unsigned)g.rows(), 256, 0, s>>>(src, sp, dst, dp, g.n);
+  pdl_launch(k_repack_real, (unsigned)g.rows(), 256, 0, s, src, sp, dst, dp, g.n);
 }
 
 void repack_complex(pm_ctx* c, const Geom& g, const float2* src, int sp, float2* dst, int dp,
                     cudaStream_t s) {
   LaunchScope L(c, s, K_REPACK);
-  k_repack_complex<<<(unsigned)g.rows(), 256, 0, s>>>(src, sp, dst, dp, g.n / 2 + 1);
+  pdl_launch(k_repack_complex, (unsigned)g.rows(), 256, 0, s, src, sp, dst, dp, g.n / 2 + 1);
 }
 
 }  // namespace pmnu

@@ -62,6 +62,7 @@ __device__ __forceinline__ void count_unit(int a, int b, int nm, int tmax, uint3
 }
 
 __global__ void k_power_counts(int nm, int units, int tmax, uint32_t* __restrict__ r2) {
+  pdl_begin();
   const int w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= units) return;
   int a, b;
@@ -78,6 +79,7 @@ __global__ void __launch_bounds__(kPowThreads) k_power_bin(const float2* __restr
                                                            const float* __restrict__ winv,
                                                            double* __restrict__ partial,
                                                            uint32_t* __restrict__ r2) {
+  pdl_begin();
   extern __shared__ double sh[];  // nbins per warp
   for (int i = threadIdx.x; i < kPowWarps * nbins; i += kPowThreads) sh[i] = 0.0;
   __syncthreads();
@@ -153,6 +155,7 @@ __global__ void __launch_bounds__(kRedThreads) k_power_reduce(const double* __re
                                                               int nm, const uint32_t* __restrict__ r2, double kf,
                                                               float norm, const float2* __restrict__ da,
                                                               const float2* __restrict__ db, double* __restrict__ out) {
+  pdl_begin();
   constexpr int W = kRedThreads / 32;
   __shared__ double red[3][W];
   const int b = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5, half = nm / 2;
@@ -202,6 +205,7 @@ __global__ void __launch_bounds__(kRedThreads) k_power_reduce(const double* __re
 // cw[b] = 2 dL_dP[b] V / (N^6 rho_bar^2 N_b), the weights of k_power_weight (0 for empty bins)
 __global__ void k_power_cw(const double* __restrict__ counts, const double* __restrict__ dL, int nbins, double vol,
                            double n3, const float2* __restrict__ d, float* __restrict__ cw) {
+  pdl_begin();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nbins) return;
   const double rho_bar = (double)d[0].x / n3, nb = counts[b];
@@ -213,6 +217,7 @@ __global__ void k_power_cw(const double* __restrict__ counts, const double* __re
 __global__ void __launch_bounds__(kPowThreads) k_power_weight(float2* __restrict__ d, int nm, int pc, int nbins,
                                                               const float* __restrict__ winv,
                                                               const float* __restrict__ cw) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const long long row = (long long)blockIdx.x * kPowWarps + (threadIdx.x >> 5);  // x N + y, N^2 rows in all
   const int x = (int)(row / nm), y = (int)(row % nm);
@@ -265,19 +270,19 @@ int power_weight(pm_ctx* c, int nbins, const double* dL_dP, cudaStream_t s) {
   PM_CUDA_TRY(cudaMemsetAsync(p.r2, 0, sizeof(uint32_t) * (p.tmax + 1), s));
   {
     LaunchScope L(c, s, K_POWER_BIN);
-    k_power_counts<<<(p.units + 255) / 256, 256, 0, s>>>(g.n, p.units, p.tmax, p.r2);
+    pdl_launch(k_power_counts, (p.units + 255) / 256, 256, 0, s, g.n, p.units, p.tmax, p.r2);
   }
   {
     LaunchScope L(c, s, K_POWER_REDUCE);
-    k_power_reduce<<<nbins, kRedThreads, 0, s>>>(nullptr, 0, nbins, g.n, p.r2, kf, 0.0f, nullptr, nullptr, c->pk_final);
+    pdl_launch(k_power_reduce, nbins, kRedThreads, 0, s, nullptr, 0, nbins, g.n, p.r2, kf, 0.0f, nullptr, nullptr, c->pk_final);
   }
   {
     LaunchScope L(c, s, K_POWER_REDUCE);
-    k_power_cw<<<(nbins + 255) / 256, 256, 0, s>>>(c->pk_final, p.dL, nbins, c->cfg.box * c->cfg.box * c->cfg.box, n3,
+    pdl_launch(k_power_cw, (nbins + 255) / 256, 256, 0, s, c->pk_final, p.dL, nbins, c->cfg.box * c->cfg.box * c->cfg.box, n3,
                                                    c->meshA, c->pk_w);
   }
   LaunchScope L(c, s, K_POWER_BIN);
-  k_power_weight<<<(unsigned)(g.rows() / kPowWarps), kPowThreads, 0, s>>>(c->meshA, g.n, g.pc, nbins, c->winv, c->pk_w);
+  pdl_launch(k_power_weight, (unsigned)(g.rows() / kPowWarps), kPowThreads, 0, s, c->meshA, g.n, g.pc, nbins, c->winv, c->pk_w);
   return PM_OK;
 }
 
@@ -299,11 +304,11 @@ int power_bin(pm_ctx* c, const float2* da, const float2* db, int nbins, double* 
   PM_CUDA_TRY(cudaMemsetAsync(p.r2, 0, sizeof(uint32_t) * (p.tmax + 1), s));
   {
     LaunchScope L(c, s, K_POWER_BIN);
-    kern<<<p.rows, kPowThreads, smem, s>>>(da, db, g.n, g.pc, nbins, p.units, p.tmax, c->winv, c->pk_partial, p.r2);
+    pdl_launch(kern, p.rows, kPowThreads, smem, s, da, db, g.n, g.pc, nbins, p.units, p.tmax, c->winv, c->pk_partial, p.r2);
   }
   {
     LaunchScope L(c, s, K_POWER_REDUCE);
-    k_power_reduce<<<nbins, kRedThreads, 0, s>>>(c->pk_partial, p.rows, nbins, g.n, p.r2, kf, norm, da, db,
+    pdl_launch(k_power_reduce, nbins, kRedThreads, 0, s, c->pk_partial, p.rows, nbins, g.n, p.r2, kf, norm, da, db,
                                                  c->pk_final);
   }
   std::vector<double> h(3 * nbins);

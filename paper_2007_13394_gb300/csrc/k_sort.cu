@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* __restric
                                                        uint32_t* __restrict__ out,
                                                        unsigned long long* __restrict__ status,
                                                        uint32_t* __restrict__ counter, int* __restrict__ err) {
+  pdl_begin();
   __shared__ uint32_t ws[32], s_tile, s_before;
   const int t = threadIdx.x;
   if (t == 0) s_tile = atomicAdd(counter, 1u);
@@ -178,6 +179,7 @@ __device__ __forceinline__ void count_digit(uint32_t d, uint32_t* h) {
 template <int BITS>
 __global__ void __launch_bounds__(kCountThreads) k_keys(const uint32_t* __restrict__ u, int64_t n, int shift, int ntl,
                                                         uint32_t* __restrict__ keys, uint32_t* __restrict__ hist) {
+  pdl_begin();
   constexpr int DIG = 1 << BITS;
   __shared__ uint32_t h[DIG];
   for (int i = threadIdx.x; i < DIG; i += kCountThreads) h[i] = 0;
@@ -217,6 +219,7 @@ __global__ void __launch_bounds__(kCountThreads) k_digits(const uint32_t* __rest
                                                           uint32_t* __restrict__ hist,
                                                           const uint32_t* __restrict__ flags,
                                                           const uint32_t* __restrict__ bstart3, long long nb1) {
+  pdl_begin();
   constexpr int DIG = 1 << BITS;
   __shared__ uint32_t h[DIG];
   for (int i = threadIdx.x; i < DIG; i += kCountThreads) h[i] = 0;
@@ -242,6 +245,7 @@ __global__ void __launch_bounds__(kCountThreads) k_digits(const uint32_t* __rest
 // Exclusive scan of each digit's counts over the C chunks, in place; totals[d].  A warp a digit.
 __global__ void __launch_bounds__(256) k_chunk_scan(uint32_t* __restrict__ hist, int C, int digits,
                                                     uint32_t* __restrict__ totals) {
+  pdl_begin();
   const int d = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (d >= digits) return;
   uint32_t* const h = hist + (size_t)d * C;
@@ -282,6 +286,7 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
     const uint32_t* __restrict__ hist, const uint32_t* __restrict__ totals, uint32_t* __restrict__ kout,
     uint32_t* __restrict__ vout, const uint32_t* __restrict__ flags, const uint32_t* __restrict__ bstart3,
     long long nb1) {
+  pdl_begin();
   constexpr int DIG = 1 << BITS, PER = DIG > kRadixThreads ? DIG / kRadixThreads : 1;
   constexpr uint32_t MASK = DIG - 1;
   constexpr int KPW = kRadixTile / kRadixWarps;  // keys per warp
@@ -421,6 +426,7 @@ constexpr int kPackThreads = 256;
 __global__ void __launch_bounds__(kPackThreads) k_pack(const uint32_t* __restrict__ u, const float* __restrict__ p,
                                                        const uint32_t* __restrict__ id, int64_t n, int64_t i0,
                                                        uint32_t* __restrict__ rec) {
+  pdl_begin();
   __shared__ uint32_t sh[7 * kPackThreads];
   const int W = p ? 7 : 4, t = threadIdx.x;
   const int64_t first = i0 + (int64_t)blockIdx.x * kPackThreads, i = first + t;
@@ -448,6 +454,7 @@ __global__ void k_gather(const uint32_t* __restrict__ u, const float* __restrict
                          float* __restrict__ ps, uint32_t* __restrict__ ids, const uint32_t* __restrict__ skeys,
                          long long nb1, unsigned nbb, uint32_t* __restrict__ bstart,
                          const uint32_t* __restrict__ rec, int64_t i0) {
+  pdl_begin();
   if (blockIdx.x < nbb) {
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nb1) return;
@@ -523,6 +530,7 @@ __global__ void __launch_bounds__(NT) k_resort_old_tiles(
     long long nb1, const uint32_t* __restrict__ low, uint32_t* __restrict__ us, float* __restrict__ ps,
     uint32_t* __restrict__ ids, uint32_t* __restrict__ mk, uint32_t* __restrict__ mv,
     const uint32_t* __restrict__ flags, int* __restrict__ err, uint4* __restrict__ stage, int64_t stage_room) {
+  pdl_begin();
   constexpr int W = NT / 32;
   __shared__ uint32_t cls_lo[9];   // bprev[8 O + c]
   __shared__ uint32_t cls_m0[8];   // movers of the tile before class c's first particle
@@ -667,6 +675,7 @@ __global__ void k_place_movers(const uint32_t* __restrict__ mk, const uint32_t* 
                                uint32_t* __restrict__ us, float* __restrict__ ps, uint32_t* __restrict__ ids,
                                const uint32_t* __restrict__ flags, int* __restrict__ err,
                                const uint4* __restrict__ stage, int64_t stage_room, long long* __restrict__ stats) {
+  pdl_begin();
   const bool all = (*flags & 1u) != 0u;
   const int64_t nm = movers_of(flags, bstart3, nb1, n);
   if (all || nm > stage_room) stage = nullptr;
@@ -697,7 +706,7 @@ void launch_scatter(pm_ctx* c, const uint32_t* kin, const uint32_t* vin, int64_t
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     attr[raw] = true;
   }
-  kern<<<chunks_of(n), kRadixThreads, dyn, s>>>(kin, vin, n, shift, c->hist, c->digit_totals, kout, vout, flags,
+  pdl_launch(kern, chunks_of(n), kRadixThreads, dyn, s, kin, vin, n, shift, c->hist, c->digit_totals, kout, vout, flags,
                                                 c->bstart, c->nbuckets + 1);
 }
 
@@ -713,11 +722,11 @@ int passes_of(pm_ctx* c, uint32_t* const kb[2], uint32_t* const vb[2], bool inde
     const int shift = BITS * pass;
     if (!counted || pass > 0) {
       LaunchScope L(c, s, K_RADIX_HIST);
-      k_digits<BITS><<<C, kCountThreads, 0, s>>>(kb[cur], n, shift, c->hist, flags, c->bstart, c->nbuckets + 1);
+      pdl_launch(k_digits<BITS>, C, kCountThreads, 0, s, kb[cur], n, shift, c->hist, flags, c->bstart, c->nbuckets + 1);
     }
     if (!raw_counts(n)) {
       LaunchScope L(c, s, K_SCAN);
-      k_chunk_scan<<<(1 << BITS) / 8, 256, 0, s>>>(c->hist, (int)C, 1 << BITS, c->digit_totals);
+      pdl_launch(k_chunk_scan, (1 << BITS) / 8, 256, 0, s, c->hist, (int)C, 1 << BITS, c->digit_totals);
     }
     LaunchScope L(c, s, K_RADIX_SCATTER);
     launch_scatter<BITS>(c, kb[cur], (pass == 0 && index_vals) ? nullptr : vb[cur], n, shift, kb[cur ^ 1], vb[cur ^ 1],
@@ -759,7 +768,7 @@ int sort_particles(pm_ctx* c, const uint32_t* u, int64_t n, cudaStream_t s) {
     LaunchScope L(c, s, K_KEYS);
     const int shift = 32 - c->g.logn;
     auto kern = c->radix_bits == 9 ? k_keys<9> : (c->radix_bits == 8 ? k_keys<8> : k_keys<7>);
-    kern<<<chunks_of(n), kCountThreads, 0, s>>>(u, n, shift, c->ntl, c->keys[0], c->hist);
+    pdl_launch(kern, chunks_of(n), kCountThreads, 0, s, u, n, shift, c->ntl, c->keys[0], c->hist);
   }
   sort_keys0(c, true, n, s);
   return PM_OK;
@@ -777,13 +786,13 @@ void gather_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint32_t*
   const int64_t rec_bytes = (n - i0) * (p ? 28 : 16);
   if (n - i0 >= (1 << 21) && rec_bytes <= 16 * std::max<int64_t>(c->n_max, 1)) {
     LaunchScope L(c, s, K_GATHER);
-    k_pack<<<(unsigned)((n - i0 + kPackThreads - 1) / kPackThreads), kPackThreads, 0, s>>>(u, p, id, n, i0, rec);
+    pdl_launch(k_pack, (unsigned)((n - i0 + kPackThreads - 1) / kPackThreads), kPackThreads, 0, s, u, p, id, n, i0, rec);
   } else {
     i0 = n;
   }
   LaunchScope L(c, s, K_GATHER);
   const unsigned nbb = (unsigned)((c->nbuckets + 1 + 255) / 256);
-  k_gather<<<nbb + (unsigned)((n + 255) / 256), 256, 0, s>>>(u, p, id, n, perm, c->us, c->ps, c->ids, c->keys[0],
+  pdl_launch(k_gather, nbb + (unsigned)((n + 255) / 256), 256, 0, s, u, p, id, n, perm, c->us, c->ps, c->ids, c->keys[0],
                                                             c->nbuckets + 1, nbb, c->bstart, rec, i0);
 }
 
@@ -797,7 +806,7 @@ int resort_near_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint3
   const long long nb1 = c->nbuckets + 1;
   {  // bucket starts, stayers' and old keys' movers' starts in one scan
     LaunchScope L(c, s, K_SCAN);
-    k_scan<<<(unsigned)((3 * nb1 + kScanTile - 1) / kScanTile), kScanThreads, 0, s>>>(
+    pdl_launch(k_scan, (unsigned)((3 * nb1 + kScanTile - 1) / kScanTile), kScanThreads, 0, s, 
         c->counts, 3 * nb1, c->bstart, c->scan_status, c->scan_tile, c->err_dev);
   }
   // the movers' records go to the second mesh, free during a step, when they fit (32 bytes a
@@ -808,7 +817,7 @@ int resort_near_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint3
     LaunchScope L(c, s, K_RESORT_PLACE);
     const int threads = tile_threads(c);
     auto kern = threads == 1024 ? k_resort_old_tiles<1024> : (threads == 512 ? k_resort_old_tiles<512> : k_resort_old_tiles<256>);
-    kern<<<(unsigned)((long long)c->nt * c->nt * c->nt), threads, 0, s>>>(
+    pdl_launch(kern, (unsigned)((long long)c->nt * c->nt * c->nt), threads, 0, s, 
         u, p, id, n, c->keys[0], c->bprev, c->bstart, nb1, c->rs_low, c->us, c->ps, c->ids, c->keys[1], c->vals[1],
         c->rs_dev, c->err_dev, stage, room);
   }
@@ -823,7 +832,7 @@ int resort_near_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint3
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     full = std::max(per_sm, 1) * std::max(sms, 1);
   }
-  k_place_movers<<<(unsigned)std::min<int64_t>(full, (n + 255) / 256), 256, 0, s>>>(
+  pdl_launch(k_place_movers, (unsigned)std::min<int64_t>(full, (n + 255) / 256), 256, 0, s, 
       kb[r], vb[r], u, p, id, n, c->bstart, nb1, c->nbuckets, c->rs_low, c->us, c->ps, c->ids, c->rs_dev, c->err_dev,
       stage, room, c->rs_stats);
   return PM_OK;
