@@ -495,14 +495,12 @@ __global__ void k_vjp_end(const float* __restrict__ g, const float* __restrict__
   }
 }
 
-// gather per-component weights into the sorted order: ws[j][k] = w[j][perm[k]]
-__global__ void k_gather3(const float* __restrict__ w, const uint32_t* __restrict__ perm, int64_t n,
-                          int ncomp, float* __restrict__ ws) {
+// gather weights into the sorted order: ws[k] = w[perm[k]]
+__global__ void k_gather_weights(const float* __restrict__ w, const uint32_t* __restrict__ perm, int64_t n,
+                                 float* __restrict__ ws) {
   pdl_begin();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const uint32_t i = perm[k];
-  for (int j = 0; j < ncomp; ++j) ws[(int64_t)j * n + k] = w[(int64_t)j * n + i];
+  if (k < n) ws[k] = w[perm[k]];
 }
 
 // IC transpose: lattice mesh (padded real, nc) of lambda_s for CDM nodes (canonical order)
@@ -587,7 +585,7 @@ unsigned blocks(int64_t n) { return (unsigned)((n + 255) / 256); }
 int gather_weights(pm_ctx* c, const float* w, int64_t n, float* w_sorted, cudaStream_t s) {
   if (n == 0) return PM_OK;
   LaunchScope L(c, s, K_ADJOINT);
-  pdl_launch(k_gather3, blocks(n), 256, 0, s, w, c->vals[0], n, 1, w_sorted);
+  pdl_launch(k_gather_weights, blocks(n), 256, 0, s, w, c->vals[0], n, w_sorted);
   return PM_OK;
 }
 
@@ -616,12 +614,9 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
   if (rc != PM_OK) return rc;
   rc = sort_particles(c, u, n, s);
   if (rc != PM_OK) return rc;
-  gather_sorted(c, u, nullptr, id, n, c->vals[0], s);
-  float* lam_s = c->adj + 6 * 3 * n;  // sorted cotangent, 3n
-  {
-    LaunchScope L(c, s, K_ADJOINT);
-    pdl_launch(k_gather3, blocks(n), 256, 0, s, lam_f, c->vals[0], n, 3, lam_s);
-  }
+  // the cotangents travel with the particles, where the momenta of a step do
+  gather_sorted(c, u, lam_f, id, n, c->vals[0], s);
+  const float* lam_s = c->ps;  // sorted cotangent, 3n
   float* realA = reinterpret_cast<float*>(c->meshA);
   float* realB = reinterpret_cast<float*>(c->meshB);
   const int rp = 2 * c->g.pc;
@@ -675,7 +670,7 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
         attr3[threads == 512] = true;
       }
       const unsigned tiles = (unsigned)(c->nt * c->nt * c->nt);
-      float* const tmp = c->adj + 7 * 3 * n;  // the second term, sorted order
+      float* const tmp = c->adj + 6 * 3 * n;  // the second term, sorted order
       {
         LaunchScope L(c, s, K_ADJOINT);
         pdl_launch(read1, tiles, threads, sm1, s, c->us, c->ids, n, c->bstart, realP, nullptr, nullptr, c->g.n, 32 - c->g.logn,
