@@ -145,6 +145,7 @@ __device__ __forceinline__ void vjp_cp_async16(void* smem_dst, const void* gmem_
 // the CIC weight derivatives.  Bound by the shared-memory pipe (56 + 8 random gathers a
 // particle); a separate pass over B gathered 8 values from global memory and updated the
 // gradient a second time (step_vjp at 256^3: 124 us a force).
+constexpr long long kStagedMin = 200;                  // mean particles a tile, see readout_grad
 constexpr int kVjpSpanB = kTile + 1;                   // cells 0 .. 16 along x and y
 constexpr int kVjpSpanBZ = kTile + 4;                  // cells 0 .. 19 along z
 constexpr int kVjpStageB = kVjpSpanB * kVjpSpanB * (kVjpSpanBZ / 4);
@@ -253,14 +254,16 @@ __global__ void __launch_bounds__(NT) k_force_vjp_readout(
 }
 
 // One mesh's or three meshes' worth of the VJP, staged per tile like B above (the learned path):
-// NM = 1: tmp[d][i] = m_i d/dx_d R[B](x_i) in sorted order; NM = 3: out[d][perm[i]] = tmp[d][i] +
-// sum_j lambda_j(i) d/dx_d R[F_j](x_i).  Staging replaces 8 NM scattered global reads a particle.
+// NM = 1: m_i d/dx_d R[B](x_i), m_i the mass if the species is selected, to out[d][perm[i]] or
+// (perm null) in sorted order to tmp[d][i]; NM = 3: out[d][perm[i]] = tmp[d][i] + sum_j lambda_j(i)
+// d/dx_d R[F_j](x_i).  Staging replaces 8 NM scattered global reads a particle.
 template <int NM, int NT>
 __global__ void __launch_bounds__(NT) k_vjp_readout(
     const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n, const uint32_t* __restrict__ bstart,
     const float* __restrict__ m0, const float* __restrict__ m1, const float* __restrict__ m2, int nm, int shift,
     int ntl, int row_pitch, float inv_h, const float* __restrict__ lam, MassTable mt,
-    const uint32_t* __restrict__ perm, float* __restrict__ tmp, float* __restrict__ out, int* __restrict__ err) {
+    const uint32_t* __restrict__ perm, float* __restrict__ tmp, float* __restrict__ out, int species,
+    int* __restrict__ err) {
   pdl_begin();
   extern __shared__ __align__(16) float sb[];
   const int t = threadIdx.x;
@@ -301,7 +304,7 @@ __global__ void __launch_bounds__(NT) k_vjp_readout(
     float o[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int j = 0; j < NM; ++j) {
-      const float a = NM == 1 ? id_mass(mt, ids[i], PM_SPECIES_ALL, &bad) : lam[(int64_t)j * n + i];
+      const float a = NM == 1 ? id_mass(mt, ids[i], species, &bad) : lam[(int64_t)j * n + i];
       const float* const q = sb + j * kVjpSpanB * kVjpBSX + lx * kVjpBSX + ly * kVjpBSY + lz;
       const float v000 = q[0], v001 = q[1], v010 = q[kVjpBSY], v011 = q[kVjpBSY + 1];
       const float v100 = q[kVjpBSX], v101 = q[kVjpBSX + 1], v110 = q[kVjpBSX + kVjpBSY],
@@ -312,15 +315,20 @@ __global__ void __launch_bounds__(NT) k_vjp_readout(
                        fx * (gz * (v110 - v100) + fz * (v111 - v101));
       const float dZ = gx * (gy * (v001 - v000) + fy * (v011 - v010)) +
                        fx * (gy * (v101 - v100) + fy * (v111 - v110));
-      o[0] += a * dX;
-      o[1] += a * dY;
-      o[2] += a * dZ;
+      if (NM == 3 || a != 0.0f) {  // a masked species takes nothing from the mesh, whatever it holds
+        o[0] += a * dX;
+        o[1] += a * dY;
+        o[2] += a * dZ;
+      }
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const int64_t k = (int64_t)d * n + i;
       if constexpr (NM == 1) {
-        tmp[k] = o[d] * inv_h;
+        if (perm)
+          out[(int64_t)d * n + perm[i]] = o[d] * inv_h;
+        else
+          tmp[k] = o[d] * inv_h;
       } else {
         out[(int64_t)d * n + perm[i]] = fmaf(o[d], inv_h, tmp[k]);
       }
@@ -580,6 +588,11 @@ int ensure_adj(pm_ctx* c, int64_t n) {
 
 unsigned blocks(int64_t n) { return (unsigned)((n + 255) / 256); }
 
+// Threads a tile of the staged VJP readouts: 512 where tiles are full (us a launch of the
+// potentials' readout, 256 / 512 threads: 2000 a tile at 128^3 71 / 60, at 256^3 310 / 293; 580 a
+// tile 35 / 36 and 126 / 139).
+int vjp_threads(const pm_ctx* c, int64_t n) { return n >= 1000LL * c->nt * c->nt * c->nt ? 512 : 256; }
+
 }  // namespace
 
 int gather_weights(pm_ctx* c, const float* w, int64_t n, float* w_sorted, cudaStream_t s) {
@@ -596,6 +609,20 @@ void readout_grad(pm_ctx* c, int64_t n, const float* const* meshes, int nmeshes,
   if (n == 0) return;
   LaunchScope L(c, s, K_ADJOINT);
   const float inv_h = (float)(c->g.n / c->cfg.box);
+  const long long tiles = (long long)c->nt * c->nt * c->nt;
+  // one mesh and the particles' masses: staged per tile where the tiles hold enough particles to
+  // pay for it, and the mesh takes 16-byte copies (rows are whole 16-byte groups).  us, gathered /
+  // staged, by mean particles a tile: 256^3 128 21 / 23, 256 36 / 32, 580 75 / 55; 512^3 128
+  // 150 / 169, 256 257 / 228, 580 576 / 456.
+  if (nmeshes == 1 && !wts_sorted && !accumulate && perm && (reinterpret_cast<uintptr_t>(meshes[0]) & 15) == 0 &&
+      n >= kStagedMin * tiles) {
+    const int threads = vjp_threads(c, n);
+    auto kern = threads == 512 ? k_vjp_readout<1, 512> : k_vjp_readout<1, 256>;
+    pdl_launch(kern, (unsigned)tiles, threads, sizeof(float) * kVjpSpanB * kVjpBSX, s, c->us, c->ids, n, c->bstart,
+               meshes[0], nullptr, nullptr, c->g.n, 32 - c->g.logn, c->ntl, row_pitch, inv_h, nullptr, c->mt, perm,
+               nullptr, out, species, c->err_dev);
+    return;
+  }
   pdl_launch(k_readout_grad, blocks(n), 256, 0, s, c->us, c->ids, n, meshes[0], nmeshes > 1 ? meshes[1] : nullptr,
                                            nmeshes > 2 ? meshes[2] : nullptr, nmeshes, c->g.n,
                                            32 - c->g.logn, row_pitch, inv_h, wts_sorted, c->mt, perm,
@@ -661,7 +688,7 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
       }
       fft_inverse_plain(c, c->g, pot, s);  // B
       const size_t sm1 = sizeof(float) * kVjpSpanB * kVjpBSX;
-      const int threads = std::min(tile_threads(c), 512);
+      const int threads = vjp_threads(c, n);
       auto read1 = threads == 512 ? k_vjp_readout<1, 512> : k_vjp_readout<1, 256>;
       auto read3 = threads == 512 ? k_vjp_readout<3, 512> : k_vjp_readout<3, 256>;
       static bool attr3[2] = {false, false};
@@ -674,7 +701,8 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
       {
         LaunchScope L(c, s, K_ADJOINT);
         pdl_launch(read1, tiles, threads, sm1, s, c->us, c->ids, n, c->bstart, realP, nullptr, nullptr, c->g.n, 32 - c->g.logn,
-                                          c->ntl, rp, inv_h, nullptr, c->mt, nullptr, tmp, nullptr, c->err_dev);
+                                          c->ntl, rp, inv_h, nullptr, c->mt, nullptr, tmp, nullptr, PM_SPECIES_ALL,
+                   c->err_dev);
       }
       // F_y, F_z into the other meshes, F_x in place over phi_k
       fft_inverse_component(c, c->g, c->meshA, c->meshB, 1, s);
@@ -683,14 +711,15 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
       {
         LaunchScope L(c, s, K_ADJOINT);
         pdl_launch(read3, tiles, threads, 3 * sm1, s, c->us, c->ids, n, c->bstart, realA, realB, realP, c->g.n, 32 - c->g.logn,
-                                              c->ntl, rp, inv_h, lam_s, c->mt, c->vals[0], tmp, grad, c->err_dev);
+                                              c->ntl, rp, inv_h, lam_s, c->mt, c->vals[0], tmp, grad, PM_SPECIES_ALL,
+                   c->err_dev);
       }
       mlp_backward(c, a, s);
       return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ECUDA;
     }
     fft_potential(c, c->g, c->meshA, s);
     fft_potential(c, c->g, pot, s);
-    const int threads = std::min(tile_threads(c), 512);
+    const int threads = vjp_threads(c, n);
     auto kern = threads == 512 ? k_force_vjp_readout<512> : k_force_vjp_readout<256>;
     static bool attr[2] = {false, false};
     if (!attr[threads == 512]) {

@@ -304,7 +304,7 @@ void mlp_backward(pm_ctx* c, double a, cudaStream_t s);
 // Threads of a kernel with one CTA per 16^3 tile: 256, and more where the tiles are too few to
 // fill the SMs with that (64^3: 64 tiles of 1024 threads, 128^3: 512 of 512).  us a launch, 256
 // threads / this: 1070 particles a tile at 64^3, paint 9.3 / 5.8, readout 10.9 / 9.6, re-sort
-// 8.2 / 6.9; 8600 a tile at 128^3, readout of three force meshes 170 / 136.
+// 8.2 / 6.9.
 inline int tile_threads(const pm_ctx* c) { return c->nt <= 4 ? 1024 : (c->nt <= 8 ? 512 : 256); }
 
 #define PM_CUDA_TRY(expr)                      \
