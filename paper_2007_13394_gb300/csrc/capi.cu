@@ -452,9 +452,9 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
   const size_t me = c->g.elems();
   const int64_t nm = std::max<int64_t>(c->n_max, 1);
   const long long hb = (nm + 4095) / 4096;
-  // zeroed words: counts, rs_low, rs_dev, the scan's tile counter, its status (8-byte aligned)
-  const size_t flag_at = 4 * (size_t)(c->nbuckets + 1), scan_at = (flag_at + 3) / 2 * 2;
-  const size_t clear_words = scan_at + 2 * ((3 * (size_t)(c->nbuckets + 1) + kScanTile - 1) / kScanTile);
+  // counts, rs_low and rs_dev (the zeroed words), then the scan's tile sums
+  const size_t flag_at = 4 * (size_t)(c->nbuckets + 1), clear_words = flag_at + 1;
+  const size_t scan_words = (3 * (size_t)(c->nbuckets + 1) + kScanTile - 1) / kScanTile;
   const size_t hist_words = ((size_t)std::min<long long>(hb, kMaxChunks) + 1) << c->radix_bits;
   // flag bit 0, or a 2048^3 mesh: per-component force path with two meshes (at 2048^3 it is
   // also the faster one: reading three 34 GB meshes at once starves the readout)
@@ -463,7 +463,7 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
       dalloc(c, &c->ksq, N) ||
       dalloc(c, &c->winv, N) || dalloc(c, &c->wforce, N) || dalloc(c, &c->kvec0, N) || dalloc(c, &c->sortbuf, 6 * nm) ||
       dalloc(c, &c->us, 3 * nm) || dalloc(c, &c->ps, 3 * nm) || dalloc(c, &c->ids, nm) ||
-      dalloc(c, &c->counts, clear_words) || dalloc(c, &c->bstart, 3 * (c->nbuckets + 1)) ||
+      dalloc(c, &c->counts, clear_words + scan_words) || dalloc(c, &c->bstart, 3 * (c->nbuckets + 1)) ||
       dalloc(c, &c->bprev, 3 * (c->nbuckets + 1)) ||
       dalloc(c, &c->rs_stats, 3) || dalloc(c, &c->hist, hist_words) ||
       dalloc(c, &c->pk_partial, (size_t)N * 2 * 2048) ||
@@ -482,8 +482,7 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
   for (int i = 0; i < 6; ++i) *sorted[i] = c->sortbuf + i * nm;
   c->rs_low = c->counts + 3 * (c->nbuckets + 1);
   c->rs_dev = c->counts + flag_at;
-  c->scan_tile = c->rs_dev + 1;
-  c->scan_status = reinterpret_cast<unsigned long long*>(c->counts + scan_at);
+  c->scan_sums = c->counts + clear_words;
   c->clear_words = clear_words;
   c->digit_totals = c->hist + (hist_words - ((size_t)1 << c->radix_bits));
   cudaMemset(c->rs_stats, 0, 3 * sizeof(long long));

@@ -43,19 +43,6 @@ constexpr int kRadixTile = kRadixThreads * kRadixRounds;  // 4096 keys per tile
 constexpr int kRadixWarps = kRadixThreads / 32;
 constexpr int kCountThreads = 512;
 constexpr int kCountUnroll = 4;
-constexpr int kSpinLimit = 1 << 22;  // look-back polls of the scan before a CTA gives up (PM_ETIMEOUT)
-
-// look-back status word of the scan: state (1 the tile's own sum, 2 the sum up to it) above a
-// 32-bit value; one 64-bit access carries both, so no fence is needed
-__device__ __forceinline__ unsigned long long ld_status(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_status(unsigned long long* p, uint32_t flag, uint32_t value) {
-  const unsigned long long v = ((unsigned long long)flag << 32) | value;
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
 
 // Number of movers of a near-sorted re-sort (every particle when the state was not in
 // bprev's order), from the device: flags of k_kick_drift_keys<true>, scans in bstart3.
@@ -93,58 +80,48 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
   return before;
 }
 
-// Exclusive scan in one launch: tiles of kScanTile words handed out in order, each adds up its
-// predecessors' sums by look-back (a warp reads 32 of them at a time).  status and the tile
-// counter start at 0.
+// Exclusive scan without a wait between CTAs: a launch sums the tiles of kScanTile words, the next
+// one scans each tile behind the sum of the tiles before it, which every CTA adds up itself.  Up to
+// kScanFew tiles (meshes of 128^3 or less) the second launch alone, its CTAs adding up the words
+// before their tile: a launch costs more than they do.  (One launch whose tiles look back at their
+// predecessors' sums, with a bounded wait for them, left the starts unordered when the wait ran
+// out, and the paint reads its particles between two starts.)
 constexpr int kScanThreads = 512;
 constexpr int kScanItems = 8;
-__global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* __restrict__ in, long long n,
-                                                       uint32_t* __restrict__ out,
-                                                       unsigned long long* __restrict__ status,
-                                                       uint32_t* __restrict__ counter, int* __restrict__ err) {
+constexpr int kScanFew = 8;
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const uint32_t* __restrict__ in, long long n,
+                                                            uint32_t* __restrict__ sums) {
   pdl_begin();
-  __shared__ uint32_t ws[32], s_tile, s_before;
+  __shared__ uint32_t ws[32];
+  const long long base = (long long)blockIdx.x * kScanTile + threadIdx.x;
+  uint32_t s = 0, total;
+#pragma unroll
+  for (int k = 0; k < kScanItems; ++k) s += base + k * kScanThreads < n ? in[base + k * kScanThreads] : 0u;
+  block_exclusive_scan(s, ws, &total);
+  if (threadIdx.x == 0) sums[blockIdx.x] = total;
+}
+
+// sums null: few tiles
+__global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* __restrict__ in, long long n,
+                                                       const uint32_t* __restrict__ sums, uint32_t* __restrict__ out) {
+  pdl_begin();
+  __shared__ uint32_t ws[32], wb[32];
   const int t = threadIdx.x;
-  if (t == 0) s_tile = atomicAdd(counter, 1u);
-  __syncthreads();
-  const uint32_t tile = s_tile;
-  const long long base = (long long)tile * kScanTile + (long long)t * kScanItems;
+  const long long base = (long long)blockIdx.x * kScanTile + (long long)t * kScanItems;
   uint32_t v[kScanItems], s = 0;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
     v[k] = (base + k < n) ? in[base + k] : 0u;
     s += v[k];
   }
-  uint32_t total;
-  uint32_t run = block_exclusive_scan(s, ws, &total);
-  if (t == 0) st_status(status + tile, tile == 0 ? 2u : 1u, total);
-  if (t < 32) {  // look-back
-    uint32_t before = 0;
-    int p = (int)tile - 1, spins = 0;
-    while (p >= 0) {
-      const unsigned long long w = p - t >= 0 ? ld_status(status + p - t) : (2ull << 32);
-      const uint32_t st = (uint32_t)(w >> 32);
-      const unsigned incl = __ballot_sync(0xffffffffu, st == 2u), ready = __ballot_sync(0xffffffffu, st != 0u);
-      const int first = incl ? __ffs(incl) - 1 : 31;
-      const unsigned need = first == 31 ? 0xffffffffu : (2u << first) - 1u;
-      if ((ready & need) != need) {
-        if (++spins > kSpinLimit) {
-          if (t == 0) atomicOr(err, 2);
-          break;
-        }
-        continue;
-      }
-      before += __reduce_add_sync(0xffffffffu, t <= first ? (uint32_t)w : 0u);
-      if (incl) break;
-      p -= 32;
-    }
-    if (t == 0) {
-      if (tile != 0) st_status(status + tile, 2u, before + total);
-      s_before = before;
-    }
-  }
-  __syncthreads();
-  run += s_before;
+  const uint32_t* const prev = sums ? sums : in;
+  const int nprev = sums ? blockIdx.x : blockIdx.x * kScanTile;
+  uint32_t b = 0, before;
+#pragma unroll 8
+  for (int i = t; i < nprev; i += kScanThreads) b += prev[i];
+  block_exclusive_scan(b, wb, &before);
+  uint32_t run = block_exclusive_scan(s, ws, nullptr) + before;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
     if (base + k < n) out[base + k] = run;
@@ -805,9 +782,14 @@ int resort_near_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint3
                        cudaStream_t s) {
   const long long nb1 = c->nbuckets + 1;
   {  // bucket starts, stayers' and old keys' movers' starts in one scan
+    const unsigned tiles = (unsigned)((3 * nb1 + kScanTile - 1) / kScanTile);
+    const bool few = tiles <= kScanFew;
+    if (!few) {
+      LaunchScope L(c, s, K_SCAN);
+      pdl_launch(k_scan_sums, tiles, kScanThreads, 0, s, c->counts, 3 * nb1, c->scan_sums);
+    }
     LaunchScope L(c, s, K_SCAN);
-    pdl_launch(k_scan, (unsigned)((3 * nb1 + kScanTile - 1) / kScanTile), kScanThreads, 0, s, 
-        c->counts, 3 * nb1, c->bstart, c->scan_status, c->scan_tile, c->err_dev);
+    pdl_launch(k_scan, tiles, kScanThreads, 0, s, c->counts, 3 * nb1, few ? nullptr : c->scan_sums, c->bstart);
   }
   // the movers' records go to the second mesh, free during a step, when they fit (32 bytes a
   // mover: up to 2^30 movers at 2048^3); else the placement gathers from the state itself

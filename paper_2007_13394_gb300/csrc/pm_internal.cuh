@@ -136,14 +136,13 @@ struct pm_ctx {
   // step left its state in (valid for rs_n particles, -1: none).
   uint32_t* bprev = nullptr;
   int64_t rs_n = -1;
-  // one allocation, zeroed (clear_words) before each drift that counts: counts, rs_low,
-  // rs_dev, the scan's tile counter and status words
+  // one allocation: counts, rs_low and rs_dev, zeroed (clear_words) before each drift that
+  // counts, then the scan's tile sums
   uint32_t* counts = nullptr;     // 3 (nbuckets + 1)
   size_t clear_words = 0;
   uint32_t* rs_low = nullptr;     // movers from a lower old key, per new key (nbuckets + 1)
   uint32_t* rs_dev = nullptr;     // flag bits of k_kick_drift_keys<true>
-  unsigned long long* scan_status = nullptr;
-  uint32_t* scan_tile = nullptr;
+  uint32_t* scan_sums = nullptr;
   uint32_t* rs_k2 = nullptr;      // second (key, index) buffer pair of the movers' radix
   uint32_t* rs_v2 = nullptr;
   long long* rs_stats = nullptr;  // device: re-sorts near-sorted, from scratch, movers of the last near-sorted one
