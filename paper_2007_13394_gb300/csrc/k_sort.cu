@@ -523,7 +523,9 @@ __global__ void __launch_bounds__(NT) k_resort_old_tiles(
   }
   const int64_t nm = movers_of(flags, bstart3, nb1, n);
   if (nm > stage_room) stage = nullptr;
-  if (t < 9) cls_lo[t] = bprev[8 * O + t];
+  // (bprev may be of more particles: a captured step replayed after another call has sorted into
+  // its array, the state's n being the first of those in order)
+  if (t < 9) cls_lo[t] = min(bprev[8 * O + t], (uint32_t)n);
   __syncthreads();
   const uint32_t lo = cls_lo[0], hi = cls_lo[8];
   if (lo == hi) return;
