@@ -46,10 +46,13 @@ constexpr int kCountUnroll = 4;
 
 // Number of movers of a near-sorted re-sort (every particle when the state was not in
 // bprev's order), from the device: flags of k_kick_drift_keys<true>, scans in bstart3.
-__device__ __forceinline__ int64_t movers_of(const uint32_t* flags, const uint32_t* bstart3, long long nb1, int64_t n) {
+// Counts that are not those of n particles give more than n: err is set (by the caller that has it).
+__device__ __forceinline__ int64_t movers_of(const uint32_t* flags, const uint32_t* bstart3, long long nb1, int64_t n,
+                                             int* err = nullptr) {
   if (*flags & 1u) return n;
-  const int64_t m = (int64_t)bstart3[3 * nb1 - 1] - (int64_t)bstart3[2 * nb1];
-  return m < 0 ? 0 : (m > n ? n : m);
+  const int64_t m = scan_difference(bstart3[2 * nb1], bstart3[3 * nb1 - 1]);
+  if (m > n && err) atomicOr(err, 1);
+  return m > n ? n : m;
 }
 
 // ------------------------------------------------------------------ scan
@@ -656,7 +659,7 @@ __global__ void k_place_movers(const uint32_t* __restrict__ mk, const uint32_t* 
                                const uint4* __restrict__ stage, int64_t stage_room, long long* __restrict__ stats) {
   pdl_begin();
   const bool all = (*flags & 1u) != 0u;
-  const int64_t nm = movers_of(flags, bstart3, nb1, n);
+  const int64_t nm = movers_of(flags, bstart3, nb1, n, err);
   if (all || nm > stage_room) stage = nullptr;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     stats[all ? 1 : 0] += 1;

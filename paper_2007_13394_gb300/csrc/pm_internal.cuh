@@ -344,6 +344,11 @@ void pdl_launch(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, 
 }
 
 // ---------------------------------------------------------------- device helpers
+// Particles counted between two words of the re-sort's scan.  The scan counts every particle
+// twice, so from 2^31 particles on its words wrap; the number between two of them is below 2^32
+// and comes out of the 32-bit difference all the same.
+__host__ __device__ constexpr uint32_t scan_difference(uint32_t lo, uint32_t hi) { return hi - lo; }
+
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
