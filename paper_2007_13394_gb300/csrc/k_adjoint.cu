@@ -691,11 +691,8 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
       const int threads = vjp_threads(c, n);
       auto read1 = threads == 512 ? k_vjp_readout<1, 512> : k_vjp_readout<1, 256>;
       auto read3 = threads == 512 ? k_vjp_readout<3, 512> : k_vjp_readout<3, 256>;
-      static bool attr3[2] = {false, false};
-      if (!attr3[threads == 512]) {
-        cudaFuncSetAttribute(read3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(3 * sm1));
-        attr3[threads == 512] = true;
-      }
+      static DeviceOnce once3[2];
+      allow_smem(once3[threads == 512], (const void*)read3, 3 * sm1);
       const unsigned tiles = (unsigned)(c->nt * c->nt * c->nt);
       float* const tmp = c->adj + 6 * 3 * n;  // the second term, sorted order
       {
@@ -721,11 +718,8 @@ int force_vjp(pm_ctx* c, const uint32_t* u, const uint32_t* id, int64_t n, const
     fft_potential(c, c->g, pot, s);
     const int threads = vjp_threads(c, n);
     auto kern = threads == 512 ? k_force_vjp_readout<512> : k_force_vjp_readout<256>;
-    static bool attr[2] = {false, false};
-    if (!attr[threads == 512]) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVjpSmem);
-      attr[threads == 512] = true;
-    }
+    static DeviceOnce once[2];
+    allow_smem(once[threads == 512], (const void*)kern, kVjpSmem);
     {
       LaunchScope L(c, s, K_ADJOINT);
       pdl_launch(kern, (unsigned)(c->nt * c->nt * c->nt), threads, kVjpSmem, s, 

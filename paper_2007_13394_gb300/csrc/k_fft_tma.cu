@@ -239,14 +239,17 @@ int launch(pm_ctx* c, const CUtensorMap* map, float2* d0, float2* d1, float2* d2
   constexpr bool GREEN = MODE == MODE_FUSED;  // reads the window
   const int w = (GREEN && kt.winv) ? 1 : 0;
   auto kern = w ? k_fft_strided_tma<LOGM, TK, INV, MODE, GREEN> : k_fft_strided_tma<LOGM, TK, INV, MODE, false>;
-  static int blocks_per_sm[2] = {0, 0};
-  if (blocks_per_sm[w] == 0) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM) != cudaSuccess)
-      return PM_ECUDA;
+  static DeviceOnce once[2];
+  static std::atomic<int> blocks_per_sm[2];  // of the device seen last; 0: not asked yet, or refused
+  once[w].run(c->device, [&] {
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, SH::THREADS, SH::SMEM);
-    blocks_per_sm[w] = b > 0 ? b : 1;
-  }
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, SH::THREADS, SH::SMEM) != cudaSuccess)
+      b = 0;
+    blocks_per_sm[w] = b;
+    return b > 0;
+  });
+  if (blocks_per_sm[w] == 0) return PM_ECUDA;
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   const int ntz = (M / 2 + 1 + TK - 1) / TK;

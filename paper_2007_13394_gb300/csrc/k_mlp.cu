@@ -360,11 +360,8 @@ void mlp_green_apply(pm_ctx* c, const float2* rho_k, float2* phi_k, cudaStream_t
 
 void mlp_backward(pm_ctx* c, double a, cudaStream_t s) {
   if (!c->mlp_on) return;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BW_SMEM);
-    attr = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, (const void*)k_mlp_backward, BW_SMEM);
   LaunchScope L(c, s, K_MLP_BACKWARD);
   pdl_launch(k_mlp_backward, nblocks(c->mlp_ntab, CH), BW_THREADS, BW_SMEM, s, 
       c->mlp_theta, (float)a, 2.0f / (float)c->g.n, c->mlp_ntab, c->mlp_gbin, c->mlp_dtheta);

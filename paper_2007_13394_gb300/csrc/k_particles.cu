@@ -780,11 +780,8 @@ void paint_tiles(pm_ctx* c, const uint32_t* us, const uint32_t* ids, int64_t n, 
 
 void paint_weights3(pm_ctx* c, const uint32_t* us, int64_t n, const float* weights, float* m0, float* m1, float* m2,
                     int row_pitch, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_paint_weights3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPaint3Smem);
-    attr = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, (const void*)k_paint_weights3, kPaint3Smem);
   LaunchScope L(c, s, K_PAINT);
   pdl_launch(k_paint_weights3, (unsigned)(c->nt * c->nt * c->nt), kPaint3Threads, kPaint3Smem, s, 
       us, n, c->bstart, m0, m1, m2, c->g.n, 32 - c->g.logn, c->ntl, row_pitch, c->err_dev, weights);
@@ -833,11 +830,8 @@ void readout_fd4_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint
        k_readout_fd4_kick<true, true, kNodeThreads>}};
   const auto kern = kerns[dn != nullptr][v];
   const size_t smem = nodes ? kNodeSmem : kFd4Smem;
-  static bool attr[2][3] = {};
-  if (!attr[dn != nullptr][v]) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr[dn != nullptr][v] = true;
-  }
+  static DeviceOnce once[2][3];
+  allow_smem(once[dn != nullptr][v], (const void*)kern, smem);
   pdl_launch(kern, grid, threads, smem, s, us, ps, ids, n, c->bstart, phi, c->g.n, 32 - c->g.logn,
                                                              c->ntl, row_pitch, inv12h, K, p_out, f_out, u_out, id_out,
                                                              dn ? nullptr : perm_scatter, c->err_dev,

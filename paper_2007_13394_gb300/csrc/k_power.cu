@@ -296,11 +296,8 @@ int power_bin(pm_ctx* c, const float2* da, const float2* db, int nbins, double* 
   const PowerPlan p = power_plan(c, nbins);
   const size_t smem = sizeof(double) * kPowWarps * nbins;
   auto kern = da == db ? k_power_bin<false> : k_power_bin<true>;
-  static bool attr[2] = {false, false};
-  if (!attr[da == db]) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * kPowWarps * kMaxBins));
-    attr[da == db] = true;
-  }
+  static DeviceOnce once[2];
+  allow_smem(once[da == db], (const void*)kern, sizeof(double) * kPowWarps * kMaxBins);
   PM_CUDA_TRY(cudaMemsetAsync(p.r2, 0, sizeof(uint32_t) * (p.tmax + 1), s));
   {
     LaunchScope L(c, s, K_POWER_BIN);

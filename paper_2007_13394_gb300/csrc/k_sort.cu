@@ -683,11 +683,8 @@ void launch_scatter(pm_ctx* c, const uint32_t* kin, const uint32_t* vin, int64_t
   const size_t dyn = 2 * kRadixTile * sizeof(uint32_t);
   const bool raw = raw_counts(n);
   auto kern = raw ? k_radix_scatter<BITS, true> : k_radix_scatter<BITS, false>;
-  static bool attr[2] = {false, false};
-  if (!attr[raw]) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    attr[raw] = true;
-  }
+  static DeviceOnce once[2];
+  allow_smem(once[raw], (const void*)kern, dyn);
   pdl_launch(kern, chunks_of(n), kRadixThreads, dyn, s, kin, vin, n, shift, c->hist, c->digit_totals, kout, vout, flags,
                                                 c->bstart, c->nbuckets + 1);
 }
@@ -812,14 +809,13 @@ int resort_near_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint3
   uint32_t* const vb[2] = {c->vals[1], c->rs_v2};
   const int r = radix_passes(c, kb, vb, false, false, n, c->rs_dev, s);
   LaunchScope L(c, s, K_RESORT_MISC);
-  static int full = 0;  // grid-stride: the CTAs that fill the GPU once
-  if (full == 0) {
+  if (c->place_ctas == 0) {  // grid-stride: the CTAs that fill the GPU once
     int per_sm = 0, sms = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_place_movers, 256, 0);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    full = std::max(per_sm, 1) * std::max(sms, 1);
+    c->place_ctas = (unsigned)(std::max(per_sm, 1) * std::max(sms, 1));
   }
-  pdl_launch(k_place_movers, (unsigned)std::min<int64_t>(full, (n + 255) / 256), 256, 0, s, 
+  pdl_launch(k_place_movers, (unsigned)std::min<int64_t>(c->place_ctas, (n + 255) / 256), 256, 0, s, 
       kb[r], vb[r], u, p, id, n, c->bstart, nb1, c->nbuckets, c->rs_low, c->us, c->ps, c->ids, c->rs_dev, c->err_dev,
       stage, room, c->rs_stats);
   return PM_OK;

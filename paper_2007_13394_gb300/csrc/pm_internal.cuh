@@ -12,6 +12,7 @@
 
 #include "../../include/pm.h"
 #include "cosmo.h"
+#include "device_once.h"
 
 namespace pmnu {
 
@@ -147,6 +148,7 @@ struct pm_ctx {
   uint32_t* rs_v2 = nullptr;
   long long* rs_stats = nullptr;  // device: re-sorts near-sorted, from scratch, movers of the last near-sorted one
   int64_t rs_full = 0;            // re-sorts that the host sent to the sort from scratch
+  unsigned place_ctas = 0;        // CTAs of the movers' placement that fill this context's device
   uint32_t* hist = nullptr;       // digit counts per chunk of a radix pass, then the digits' totals
   uint32_t* digit_totals = nullptr;
   // masses
@@ -305,6 +307,16 @@ void mlp_backward(pm_ctx* c, double a, cudaStream_t s);
 // threads / this: 1070 particles a tile at 64^3, paint 9.3 / 5.8, readout 10.9 / 9.6, re-sort
 // 8.2 / 6.9.
 inline int tile_threads(const pm_ctx* c) { return c->nt <= 4 ? 1024 : (c->nt <= 8 ? 512 : 256); }
+
+// More than 48 KB of dynamic shared memory has to be allowed for each kernel on each device, not
+// once a process: contexts may live on several devices.
+inline void allow_smem(DeviceOnce& once, const void* kern, size_t bytes) {
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess) return;  // the launch reports it
+  once.run(device, [&] {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+  });
+}
 
 #define PM_CUDA_TRY(expr)                      \
   do {                                         \
