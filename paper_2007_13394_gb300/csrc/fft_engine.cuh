@@ -367,6 +367,7 @@ struct KTables {
   const float* winv;   // per-axis factor of the Green's function, 1 / sinc^4(pi n_s / N) for the
                        // deconvolved spectral kernel; null: all factors 1 (the default kernel)
   const float* kvec0;  // gradient kernel D(k_n), 0 on the Nyquist index
+  float kf2_lo;        // k_F^2 minus ksq[1]: the two words together carry 48 bits
   float gcoef;         // -1.5 Omega_m0 / N^3
   const float* mtab;   // learned factor by |n|^2 (n signed indices), null: plain kernel
 };
