@@ -32,11 +32,11 @@ namespace {
 
 // out[d][perm[i]] (+)= sum_j a_j(i) d/dx_d R[M_j](x_i) for the sorted particle i.
 // a_j(i) = wts[j * n + i] when wts is set, else the particle's mass.
-__global__ void k_readout_grad(const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids,
-                               int64_t n, const float* __restrict__ m0, const float* __restrict__ m1,
-                               const float* __restrict__ m2, int nmesh_used, int nm, int shift,
-                               int row_pitch, float inv_h, const float* __restrict__ wts, MassTable mt,
-                               const uint32_t* __restrict__ perm, float* __restrict__ out,
+__global__ void k_readout_grad(const uint32_t* us, const uint32_t* ids,
+                               int64_t n, const float* m0, const float* m1,
+                               const float* m2, int nmesh_used, int nm, int shift,
+                               int row_pitch, float inv_h, const float* wts, MassTable mt,
+                               const uint32_t* perm, float* __restrict__ out,
                                int accumulate, int species) {
   pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -59,10 +59,10 @@ __global__ void k_readout_grad(const uint32_t* __restrict__ us, const uint32_t* 
     const float* M = ms[j];
     const float a = wts ? wts[(int64_t)j * n + i] : mass;
     if (a == 0.0f) continue;
-    const float v000 = __ldg(M + r00 + cz), v001 = __ldg(M + r00 + cz1);
-    const float v010 = __ldg(M + r01 + cz), v011 = __ldg(M + r01 + cz1);
-    const float v100 = __ldg(M + r10 + cz), v101 = __ldg(M + r10 + cz1);
-    const float v110 = __ldg(M + r11 + cz), v111 = __ldg(M + r11 + cz1);
+    const float v000 = M[r00 + cz], v001 = M[r00 + cz1];
+    const float v010 = M[r01 + cz], v011 = M[r01 + cz1];
+    const float v100 = M[r10 + cz], v101 = M[r10 + cz1];
+    const float v110 = M[r11 + cz], v111 = M[r11 + cz1];
     // d/dx: (x1 plane - x0 plane) weighted in y, z; likewise for y and z
     const float dX = gy * (gz * (v100 - v000) + fz * (v101 - v001)) +
                      fy * (gz * (v110 - v010) + fz * (v111 - v011));
@@ -89,10 +89,10 @@ __global__ void k_readout_grad(const uint32_t* __restrict__ us, const uint32_t* 
 // of -G_j (D the gradient kernel); m = 1 without the learned factor.  With rho (the
 // density's half spectrum) it also bins d <lambda_F, F> / d m(k) =
 // Re[(-i D(k_j)) g rho_k conj(A_k)] (twice for 0 < k_z < N/2) by s = |n|^2 into gbin.
-__global__ void k_adj_combine(const float2* __restrict__ a, float2* __restrict__ b, int nm, int pc,
+__global__ void k_adj_combine(const float2* a, float2* __restrict__ b, int nm, int pc,
                               const float* __restrict__ ksq, const float* __restrict__ winv,
                               const float* __restrict__ kvec0, float gcoef, int comp, int accumulate,
-                              const float* __restrict__ mtab, const float2* __restrict__ rho,
+                              const float* mtab, const float2* rho,
                               double* __restrict__ gbin) {
   pdl_begin();
   const int x = blockIdx.x / nm, y = blockIdx.x % nm;
@@ -154,9 +154,9 @@ constexpr size_t kVjpSmem = sizeof(float) * (kVjpSpanXY * kVjpSX + kVjpSpanB * k
 
 template <int NT>
 __global__ void __launch_bounds__(NT) k_force_vjp_readout(
-    const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n, const uint32_t* __restrict__ bstart,
-    const float* __restrict__ phi, const float* __restrict__ B, int nm, int shift, int ntl, int row_pitch,
-    float inv12h, float inv_h, const float* __restrict__ lam, MassTable mt, const uint32_t* __restrict__ perm,
+    const uint32_t* us, const uint32_t* ids, int64_t n, const uint32_t* bstart,
+    const float* phi, const float* B, int nm, int shift, int ntl, int row_pitch,
+    float inv12h, float inv_h, const float* lam, MassTable mt, const uint32_t* perm,
     float* __restrict__ out, int* __restrict__ err) {
   pdl_begin();
   extern __shared__ __align__(16) float sp[];
@@ -259,10 +259,10 @@ __global__ void __launch_bounds__(NT) k_force_vjp_readout(
 // d/dx_d R[F_j](x_i).  Staging replaces 8 NM scattered global reads a particle.
 template <int NM, int NT>
 __global__ void __launch_bounds__(NT) k_vjp_readout(
-    const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n, const uint32_t* __restrict__ bstart,
-    const float* __restrict__ m0, const float* __restrict__ m1, const float* __restrict__ m2, int nm, int shift,
-    int ntl, int row_pitch, float inv_h, const float* __restrict__ lam, MassTable mt,
-    const uint32_t* __restrict__ perm, float* __restrict__ tmp, float* __restrict__ out, int species,
+    const uint32_t* us, const uint32_t* ids, int64_t n, const uint32_t* bstart,
+    const float* m0, const float* m1, const float* m2, int nm, int shift,
+    int ntl, int row_pitch, float inv_h, const float* lam, MassTable mt,
+    const uint32_t* perm, float* __restrict__ tmp, float* __restrict__ out, int species,
     int* __restrict__ err) {
   pdl_begin();
   extern __shared__ __align__(16) float sb[];
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(NT) k_vjp_readout(
 // three meshes: three single-axis passes that add into one mesh took 307 us at 256^3.
 constexpr int kDivThreads = 256;
 constexpr int kDivSteps = 8;
-__global__ void __launch_bounds__(kDivThreads) k_stencil_div(const float* __restrict__ A, const float* __restrict__ B,
+__global__ void __launch_bounds__(kDivThreads) k_stencil_div(const float* A, const float* B,
                                                              float* C, int nm, int rp, float inv12h) {
   pdl_begin();
   const int quads = nm / 4, rows = kDivThreads / quads;  // rows of z quads a CTA (nm <= 1024)
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kDivThreads) k_stencil_div(const float* __rest
 // The same divergence from the three half spectra, C <- i (D_x A + D_y B + D_z C): the learned
 // path's form.  The factor's gradient weighs the largest scales by 1 / k^2, and there the
 // transform of the real-space divergence has lost digits to its smallest scales.
-__global__ void __launch_bounds__(256) k_spectrum_div(const float2* __restrict__ A, const float2* __restrict__ B,
+__global__ void __launch_bounds__(256) k_spectrum_div(const float2* A, const float2* B,
                                                       float2* __restrict__ C, int nm, int pc,
                                                       const float* __restrict__ kvec0) {
   pdl_begin();
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(256) k_spectrum_div(const float2* __restrict__
 __global__ void __launch_bounds__(256) k_vjp_combine(float2* __restrict__ rho, float2* __restrict__ C, int nm, int pc,
                                                      int units, const float* __restrict__ ksq,
                                                      const float* __restrict__ winv, float gcoef,
-                                                     const float* __restrict__ mtab, double* __restrict__ gbin) {
+                                                     const float* mtab, double* __restrict__ gbin) {
   pdl_begin();
   const int wu = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31, half = nm / 2;
   if (wu >= units) return;
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(256) k_vjp_combine(float2* __restrict__ rho, f
 }
 
 // B (+)= S_j A on real meshes (row pitch rp): the 4-point stencil along axis j, periodic.
-__global__ void k_stencil_axis(const float* __restrict__ A, float* __restrict__ B, int nm, int rp, int axis,
+__global__ void k_stencil_axis(const float* A, float* __restrict__ B, int nm, int rp, int axis,
                                float inv12h, int accumulate) {
   pdl_begin();
   const int x = blockIdx.x / nm, y = blockIdx.x % nm;
@@ -445,9 +445,9 @@ __global__ void k_stencil_axis(const float* __restrict__ A, float* __restrict__ 
   const size_t row = ((size_t)x * nm + y) * rp;
   for (int z = threadIdx.x; z < nm; z += blockDim.x) {
     auto at = [&](int o) -> float {  // A at offset o along the axis
-      if (axis == 0) return __ldg(A + ((size_t)((x + o) & w) * nm + y) * rp + z);
-      if (axis == 1) return __ldg(A + ((size_t)x * nm + ((y + o) & w)) * rp + z);
-      return __ldg(A + row + ((z + o) & w));
+      if (axis == 0) return A[((size_t)((x + o) & w) * nm + y) * rp + z];
+      if (axis == 1) return A[((size_t)x * nm + ((y + o) & w)) * rp + z];
+      return A[row + ((z + o) & w)];
     };
     const float v = inv12h * (8.0f * (at(1) - at(-1)) - (at(2) - at(-2)));
     B[row + z] = accumulate ? B[row + z] + v : v;
@@ -456,28 +456,35 @@ __global__ void k_stencil_axis(const float* __restrict__ A, float* __restrict__ 
 
 // Start of a step's VJP, in state order: the cotangents by id, the drifted positions
 // u1 = u0 + rne(Delta (p0 + K1 f0) 2^32 / L) and the force cotangent K2 lambda_p of x1.
-__global__ void k_vjp_begin(const float* __restrict__ lx1, const float* __restrict__ lp1,
-                            const uint32_t* __restrict__ id, const uint32_t* __restrict__ u0,
-                            const float* __restrict__ p0, const float* __restrict__ f0, int64_t n, float K1,
+__global__ void k_vjp_begin(const float* lx1, const float* lp1,
+                            const uint32_t* id, const uint32_t* u0,
+                            const float* p0, const float* f0, int64_t n, float K1,
                             float dscale, float K2, float* __restrict__ Lx, float* __restrict__ Lp,
                             float* __restrict__ lamF, uint32_t* __restrict__ u1) {
   pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t j = (int64_t)id[i];
+  float lx[3], lp[3], ph[3];  // every load before the first store
+  uint32_t uq[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const float lp = lp1[d * n + j];
-    Lx[d * n + i] = lx1[d * n + j];
-    Lp[d * n + i] = lp;
-    lamF[d * n + i] = K2 * lp;
-    const float ph = p0[d * n + i] + K1 * f0[d * n + i];
-    u1[d * n + i] = u0[d * n + i] + (uint32_t)(unsigned long long)__float2ll_rn(dscale * ph);
+    lx[d] = lx1[d * n + j];
+    lp[d] = lp1[d * n + j];
+    ph[d] = p0[d * n + i] + K1 * f0[d * n + i];
+    uq[d] = u0[d * n + i];
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    Lx[d * n + i] = lx[d];
+    Lp[d * n + i] = lp[d];
+    lamF[d * n + i] = K2 * lp[d];
+    u1[d * n + i] = uq[d] + (uint32_t)(unsigned long long)__float2ll_rn(dscale * ph[d]);
   }
 }
 
 // Between the two force VJPs, over 3n: Lx += g, Lp += Delta Lx, lamF = K1 Lp.
-__global__ void k_vjp_middle(const float* __restrict__ g, int64_t m, float delta, float K1, float* __restrict__ Lx,
+__global__ void k_vjp_middle(const float* g, int64_t m, float delta, float K1, float* __restrict__ Lx,
                              float* __restrict__ Lp, float* __restrict__ lamF) {
   pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -489,22 +496,28 @@ __global__ void k_vjp_middle(const float* __restrict__ g, int64_t m, float delta
 }
 
 // End: lx0 = Lx + g and lp0 = Lp in canonical order.
-__global__ void k_vjp_end(const float* __restrict__ g, const float* __restrict__ Lx, const float* __restrict__ Lp,
-                          const uint32_t* __restrict__ id, int64_t n, float* __restrict__ lx0,
+__global__ void k_vjp_end(const float* g, const float* Lx, const float* Lp,
+                          const uint32_t* id, int64_t n, float* __restrict__ lx0,
                           float* __restrict__ lp0) {
   pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t j = (int64_t)id[i];
+  float x[3], p[3];  // every load before the first store
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    lx0[d * n + j] = Lx[d * n + i] + g[d * n + i];
-    lp0[d * n + j] = Lp[d * n + i];
+    x[d] = Lx[d * n + i] + g[d * n + i];
+    p[d] = Lp[d * n + i];
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    lx0[d * n + j] = x[d];
+    lp0[d * n + j] = p[d];
   }
 }
 
 // gather weights into the sorted order: ws[k] = w[perm[k]]
-__global__ void k_gather_weights(const float* __restrict__ w, const uint32_t* __restrict__ perm, int64_t n,
+__global__ void k_gather_weights(const float* w, const uint32_t* perm, int64_t n,
                                  float* __restrict__ ws) {
   pdl_begin();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -512,7 +525,7 @@ __global__ void k_gather_weights(const float* __restrict__ w, const uint32_t* __
 }
 
 // IC transpose: lattice mesh (padded real, nc) of lambda_s for CDM nodes (canonical order)
-__global__ void k_icadj_cdm(const float* __restrict__ lx, const float* __restrict__ lp, int nc,
+__global__ void k_icadj_cdm(const float* lx, const float* lp, int nc,
                             int rp, int comp, float D0, float gp0, int64_t n_total,
                             float* __restrict__ mesh) {
   pdl_begin();
@@ -525,7 +538,7 @@ __global__ void k_icadj_cdm(const float* __restrict__ lx, const float* __restric
 }
 
 // neutrino sites: sum of lambda_s over the site's shell x direction particles
-__global__ void k_icadj_nu(const float* __restrict__ lx, const float* __restrict__ lp, int nc,
+__global__ void k_icadj_nu(const float* lx, const float* lp, int nc,
                            int rp, int comp, float D0, float gp0, int nsites, int stride, int j0,
                            int per_site, int64_t n_offset, int64_t n_total, float* __restrict__ mesh) {
   pdl_begin();
@@ -545,7 +558,7 @@ __global__ void k_icadj_nu(const float* __restrict__ lx, const float* __restrict
 
 // K (+)= conj(S_j) A_k with S_j = i f e^{i theta}, f = amp(|n|^2) n_j / |n|^2 (the forward
 // ZA multiplier of k_ic_za), theta = pi (n_x + n_y + n_z) / nc for shifted sites.
-__global__ void k_icadj_kspace(const float2* __restrict__ a, float2* __restrict__ kacc, int nc, int pc,
+__global__ void k_icadj_kspace(const float2* a, float2* __restrict__ kacc, int nc, int pc,
                                const float* __restrict__ amp, int comp, int phase_shift,
                                int accumulate) {
   pdl_begin();

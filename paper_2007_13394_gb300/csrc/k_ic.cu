@@ -19,7 +19,7 @@ namespace pmnu {
 
 namespace {
 
-__global__ void k_ic_za(const float2* __restrict__ wk, float2* __restrict__ sk, int nc, int pc,
+__global__ void k_ic_za(const float2* wk, float2* __restrict__ sk, int nc, int pc,
                         const float* __restrict__ amp, int comp, int phase_shift) {
   pdl_begin();
   const int x = blockIdx.x / nc, y = blockIdx.x % nc;
@@ -45,7 +45,7 @@ __global__ void k_ic_za(const float2* __restrict__ wk, float2* __restrict__ sk, 
   }
 }
 
-__global__ void k_ic_cdm(const float* __restrict__ s, int nc, int rp, int comp, double cell,
+__global__ void k_ic_cdm(const float* s, int nc, int rp, int comp, double cell,
                          double D0, double gp0, double to_fix, int64_t n_offset,
                          uint32_t* __restrict__ u, float* __restrict__ p, int64_t n_total) {
   pdl_begin();
@@ -61,7 +61,7 @@ __global__ void k_ic_cdm(const float* __restrict__ s, int nc, int rp, int comp, 
   p[comp * n_total + n_offset + i] = (float)(gp0 * (double)sv);
 }
 
-__global__ void k_ic_nu(const float* __restrict__ s, int nc, int rp, int comp, int nsites,
+__global__ void k_ic_nu(const float* s, int nc, int rp, int comp, int nsites,
                         int stride, int j0, double site_dx, double site_off, double D0, double gp0,
                         double to_fix, int nshell, int ndir, const double* __restrict__ tab,
                         int64_t n_offset, int64_t n_nu, uint32_t* __restrict__ u,
@@ -89,10 +89,10 @@ __global__ void k_ic_nu(const float* __restrict__ s, int nc, int rp, int comp, i
 // Pseudo-random sampling: one particle per site, no shell offset, thermal momentum of
 // speed q = F^-1(u_0) (F tabulated at nF equally spaced q; bisection, then linear
 // interpolation inside the bracket) along cos(theta) = 2 u_1 - 1, phi = 2 pi u_2.
-__global__ void k_ic_nu_pseudo(const float* __restrict__ s, int nc, int rp, int comp, int nsites,
+__global__ void k_ic_nu_pseudo(const float* s, int nc, int rp, int comp, int nsites,
                                int stride, int j0, double site_dx, double site_off, double D0,
-                               double gp0, double to_fix, double pscale, const double* __restrict__ F,
-                               int nF, double dq, const float* __restrict__ uni, int64_t n_offset,
+                               double gp0, double to_fix, double pscale, const double* F,
+                               int nF, double dq, const float* uni, int64_t n_offset,
                                int64_t n_nu, uint32_t* __restrict__ u, float* __restrict__ p,
                                int64_t n_total) {
   pdl_begin();

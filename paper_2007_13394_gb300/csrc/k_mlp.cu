@@ -57,13 +57,13 @@ __device__ float mlp_m(const float* __restrict__ th, float kappa, float a) {
   return 1.0f + out;
 }
 
-__device__ __forceinline__ void load_theta(const float* __restrict__ theta, float* th) {
+__device__ __forceinline__ void load_theta(const float* theta, float* th) {
   for (int i = threadIdx.x; i < NP; i += blockDim.x) th[i] = theta[i];
   __syncthreads();
 }
 
 // tab[s] = m(sqrt(s) / (N/2), a)
-__global__ void __launch_bounds__(256) k_mlp_table(const float* __restrict__ theta, float a, float inv_half,
+__global__ void __launch_bounds__(256) k_mlp_table(const float* theta, float a, float inv_half,
                                                    int64_t ntab, float* __restrict__ tab) {
   pdl_begin();
   __shared__ __align__(16) float th[NP + 3];
@@ -74,8 +74,8 @@ __global__ void __launch_bounds__(256) k_mlp_table(const float* __restrict__ the
 }
 
 // out[i] = m(kappa[i], a[i])
-__global__ void __launch_bounds__(256) k_mlp_eval(const float* __restrict__ theta, const float* __restrict__ kappa,
-                                                  const float* __restrict__ av, int64_t n, float* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_mlp_eval(const float* theta, const float* kappa,
+                                                  const float* av, int64_t n, float* __restrict__ out) {
   pdl_begin();
   __shared__ __align__(16) float th[NP + 3];
   load_theta(theta, th);
@@ -84,9 +84,9 @@ __global__ void __launch_bounds__(256) k_mlp_eval(const float* __restrict__ thet
 }
 
 // phi = c(k) m(|n|^2) rho on the half spectrum of the force mesh (padded pitch pc)
-__global__ void k_green_apply(const float2* __restrict__ rho, float2* __restrict__ phi, int nm, int pc,
+__global__ void k_green_apply(const float2* rho, float2* __restrict__ phi, int nm, int pc,
                               const float* __restrict__ ksq, const float* __restrict__ winv, float gcoef,
-                              const float* __restrict__ mtab) {
+                              const float* mtab) {
   pdl_begin();
   const int x = blockIdx.x / nm, y = blockIdx.x % nm;
   const int nx = x < nm / 2 ? x : x - nm, ny = y < nm / 2 ? y : y - nm;
@@ -110,7 +110,7 @@ constexpr int HP = H + 1;
 constexpr int BW_THREADS = 256;
 constexpr size_t BW_SMEM = sizeof(float) * ((NP + 3) + 4 * CH * HP + 2 * CH);
 
-__global__ void __launch_bounds__(BW_THREADS) k_mlp_backward(const float* __restrict__ theta, float a,
+__global__ void __launch_bounds__(BW_THREADS) k_mlp_backward(const float* theta, float a,
                                                              float inv_half, int64_t ntab,
                                                              double* __restrict__ gbin,
                                                              double* __restrict__ dtheta) {
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(BW_THREADS) k_mlp_backward(const float* __rest
 }
 
 // Adam with bias corrections bc1 = 1 - beta1^t, bc2 = 1 - beta2^t
-__global__ void k_adam(float* __restrict__ theta, const float* __restrict__ grad, float* __restrict__ m,
+__global__ void k_adam(float* __restrict__ theta, const float* grad, float* __restrict__ m,
                        float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float bc1,
                        float bc2) {
   pdl_begin();
@@ -218,7 +218,7 @@ __global__ void k_adam(float* __restrict__ theta, const float* __restrict__ grad
   theta[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
 }
 
-__global__ void k_grad_out(const double* __restrict__ acc, float* __restrict__ out, int n, int reset,
+__global__ void k_grad_out(const double* acc, float* __restrict__ out, int n, int reset,
                            double* __restrict__ acc_w) {
   pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -228,7 +228,7 @@ __global__ void k_grad_out(const double* __restrict__ acc, float* __restrict__ o
 }
 
 // ref_c[d][id_ref[i]] = u_ref[d][i]
-__global__ void k_ref_canonical(const uint32_t* __restrict__ u_ref, const uint32_t* __restrict__ id_ref,
+__global__ void k_ref_canonical(const uint32_t* u_ref, const uint32_t* id_ref,
                                 int64_t n, uint32_t* __restrict__ ref_c, int* __restrict__ err) {
   pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -255,7 +255,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 }
 
 // sum of the particle masses
-__global__ void k_mass_sum(const uint32_t* __restrict__ id, int64_t n, MassTable mt, int species,
+__global__ void k_mass_sum(const uint32_t* id, int64_t n, MassTable mt, int species,
                            double* __restrict__ out, int* __restrict__ err) {
   pdl_begin();
   __shared__ double red[32];
@@ -271,9 +271,9 @@ __global__ void k_mass_sum(const uint32_t* __restrict__ id, int64_t n, MassTable
 }
 
 // L += m_i |d_i|^2 / W, lam[d][id_i] = 2 m_i d_i / W, d_i = int32(u_i - ref_c[id_i]) L / 2^32
-__global__ void k_disp_loss(const uint32_t* __restrict__ u, const uint32_t* __restrict__ id, int64_t n,
-                            const uint32_t* __restrict__ ref_c, MassTable mt, int species, float scale,
-                            const double* __restrict__ wsum, float* __restrict__ lam,
+__global__ void k_disp_loss(const uint32_t* u, const uint32_t* id, int64_t n,
+                            const uint32_t* ref_c, MassTable mt, int species, float scale,
+                            const double* wsum, float* __restrict__ lam,
                             double* __restrict__ loss) {
   pdl_begin();
   __shared__ double red[32];

@@ -95,7 +95,7 @@ __device__ __forceinline__ float float64w(unsigned int hi, unsigned int lo) {
 template <int NT>
 __device__ __noinline__ void paint_halves(uint32_t tile, unsigned int* __restrict__ accw,
                                           const uint32_t* __restrict__ run_lo, const uint32_t* __restrict__ run_pre,
-                                          const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
+                                          const uint32_t* us, const uint32_t* ids, int64_t n,
                                           float* __restrict__ mesh, const MassTable& mt, int species, int nm, int shift,
                                           int ntl, int row_pitch) {
   constexpr int HX = kTile / 2, WORDS = HX * kSx;
@@ -155,9 +155,9 @@ __device__ __noinline__ void paint_halves(uint32_t tile, unsigned int* __restric
 template <bool FAST, int NW, int NT>
 __device__ __forceinline__ void paint_tile(
     uint32_t tile, unsigned int* __restrict__ accw, uint32_t* __restrict__ run_lo, uint32_t* __restrict__ run_pre,
-    const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
-    const uint32_t* __restrict__ bstart, float* __restrict__ mesh, const MassTable& mt, int species, int nm,
-    int shift, int ntl, int row_pitch, int* __restrict__ err, const float* __restrict__ wts,
+    const uint32_t* us, const uint32_t* ids, int64_t n,
+    const uint32_t* bstart, float* __restrict__ mesh, const MassTable& mt, int species, int nm,
+    int shift, int ntl, int row_pitch, int* __restrict__ err, const float* wts,
     float* __restrict__ mesh1 = nullptr, float* __restrict__ mesh2 = nullptr) {
   constexpr int NA = NW > 1 ? NW : 1;  // meshes painted
   // FAST: low words, then the wrap bitmap, the event count and the event list.  Else per
@@ -321,9 +321,9 @@ __device__ __forceinline__ void paint_tile(
 // two-word form, with NW signed weights instead of masses when NW > 0.
 template <bool FAST, int NW, int NT>
 __global__ void __launch_bounds__(NT, FAST ? 2048 / NT : 1) k_paint_tiles(
-    const uint32_t* __restrict__ us, const uint32_t* __restrict__ ids, int64_t n,
-    const uint32_t* __restrict__ bstart, float* __restrict__ mesh, const __grid_constant__ MassTable mt, int species,
-    int nm, int shift, int ntl, int row_pitch, int* __restrict__ err, const float* __restrict__ wts) {
+    const uint32_t* us, const uint32_t* ids, int64_t n,
+    const uint32_t* bstart, float* __restrict__ mesh, const __grid_constant__ MassTable mt, int species,
+    int nm, int shift, int ntl, int row_pitch, int* __restrict__ err, const float* wts) {
   pdl_begin();
   __shared__ __align__(16) unsigned int accw[FAST ? kFastWords : 2 * kAccWords];
   __shared__ uint32_t run_lo[14], run_pre[15];
@@ -337,9 +337,9 @@ __global__ void __launch_bounds__(NT, FAST ? 2048 / NT : 1) k_paint_tiles(
 constexpr int kPaint3Threads = 512;
 constexpr size_t kPaint3Smem = sizeof(unsigned int) * 3 * 2 * kAccWords;
 __global__ void __launch_bounds__(kPaint3Threads, 2) k_paint_weights3(
-    const uint32_t* __restrict__ us, int64_t n, const uint32_t* __restrict__ bstart, float* __restrict__ m0,
+    const uint32_t* us, int64_t n, const uint32_t* bstart, float* __restrict__ m0,
     float* __restrict__ m1, float* __restrict__ m2, int nm, int shift, int ntl, int row_pitch, int* __restrict__ err,
-    const float* __restrict__ wts) {
+    const float* wts) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned int accw3[];
   __shared__ uint32_t run_lo[14], run_pre[15];
@@ -349,12 +349,12 @@ __global__ void __launch_bounds__(kPaint3Threads, 2) k_paint_weights3(
 }
 
 // CIC readout of one real mesh component fused with the kick p_j += K F_j.
-__global__ void k_readout_kick(const uint32_t* __restrict__ us, const float* __restrict__ ps,
-                               const uint32_t* __restrict__ ids, int64_t n,
-                               const float* __restrict__ mesh, int nm, int shift, int row_pitch,
+__global__ void k_readout_kick(const uint32_t* us, const float* ps,
+                               const uint32_t* ids, int64_t n,
+                               const float* mesh, int nm, int shift, int row_pitch,
                                int comp, float K, float* __restrict__ p_out,
                                float* __restrict__ f_out, uint32_t* __restrict__ u_out,
-                               uint32_t* __restrict__ id_out, const uint32_t* __restrict__ perm) {
+                               uint32_t* __restrict__ id_out, const uint32_t* perm) {
   pdl_begin();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -367,10 +367,10 @@ __global__ void k_readout_kick(const uint32_t* __restrict__ us, const float* __r
               fz = (float)(uz & fmask) * fscale;
   const size_t r00 = ((size_t)cx * nm + cy) * row_pitch, r01 = ((size_t)cx * nm + cy1) * row_pitch;
   const size_t r10 = ((size_t)cx1 * nm + cy) * row_pitch, r11 = ((size_t)cx1 * nm + cy1) * row_pitch;
-  const float v000 = __ldg(mesh + r00 + cz), v001 = __ldg(mesh + r00 + cz1);
-  const float v010 = __ldg(mesh + r01 + cz), v011 = __ldg(mesh + r01 + cz1);
-  const float v100 = __ldg(mesh + r10 + cz), v101 = __ldg(mesh + r10 + cz1);
-  const float v110 = __ldg(mesh + r11 + cz), v111 = __ldg(mesh + r11 + cz1);
+  const float v000 = mesh[r00 + cz], v001 = mesh[r00 + cz1];
+  const float v010 = mesh[r01 + cz], v011 = mesh[r01 + cz1];
+  const float v100 = mesh[r10 + cz], v101 = mesh[r10 + cz1];
+  const float v110 = mesh[r11 + cz], v111 = mesh[r11 + cz1];
   const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
   const float F = gx * (gy * (gz * v000 + fz * v001) + fy * (gz * v010 + fz * v011)) +
                   fx * (gy * (gz * v100 + fz * v101) + fy * (gz * v110 + fz * v111));
@@ -390,13 +390,13 @@ __global__ void k_readout_kick(const uint32_t* __restrict__ us, const float* __r
 }
 
 // CIC readout of all three force meshes at once, fused with the kick p += K F.
-__global__ void k_readout3_kick(const uint32_t* __restrict__ us, const float* __restrict__ ps,
-                                const uint32_t* __restrict__ ids, int64_t n,
-                                const float* __restrict__ mx, const float* __restrict__ my,
-                                const float* __restrict__ mz, int nm, int shift, int row_pitch,
+__global__ void k_readout3_kick(const uint32_t* us, const float* ps,
+                                const uint32_t* ids, int64_t n,
+                                const float* mx, const float* my,
+                                const float* mz, int nm, int shift, int row_pitch,
                                 float K, float* __restrict__ p_out, float* __restrict__ f_out,
                                 uint32_t* __restrict__ u_out, uint32_t* __restrict__ id_out,
-                                const uint32_t* __restrict__ perm) {
+                                const uint32_t* perm) {
   pdl_begin();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -417,9 +417,9 @@ __global__ void k_readout3_kick(const uint32_t* __restrict__ us, const float* __
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const float* g = m[d];
-    F[d] = w000 * __ldg(g + r00 + cz) + w001 * __ldg(g + r00 + cz1) + w010 * __ldg(g + r01 + cz) +
-           w011 * __ldg(g + r01 + cz1) + w100 * __ldg(g + r10 + cz) + w101 * __ldg(g + r10 + cz1) +
-           w110 * __ldg(g + r11 + cz) + w111 * __ldg(g + r11 + cz1);
+    F[d] = w000 * g[r00 + cz] + w001 * g[r00 + cz1] + w010 * g[r01 + cz] +
+           w011 * g[r01 + cz1] + w100 * g[r10 + cz] + w101 * g[r10 + cz1] +
+           w110 * g[r11 + cz] + w111 * g[r11 + cz1];
   }
   if (perm) {  // force in the caller's order
     const uint32_t j = perm[i];
@@ -548,7 +548,7 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
 // staged row (x, y) holds cells oz - 4 + 4k .. oz - 1 + 4k (mod N): contiguous and 16-byte aligned
 // because N, oz and the row pitch are multiples of 4 floats.
 template <int NT>
-__device__ __forceinline__ void stage_potential(float* sp, const float* __restrict__ phi, int ox, int oy, int oz, int nm,
+__device__ __forceinline__ void stage_potential(float* sp, const float* phi, int ox, int oy, int oz, int nm,
                                                 int row_pitch) {
   const int wrap = nm - 1;
   for (int c = threadIdx.x; c < kStageChunks; c += NT) {
@@ -570,10 +570,10 @@ __device__ __forceinline__ void stage_potential(float* sp, const float* __restri
 // to 6.2 ms against 4.1 on the late steps of 152 M particles at 1024^3).
 template <bool DRIFT, bool NODES, int NT>
 __global__ void __launch_bounds__(NT, NODES ? 2 : (NT == 256 ? 5 : 1024 / NT)) k_readout_fd4_kick(
-    const uint32_t* __restrict__ us, const float* __restrict__ ps, const uint32_t* __restrict__ ids,
-    int64_t n, const uint32_t* __restrict__ bstart, const float* __restrict__ phi, int nm, int shift,
+    const uint32_t* us, const float* ps, const uint32_t* ids,
+    int64_t n, const uint32_t* bstart, const float* phi, int nm, int shift,
     int ntl, int row_pitch, float inv12h, float K, float* __restrict__ p_out, float* __restrict__ f_out,
-    uint32_t* __restrict__ u_out, uint32_t* __restrict__ id_out, const uint32_t* __restrict__ perm,
+    uint32_t* __restrict__ u_out, uint32_t* __restrict__ id_out, const uint32_t* perm,
     int* __restrict__ err, DriftNext dn) {
   pdl_begin();
   extern __shared__ __align__(16) float sp[];  // the potential, then (NODES) the nodes' forces
@@ -706,25 +706,28 @@ __global__ void __launch_bounds__(NT, NODES ? 2 : (NT == 256 ? 5 : 1024 / NT)) k
 // state is not in bprev's order: every particle is then sorted as a mover).
 template <bool RESORT>
 __global__ void k_kick_drift_keys(uint32_t* __restrict__ u, float* __restrict__ p,
-                                  const float* __restrict__ f, int64_t n, float K1, float dscale,
+                                  const float* f, int64_t n, float K1, float dscale,
                                   int shift, int ntl, uint32_t* __restrict__ keys,
-                                  uint32_t* __restrict__ cnt3, long long nb1, const uint32_t* __restrict__ bprev,
+                                  uint32_t* __restrict__ cnt3, long long nb1, const uint32_t* bprev,
                                   uint32_t* __restrict__ low, uint32_t* __restrict__ flags, int* __restrict__ err) {
   pdl_begin();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned act = __ballot_sync(0xffffffffu, i < n);
   if (i >= n) return;
   uint32_t uu[3], u0[3];
-  float chk = 0.0f;  // a NaN or infinity in p or f poisons the sum
+  float pv[3], chk = 0.0f;  // a NaN or infinity in p or f poisons the sum
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {  // every load before the first store
+    pv[d] = __fmaf_rn(K1, f[d * n + i], p[d * n + i]);
+    u0[d] = u[d * n + i];
+  }
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const float pv = __fmaf_rn(K1, f[d * n + i], p[d * n + i]);
-    chk += pv;
-    p[d * n + i] = pv;
+    chk += pv[d];
+    p[d * n + i] = pv[d];
     // u += rne(Delta p 2^32 / L), modulo 2^32; the 32-bit conversion (same rounding)
     // whenever the step fits, the 64-bit one (FP64 pipe) only for steps of 2^31 or more
-    u0[d] = u[d * n + i];
-    uu[d] = drift_fixed(u0[d], dscale, pv);
+    uu[d] = drift_fixed(u0[d], dscale, pv[d]);
     u[d * n + i] = uu[d];
   }
   const uint32_t key = tile_key(uu[0], uu[1], uu[2], shift, ntl);
@@ -739,14 +742,14 @@ __global__ void k_kick_drift_keys(uint32_t* __restrict__ u, float* __restrict__ 
   }
 }
 
-__global__ void k_repack_real(const float* __restrict__ src, int sp, float* __restrict__ dst,
+__global__ void k_repack_real(const float* src, int sp, float* __restrict__ dst,
                               int dp, int nm) {
   pdl_begin();
   long long row = blockIdx.x;
   for (int z = threadIdx.x; z < nm; z += blockDim.x) dst[row * dp + z] = src[row * sp + z];
 }
 
-__global__ void k_repack_complex(const float2* __restrict__ src, int sp, float2* __restrict__ dst,
+__global__ void k_repack_complex(const float2* src, int sp, float2* __restrict__ dst,
                                  int dp, int ncols) {
   pdl_begin();
   long long row = blockIdx.x;

@@ -73,8 +73,8 @@ __global__ void k_power_counts(int nm, int units, int tmax, uint32_t* __restrict
 // Sums of Re(da db^*) mult / W^2 (unscaled) by bin, one row of nbins a CTA; also fills r2.
 // A warp walks its units; for each, its lanes walk n_z, so every load covers 256 contiguous bytes.
 template <bool CROSS>
-__global__ void __launch_bounds__(kPowThreads) k_power_bin(const float2* __restrict__ da,
-                                                           const float2* __restrict__ db, int nm,
+__global__ void __launch_bounds__(kPowThreads) k_power_bin(const float2* da,
+                                                           const float2* db, int nm,
                                                            int pc, int nbins, int units, int tmax,
                                                            const float* __restrict__ winv,
                                                            double* __restrict__ partial,
@@ -151,10 +151,10 @@ __device__ __forceinline__ double warp_sum(double v) {
 // over b^2 + b < s <= (b + 1)^2 + (b + 1); a lane takes one of them and walks n_z.  With no
 // partial rows (nrows = 0) only the counts and sum |k|.
 constexpr int kRedThreads = 1024;
-__global__ void __launch_bounds__(kRedThreads) k_power_reduce(const double* __restrict__ partial, int nrows, int nbins,
-                                                              int nm, const uint32_t* __restrict__ r2, double kf,
-                                                              float norm, const float2* __restrict__ da,
-                                                              const float2* __restrict__ db, double* __restrict__ out) {
+__global__ void __launch_bounds__(kRedThreads) k_power_reduce(const double* partial, int nrows, int nbins,
+                                                              int nm, const uint32_t* r2, double kf,
+                                                              float norm, const float2* da,
+                                                              const float2* db, double* __restrict__ out) {
   pdl_begin();
   constexpr int W = kRedThreads / 32;
   __shared__ double red[3][W];
@@ -203,8 +203,8 @@ __global__ void __launch_bounds__(kRedThreads) k_power_reduce(const double* __re
 }
 
 // cw[b] = 2 dL_dP[b] V / (N^6 rho_bar^2 N_b), the weights of k_power_weight (0 for empty bins)
-__global__ void k_power_cw(const double* __restrict__ counts, const double* __restrict__ dL, int nbins, double vol,
-                           double n3, const float2* __restrict__ d, float* __restrict__ cw) {
+__global__ void k_power_cw(const double* counts, const double* dL, int nbins, double vol,
+                           double n3, const float2* d, float* __restrict__ cw) {
   pdl_begin();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nbins) return;
@@ -216,7 +216,7 @@ __global__ void k_power_cw(const double* __restrict__ counts, const double* __re
 // k-space cotangent of a binned auto-spectrum.  A warp takes one row (n_x, n_y).
 __global__ void __launch_bounds__(kPowThreads) k_power_weight(float2* __restrict__ d, int nm, int pc, int nbins,
                                                               const float* __restrict__ winv,
-                                                              const float* __restrict__ cw) {
+                                                              const float* cw) {
   pdl_begin();
   const int lane = threadIdx.x & 31;
   const long long row = (long long)blockIdx.x * kPowWarps + (threadIdx.x >> 5);  // x N + y, N^2 rows in all
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kPowThreads) k_power_weight(float2* __restrict
     float w = 0.0f;
     if (n2 > 0) {
       const int b = bin_of(n2);
-      if (b < nbins) w = __ldg(cw + b) * wxy * __ldg(winv + kz);
+      if (b < nbins) w = cw[b] * wxy * __ldg(winv + kz);
     }
     rp[kz] = cscale(rp[kz], w);
   }

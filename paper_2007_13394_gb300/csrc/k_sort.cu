@@ -93,7 +93,7 @@ constexpr int kScanThreads = 512;
 constexpr int kScanItems = 8;
 constexpr int kScanFew = 8;
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const uint32_t* __restrict__ in, long long n,
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const uint32_t* in, long long n,
                                                             uint32_t* __restrict__ sums) {
   pdl_begin();
   __shared__ uint32_t ws[32];
@@ -106,8 +106,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(const uint32_t* __re
 }
 
 // sums null: few tiles
-__global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* __restrict__ in, long long n,
-                                                       const uint32_t* __restrict__ sums, uint32_t* __restrict__ out) {
+__global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* in, long long n,
+                                                       const uint32_t* sums, uint32_t* __restrict__ out) {
   pdl_begin();
   __shared__ uint32_t ws[32], wb[32];
   const int t = threadIdx.x;
@@ -157,7 +157,7 @@ __device__ __forceinline__ void count_digit(uint32_t d, uint32_t* h) {
 
 // Keys of the particles and the chunk's counts of the first digit, hist[d C + c].
 template <int BITS>
-__global__ void __launch_bounds__(kCountThreads) k_keys(const uint32_t* __restrict__ u, int64_t n, int shift, int ntl,
+__global__ void __launch_bounds__(kCountThreads) k_keys(const uint32_t* u, int64_t n, int shift, int ntl,
                                                         uint32_t* __restrict__ keys, uint32_t* __restrict__ hist) {
   pdl_begin();
   constexpr int DIG = 1 << BITS;
@@ -195,10 +195,10 @@ __global__ void __launch_bounds__(kCountThreads) k_keys(const uint32_t* __restri
 
 // A digit's counts of existing keys: n of them, or (flags set) the movers of a re-sort.
 template <int BITS>
-__global__ void __launch_bounds__(kCountThreads) k_digits(const uint32_t* __restrict__ keys, int64_t n, int shift,
+__global__ void __launch_bounds__(kCountThreads) k_digits(const uint32_t* keys, int64_t n, int shift,
                                                           uint32_t* __restrict__ hist,
-                                                          const uint32_t* __restrict__ flags,
-                                                          const uint32_t* __restrict__ bstart3, long long nb1) {
+                                                          const uint32_t* flags,
+                                                          const uint32_t* bstart3, long long nb1) {
   pdl_begin();
   constexpr int DIG = 1 << BITS;
   __shared__ uint32_t h[DIG];
@@ -262,9 +262,9 @@ __global__ void __launch_bounds__(256) k_chunk_scan(uint32_t* __restrict__ hist,
 // (RAW, few chunks: a launch costs more than the sums) the counts themselves.
 template <int BITS, bool RAW>
 __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
-    const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift,
-    const uint32_t* __restrict__ hist, const uint32_t* __restrict__ totals, uint32_t* __restrict__ kout,
-    uint32_t* __restrict__ vout, const uint32_t* __restrict__ flags, const uint32_t* __restrict__ bstart3,
+    const uint32_t* kin, const uint32_t* vin, int64_t n, int shift,
+    const uint32_t* hist, const uint32_t* totals, uint32_t* __restrict__ kout,
+    uint32_t* __restrict__ vout, const uint32_t* flags, const uint32_t* bstart3,
     long long nb1) {
   pdl_begin();
   constexpr int DIG = 1 << BITS, PER = DIG > kRadixThreads ? DIG / kRadixThreads : 1;
@@ -398,13 +398,40 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
 }
 
 // ------------------------------------------------------------------ gather
+// A particle's words in registers: every load is issued before the first store (the compiler keeps
+// loads of plain const pointers behind earlier stores).
+struct Particle {
+  uint32_t u[3], id;
+  float p[3];
+};
+__device__ __forceinline__ Particle load_particle(const uint32_t* u, const float* p, const uint32_t* id, int64_t n,
+                                                  uint32_t i) {
+  Particle q;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    q.u[d] = u[d * n + i];
+    q.p[d] = p ? p[d * n + i] : 0.0f;
+  }
+  q.id = id ? id[i] : i;
+  return q;
+}
+__device__ __forceinline__ void store_particle(const Particle& q, int64_t n, int64_t k, uint32_t* __restrict__ us,
+                                               float* __restrict__ ps, uint32_t* __restrict__ ids) {
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    us[d * n + k] = q.u[d];
+    if (ps) ps[d * n + k] = q.p[d];
+  }
+  ids[k] = q.id;
+}
+
 // Records of the particles [i0, n) for the gather, in the sort's free buffers: (u, id), or
 // (u, id, p) when there are momenta.  Neutrinos (the input's tail in canonical order) stream
 // freely, so their order says nothing about their place: gathered array by array, each costs four
 // or seven scattered sectors, from a record one or two.  Written through shared memory, whole lines.
 constexpr int kPackThreads = 256;
-__global__ void __launch_bounds__(kPackThreads) k_pack(const uint32_t* __restrict__ u, const float* __restrict__ p,
-                                                       const uint32_t* __restrict__ id, int64_t n, int64_t i0,
+__global__ void __launch_bounds__(kPackThreads) k_pack(const uint32_t* u, const float* p,
+                                                       const uint32_t* id, int64_t n, int64_t i0,
                                                        uint32_t* __restrict__ rec) {
   pdl_begin();
   __shared__ uint32_t sh[7 * kPackThreads];
@@ -428,12 +455,12 @@ __global__ void __launch_bounds__(kPackThreads) k_pack(const uint32_t* __restric
 
 // The first nbb CTAs find the bucket starts in the sorted keys (bstart[k] = number of keys
 // below k; nb1 of them), the others gather the particles (from index i0 on from rec).
-__global__ void k_gather(const uint32_t* __restrict__ u, const float* __restrict__ p,
-                         const uint32_t* __restrict__ id, int64_t n,
-                         const uint32_t* __restrict__ perm, uint32_t* __restrict__ us,
-                         float* __restrict__ ps, uint32_t* __restrict__ ids, const uint32_t* __restrict__ skeys,
+__global__ void k_gather(const uint32_t* u, const float* p,
+                         const uint32_t* id, int64_t n,
+                         const uint32_t* perm, uint32_t* __restrict__ us,
+                         float* __restrict__ ps, uint32_t* __restrict__ ids, const uint32_t* skeys,
                          long long nb1, unsigned nbb, uint32_t* __restrict__ bstart,
-                         const uint32_t* __restrict__ rec, int64_t i0) {
+                         const uint32_t* rec, int64_t i0) {
   pdl_begin();
   if (blockIdx.x < nbb) {
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -453,47 +480,21 @@ __global__ void k_gather(const uint32_t* __restrict__ u, const float* __restrict
   }
   int64_t k = (int64_t)(blockIdx.x - nbb) * blockDim.x + threadIdx.x;
   if (k >= n) return;
-  uint32_t i = perm[k];
+  const uint32_t i = perm[k];
   if ((int64_t)i >= i0) {
     const uint32_t* const r = rec + (size_t)(i - i0) * (p ? 7 : 4);
-    us[k] = r[0];
-    us[n + k] = r[1];
-    us[2 * n + k] = r[2];
-    ids[k] = r[3];
+    Particle q = {{r[0], r[1], r[2]}, r[3], {0.f, 0.f, 0.f}};
     if (p) {
-      ps[k] = __uint_as_float(r[4]);
-      ps[n + k] = __uint_as_float(r[5]);
-      ps[2 * n + k] = __uint_as_float(r[6]);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) q.p[d] = __uint_as_float(r[4 + d]);
     }
-    return;
+    store_particle(q, n, k, us, p ? ps : nullptr, ids);
+  } else {
+    store_particle(load_particle(u, p, id, n, i), n, k, us, p ? ps : nullptr, ids);
   }
-  us[k] = u[i];
-  us[n + k] = u[n + i];
-  us[2 * n + k] = u[2 * n + i];
-  if (p) {
-    ps[k] = p[i];
-    ps[n + k] = p[n + i];
-    ps[2 * n + k] = p[2 * n + i];
-  }
-  ids[k] = id ? id[i] : i;
 }
 
 // ------------------------------------------------------------------ near-sorted re-sort
-__device__ __forceinline__ void copy_particle(const uint32_t* __restrict__ u, const float* __restrict__ p,
-                                              const uint32_t* __restrict__ id, int64_t n, uint32_t i,
-                                              uint32_t dst, uint32_t* __restrict__ us, float* __restrict__ ps,
-                                              uint32_t* __restrict__ ids) {
-  us[dst] = u[i];
-  us[n + dst] = u[n + i];
-  us[2 * n + dst] = u[2 * n + i];
-  if (p) {
-    ps[dst] = p[i];
-    ps[n + dst] = p[n + i];
-    ps[2 * n + dst] = p[2 * n + i];
-  }
-  ids[dst] = id ? id[i] : i;
-}
-
 // One CTA per old tile O: walks O's range [bprev[8 O], bprev[8 O + 8]) in chunks of the
 // block size, in index order.  With stage, a mover's position, momentum and id also go to a
 // 32-byte record at its list position (the placement then reads one sector a mover
@@ -505,11 +506,11 @@ __device__ __forceinline__ void copy_particle(const uint32_t* __restrict__ u, co
 // that the staging area holds (more movers: none is staged).
 template <int NT>
 __global__ void __launch_bounds__(NT) k_resort_old_tiles(
-    const uint32_t* __restrict__ u, const float* __restrict__ p, const uint32_t* __restrict__ id, int64_t n,
-    const uint32_t* __restrict__ keys, const uint32_t* __restrict__ bprev, const uint32_t* __restrict__ bstart3,
-    long long nb1, const uint32_t* __restrict__ low, uint32_t* __restrict__ us, float* __restrict__ ps,
+    const uint32_t* u, const float* p, const uint32_t* id, int64_t n,
+    const uint32_t* keys, const uint32_t* bprev, const uint32_t* bstart3,
+    long long nb1, const uint32_t* low, uint32_t* __restrict__ us, float* __restrict__ ps,
     uint32_t* __restrict__ ids, uint32_t* __restrict__ mk, uint32_t* __restrict__ mv,
-    const uint32_t* __restrict__ flags, int* __restrict__ err, uint4* __restrict__ stage, int64_t stage_room) {
+    const uint32_t* flags, int* __restrict__ err, uint4* __restrict__ stage, int64_t stage_room) {
   pdl_begin();
   constexpr int W = NT / 32;
   __shared__ uint32_t cls_lo[9];   // bprev[8 O + c]
@@ -608,55 +609,55 @@ __global__ void __launch_bounds__(NT) k_resort_old_tiles(
 // stayers when it came from a higher key (r >= low[B]).  The movers of keys below B
 // number bstart[B] - sstart[B], sstart = the stayers' scan (bstart3's second third
 // minus n).
-__device__ __forceinline__ void place_mover(int64_t j, bool all, const uint32_t* __restrict__ mk,
-                                            const uint32_t* __restrict__ mv, int64_t nm,
-                                            const uint32_t* __restrict__ u, const float* __restrict__ p,
-                                            const uint32_t* __restrict__ id, int64_t n,
-                                            const uint32_t* __restrict__ bstart3, long long nb1, long long nbuckets,
-                                            const uint32_t* __restrict__ low, uint32_t* __restrict__ us,
+__device__ __forceinline__ void place_mover(int64_t j, bool all, const uint32_t* mk,
+                                            const uint32_t* mv, int64_t nm,
+                                            const uint32_t* u, const float* p,
+                                            const uint32_t* id, int64_t n,
+                                            const uint32_t* bstart3, long long nb1, long long nbuckets,
+                                            const uint32_t* low, uint32_t* __restrict__ us,
                                             float* __restrict__ ps, uint32_t* __restrict__ ids,
-                                            int* __restrict__ err, const uint4* __restrict__ stage) {
-  const uint32_t B = mk[j];
-  if (B >= (uint64_t)nbuckets || mv[j] >= (uint64_t)(stage ? nm : n)) {
+                                            int* __restrict__ err, const uint4* stage) {
+  const uint32_t B = mk[j], i = mv[j];
+  if (B >= (uint64_t)nbuckets || i >= (uint64_t)(stage ? nm : n)) {
     atomicOr(err, 1);
     return;
   }
-  if (all) {
-    copy_particle(u, p, id, n, mv[j], (uint32_t)j, us, ps, ids);
-    return;
-  }
-  const uint32_t s0 = bstart3[nb1 + B], s1 = bstart3[nb1 + B + 1];
-  const uint32_t r = (uint32_t)j - (bstart3[B] - (s0 - (uint32_t)n));
-  const uint32_t dst = bstart3[B] + r + (r >= low[B] ? s1 - s0 : 0u);
-  if (dst >= (uint64_t)n) {
-    atomicOr(err, 1);
-    return;
-  }
-  if (stage) {  // one 32-byte record (mv: its position in the mover list)
-    const uint4 a = stage[2 * (size_t)mv[j]], b = stage[2 * (size_t)mv[j] + 1];
-    us[dst] = a.x;
-    us[n + dst] = a.y;
-    us[2 * n + dst] = a.z;
-    ids[dst] = a.w;
-    if (p) {
-      ps[dst] = __uint_as_float(b.x);
-      ps[n + dst] = __uint_as_float(b.y);
-      ps[2 * n + dst] = __uint_as_float(b.z);
+  int64_t dst = j;
+  if (!all) {
+    const uint32_t s0 = bstart3[nb1 + B], s1 = bstart3[nb1 + B + 1], b0 = bstart3[B], lo = low[B];
+    const uint32_t r = (uint32_t)j - (b0 - (s0 - (uint32_t)n));
+    dst = b0 + r + (r >= lo ? s1 - s0 : 0u);
+    if (dst >= n) {
+      atomicOr(err, 1);
+      return;
     }
+  }
+  if (stage) {  // one 32-byte record (i: its position in the mover list)
+    const uint4 a = stage[2 * (size_t)i], b = stage[2 * (size_t)i + 1];
+    const Particle q = {{a.x, a.y, a.z}, a.w, {__uint_as_float(b.x), __uint_as_float(b.y), __uint_as_float(b.z)}};
+    store_particle(q, n, dst, us, p ? ps : nullptr, ids);
   } else {
-    copy_particle(u, p, id, n, mv[j], dst, us, ps, ids);
+    // scattered words, one array after the other: all seven loads at once spread wider than the
+    // caches hold (35 M particles at 256^3, two steps: 491 us, 692 with all loads first)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) us[d * n + dst] = u[d * n + i];
+    if (p) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) ps[d * n + dst] = p[d * n + i];
+    }
+    ids[dst] = id ? id[i] : i;
   }
 }
 
 // With flag bit 1 the movers are all particles: mover j goes to slot j.  Counts the re-sort in
 // stats (near-sorted, from scratch, movers of the last near-sorted one).
-__global__ void k_place_movers(const uint32_t* __restrict__ mk, const uint32_t* __restrict__ mv,
-                               const uint32_t* __restrict__ u, const float* __restrict__ p,
-                               const uint32_t* __restrict__ id, int64_t n, const uint32_t* __restrict__ bstart3,
-                               long long nb1, long long nbuckets, const uint32_t* __restrict__ low,
+__global__ void k_place_movers(const uint32_t* mk, const uint32_t* mv,
+                               const uint32_t* u, const float* p,
+                               const uint32_t* id, int64_t n, const uint32_t* bstart3,
+                               long long nb1, long long nbuckets, const uint32_t* low,
                                uint32_t* __restrict__ us, float* __restrict__ ps, uint32_t* __restrict__ ids,
-                               const uint32_t* __restrict__ flags, int* __restrict__ err,
-                               const uint4* __restrict__ stage, int64_t stage_room, long long* __restrict__ stats) {
+                               const uint32_t* flags, int* __restrict__ err,
+                               const uint4* stage, int64_t stage_room, long long* __restrict__ stats) {
   pdl_begin();
   const bool all = (*flags & 1u) != 0u;
   const int64_t nm = movers_of(flags, bstart3, nb1, n, err);

@@ -331,8 +331,17 @@ inline void allow_smem(DeviceOnce& once, const void* kern, size_t bytes) {
 // is that of ordinary launches; what is saved is the launch gap.  Only grids that fit the GPU
 // at once are launched early (force at 64^3 67.6 -> 55.3 us, 10 steps 953 -> 749): CTAs of a
 // larger grid that settle early, wherever the last ones of the kernel before leave room, share
-// the SMs unevenly (5 steps at 512^3 15.5 ms, 16.3 with every kernel launched early).
-// Without the launch attribute pdl_begin is a no-op.
+// the SMs unevenly (5 steps at 512^3 15.5 ms, 16.3 with every kernel launched early).  A large
+// grid, launched in the ordinary way, waits for nothing but lets a small one behind it start
+// early all the same.
+//
+// A kernel launched early is alive while the ones before it still write, and the non-coherent
+// loads (__ldg, and whatever the compiler makes of const __restrict__ pointers) are specified
+// only for memory that nothing writes during the kernel's life.  So inputs are taken through
+// plain const pointers: pdl_begin's memory clobber then tells the compiler that they may have
+// changed up to that point, and the loads after it are ordinary ones.  The exceptions are tables
+// that no kernel writes (twiddles tw, wavenumber tables ksq, winv, kvec0, amplitudes amp, the
+// neutrino table tab: copied from the host before the launches that read them).
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
