@@ -76,6 +76,38 @@ __device__ __forceinline__ float2 rotl(float2 a) {
   }
 }
 
+// The same rotation with the larger of |cos| and |sin| taken as 1 less its complement: that word
+// of the factor is then good to 4e-9 instead of half a unit in the last place (3e-8 for cos 2 pi / 16
+// and cos 2 pi / 32, the same for every element), at the same number of operations.  Relative rms
+// error of a transform in the stages of the strided passes (32 values a thread), rounded factors /
+// these / stages of radix 8 and 16 with rounded factors: 256^3 1.85e-7 / 1.73e-7 / 1.76e-7, 512^3
+// 2.07e-7 / 1.87e-7 / 1.92e-7, 1024^3 - / 2.00e-7 / 2.13e-7.  The z rows of 1024 and 2048 points
+// keep the rounded factors (their r2c pass takes 14 % longer with these).
+template <int K, int LEN, bool INV>
+__device__ __forceinline__ float2 rot_precise(float2 a) {
+  if constexpr (4 * K % LEN == 0) {
+    return rotl<K, LEN, INV>(a);
+  } else {
+    // e^{s 2 pi i t / 32}, 0 < t < 16: cos in C, its complement 1 - |cos| in D, t from the first axis
+    constexpr double D[8] = {0.0, 0.01921471959676955087, 0.07612046748871324, 0.16853038769745476,
+                             0.29289321881345247560, 0.44442976698039777, 0.61731656763491022, 0.80490967798387169};
+    constexpr int t = K * (32 / LEN), q = t & 7;
+    constexpr float e = (float)D[q <= 4 ? q : 8 - q];              // 1 - the larger word
+    constexpr float m = (float)(1.0 - D[q <= 4 ? 8 - q : q]);      // the smaller word
+    constexpr bool cos_large = (t < 8) == (q <= 4);
+    constexpr float cs = t < 8 ? 1.0f : -1.0f, ss = INV ? 1.0f : -1.0f;  // signs of cos and of sin
+    if constexpr (cos_large) {
+      // re = c x - s y, im = c y + s x, c = cs (1 - e), s = ss m
+      const float cx = fmaf(-e, a.x, a.x), cy = fmaf(-e, a.y, a.y);
+      return make_float2(fmaf(-ss * m, a.y, cs * cx), fmaf(ss * m, a.x, cs * cy));
+    } else {
+      // c = cs m, s = ss (1 - e)
+      const float sx = fmaf(-e, a.x, a.x), sy = fmaf(-e, a.y, a.y);
+      return make_float2(fmaf(cs * m, a.x, -ss * sy), fmaf(cs * m, a.y, ss * sx));
+    }
+  }
+}
+
 template <int R>
 __host__ __device__ constexpr int brev(int i) {
   int r = 0;
@@ -85,29 +117,31 @@ __host__ __device__ constexpr int brev(int i) {
 }
 
 // In-register DFT of size R (2, 4, 8, 16, 32): radix-2 decimation in time.
-template <int R, bool INV, int LEN = 2>
-__device__ __forceinline__ void dft_layers(float2 (&x)[R]);
-
-template <int R, bool INV, int LEN, int I, int K>
+// PREC: rotations by rot_precise.
+template <int R, bool INV, int LEN, int I, int K, bool PREC>
 __device__ __forceinline__ void dft_bfly(float2 (&x)[R]) {
   if constexpr (I < R) {
     if constexpr (K < LEN / 2) {
       float2 a = x[I + K];
-      float2 b = rotl<K, LEN, INV>(x[I + K + LEN / 2]);
+      float2 b;
+      if constexpr (PREC)
+        b = rot_precise<K, LEN, INV>(x[I + K + LEN / 2]);
+      else
+        b = rotl<K, LEN, INV>(x[I + K + LEN / 2]);
       x[I + K] = cadd(a, b);
       x[I + K + LEN / 2] = csub(a, b);
-      dft_bfly<R, INV, LEN, I, K + 1>(x);
+      dft_bfly<R, INV, LEN, I, K + 1, PREC>(x);
     } else {
-      dft_bfly<R, INV, LEN, I + LEN, 0>(x);
+      dft_bfly<R, INV, LEN, I + LEN, 0, PREC>(x);
     }
   }
 }
 
-template <int R, bool INV, int LEN>
+template <int R, bool INV, int LEN, bool PREC>
 __device__ __forceinline__ void dft_layers(float2 (&x)[R]) {
   if constexpr (LEN <= R) {
-    dft_bfly<R, INV, LEN, 0, 0>(x);
-    dft_layers<R, INV, LEN * 2>(x);
+    dft_bfly<R, INV, LEN, 0, 0, PREC>(x);
+    dft_layers<R, INV, LEN * 2, PREC>(x);
   }
 }
 
@@ -124,10 +158,10 @@ __device__ __forceinline__ void bitrev_perm(float2 (&x)[R]) {
   }
 }
 
-template <int R, bool INV>
+template <int R, bool INV, bool PREC = false>
 __device__ __forceinline__ void dft(float2 (&x)[R]) {
   bitrev_perm<R, 0>(x);
-  dft_layers<R, INV, 2>(x);
+  dft_layers<R, INV, 2, PREC>(x);
 }
 
 // Barrier between the shared-memory phases of a stage: the block, or only the warp when
@@ -144,7 +178,8 @@ __device__ __forceinline__ void line_sync() {
 // One Stockham stage on a line of M points (sub-transform length NS, radix R), V values
 // a thread (value s of thread j is element j + s M / V).  TAIL: a barrier after the values
 // are read back (false when nothing writes the shared memory after this exchange).
-template <int M, int TWN, int NS, int R, bool INV, bool LAST, int V = 16, bool WARP = false, bool TAIL = true>
+template <int M, int TWN, int NS, int R, bool INV, bool LAST, int V = 16, bool WARP = false, bool TAIL = true,
+          bool PREC = false>
 __device__ __forceinline__ void stage(float2 (&v)[V], int j, float2* sm, int cs,
                                       const float2* __restrict__ tw) {
   constexpr int B = V / R;  // butterflies per thread
@@ -163,7 +198,7 @@ __device__ __forceinline__ void stage(float2 (&v)[V], int j, float2* sm, int cs,
         x[r] = cmul(x[r], INV ? cconj(w) : w);
       }
     }
-    dft<R, INV>(x);
+    dft<R, INV, PREC>(x);
     if constexpr (LAST) {
 #pragma unroll
       for (int r = 0; r < R; ++r) v[b + r * B] = x[r];
@@ -183,15 +218,15 @@ __device__ __forceinline__ void stage(float2 (&v)[V], int j, float2* sm, int cs,
 
 // All stages of a line.  ENDS: the shared memory is not written again after this transform,
 // so its last exchange needs no trailing barrier.
-template <int M, int TWN, int NS, bool INV, int V = 16, bool WARP = false, bool ENDS = false>
+template <int M, int TWN, int NS, bool INV, int V = 16, bool WARP = false, bool ENDS = false, bool PREC = false>
 __device__ __forceinline__ void run_stages(float2 (&v)[V], int j, float2* sm, int cs,
                                            const float2* __restrict__ tw) {
   constexpr int REM = M / NS;
   constexpr int R = REM >= V ? V : REM;
   constexpr bool LAST = (NS * R == M);
   constexpr bool LASTX = !LAST && M / (NS * R) <= V;  // the transform's last exchange
-  stage<M, TWN, NS, R, INV, LAST, V, WARP, !(ENDS && LASTX)>(v, j, sm, cs, tw);
-  if constexpr (!LAST) run_stages<M, TWN, NS * R, INV, V, WARP, ENDS>(v, j, sm, cs, tw);
+  stage<M, TWN, NS, R, INV, LAST, V, WARP, !(ENDS && LASTX), PREC>(v, j, sm, cs, tw);
+  if constexpr (!LAST) run_stages<M, TWN, NS * R, INV, V, WARP, ENDS, PREC>(v, j, sm, cs, tw);
 }
 
 // Twiddles a thread's stages use, held in registers.  They depend only on the thread's
