@@ -1,0 +1,60 @@
+"""The gather through records with momenta (28 bytes a particle, from 2^21 particles beyond the CDM
+block): a capacity of twice the particles leaves room for the records in the sort's free buffers,
+a capacity of just the particles does not, and the array-by-array gather runs instead.  Steps from
+scratch, chained steps and force VJPs (whose cotangents travel like momenta) have to give the same
+bits either way, for one sort pass (the result in the second pair of buffers) and for two.
+"""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+
+@pytest.fixture(scope="module")
+def pm():
+    import __graft_entry__ as g
+    g.build()
+    from paper_2007_13394_gb300 import pm as _pm
+    return _pm
+
+
+@pytest.mark.parametrize("nmesh", [64, 128])  # 9 and 12 key bits: one pass and two
+@pytest.mark.parametrize("shuffled", [False, True])
+def test_records_change_no_bit(pm, nmesh, shuffled):
+    # 64^3 CDM + 32^3 x 80 neutrinos: 2.62 M of 2.88 M; 28 x 2.62 M bytes against 16 x capacity
+    base = dict(box=200.0, nmesh=nmesh, nc=64, nsites=32, nshell=16, nfib=2, m_nu=(0.1,) * 3)
+    n = pm.RunConfig(**base).n_particles()
+    tail = n - 64 ** 3
+    assert tail >= 2 ** 21 and 28 * tail > 16 * n and 28 * tail <= 16 * 2 * n
+    g = torch.Generator(device="cuda").manual_seed(nmesh)
+    u = torch.randint(-2 ** 31, 2 ** 31, (3, n), generator=g, device="cuda", dtype=torch.int64)
+    u[:, ::3] //= 16
+    u = u.to(torch.int32)
+    p = torch.randn((3, n), generator=g, device="cuda")
+    lam = torch.randn((3, n), generator=g, device="cuda")
+    ids = torch.arange(n, dtype=torch.int32, device="cuda")
+    if shuffled:
+        o = torch.randperm(n, generator=g, device="cuda")
+        u, p, ids = u[:, o].contiguous(), p[:, o].contiguous(), ids[o].contiguous()
+    out = []
+    for n_max in (n, 2 * n):
+        ctx = pm.ParticleMesh(pm.RunConfig(n_max=n_max, **base))
+        got = [ctx.force(u, ids), ctx.force_vjp(u, ids, lam)]
+        st = {"u": u.clone(), "p": p.clone(), "id": ids.clone(), "f": torch.zeros_like(p), "f_valid": 0}
+        ctx.step(st, 0.5, 0.51, 0.52)
+        st2 = {k: v.flip(-1).contiguous() if torch.is_tensor(v) else v for k, v in st.items()}
+        got += [st[k] for k in ("u", "p", "id", "f")]
+        fresh = pm.ParticleMesh(pm.RunConfig(n_max=n_max, **base))  # from scratch, with a force in hand
+        fresh.run(st2, [(0.52, 0.53, 0.54), (0.54, 0.55, 0.56)])
+        fresh.sync()
+        assert fresh.sort_stats()[1] == 1
+        got += [st2[k] for k in ("u", "p", "id", "f")]
+        ctx.sync()
+        ctx.close()
+        fresh.close()
+        out.append(got)
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
