@@ -452,7 +452,7 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
   const size_t me = c->g.elems();
   const int64_t nm = std::max<int64_t>(c->n_max, 1);
   const long long hb = (nm + 4095) / 4096;
-  // counts, rs_low and rs_dev (the zeroed words), then the scan's tile sums
+  // counts, rs_low and rs_dev (the zeroed words), then the scan's tile sums and the gather's flag
   const size_t flag_at = 4 * (size_t)(c->nbuckets + 1), clear_words = flag_at + 1;
   const size_t scan_words = (3 * (size_t)(c->nbuckets + 1) + kScanTile - 1) / kScanTile;
   const size_t hist_words = ((size_t)std::min<long long>(hb, kMaxChunks) + 1) << c->radix_bits;
@@ -463,7 +463,7 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
       dalloc(c, &c->ksq, N) ||
       dalloc(c, &c->winv, N) || dalloc(c, &c->wforce, N) || dalloc(c, &c->kvec0, N) || dalloc(c, &c->sortbuf, 6 * nm) ||
       dalloc(c, &c->us, 3 * nm) || dalloc(c, &c->ps, 3 * nm) || dalloc(c, &c->ids, nm) ||
-      dalloc(c, &c->counts, clear_words + scan_words) || dalloc(c, &c->bstart, 3 * (c->nbuckets + 1)) ||
+      dalloc(c, &c->counts, clear_words + scan_words + 1) || dalloc(c, &c->bstart, 3 * (c->nbuckets + 1)) ||
       dalloc(c, &c->bprev, 3 * (c->nbuckets + 1)) ||
       dalloc(c, &c->rs_stats, 3) || dalloc(c, &c->hist, hist_words) ||
       dalloc(c, &c->pk_partial, (size_t)N * 2 * 2048) ||
@@ -483,6 +483,7 @@ int pm_init(const pm_config* cfg, pm_ctx** out) {
   c->rs_low = c->counts + 3 * (c->nbuckets + 1);
   c->rs_dev = c->counts + flag_at;
   c->scan_sums = c->counts + clear_words;
+  c->pack_flag = c->scan_sums + scan_words;
   c->clear_words = clear_words;
   c->digit_totals = c->hist + (hist_words - ((size_t)1 << c->radix_bits));
   cudaMemset(c->rs_stats, 0, 3 * sizeof(long long));

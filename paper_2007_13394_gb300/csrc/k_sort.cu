@@ -429,38 +429,59 @@ __device__ __forceinline__ void store_particle(const Particle& q, int64_t n, int
 // (u, id, p) when there are momenta.  Neutrinos (the input's tail in canonical order) stream
 // freely, so their order says nothing about their place: gathered array by array, each costs four
 // or seven scattered sectors, from a record one or two.  Written through shared memory, whole lines.
+// A state that a step has left is in tile order, and its tail gathers whole lines already: the
+// records would only add their own traffic.  So every CTA looks at the same 256 places of the
+// permutation, and none is packed (flag 0) where the input's neighbours mostly stay neighbours.
 constexpr int kPackThreads = 256;
-__global__ void __launch_bounds__(kPackThreads) k_pack(const uint32_t* u, const float* p,
-                                                       const uint32_t* id, int64_t n, int64_t i0,
-                                                       uint32_t* __restrict__ rec) {
+constexpr int kPackCtas = 8 * 152;
+__global__ void __launch_bounds__(kPackThreads) k_pack(const uint32_t* u, const float* p, const uint32_t* id, int64_t n,
+                                                       int64_t i0, const uint32_t* perm, uint32_t* __restrict__ rec,
+                                                       uint32_t* __restrict__ flag) {
   pdl_begin();
-  __shared__ uint32_t sh[7 * kPackThreads];
+  __shared__ uint32_t sh[7 * kPackThreads], seen[kPackThreads / 32];
   const int W = p ? 7 : 4, t = threadIdx.x;
-  const int64_t first = i0 + (int64_t)blockIdx.x * kPackThreads, i = first + t;
-  if (i < n) {
-    sh[t * W] = u[i];
-    sh[t * W + 1] = u[n + i];
-    sh[t * W + 2] = u[2 * n + i];
-    sh[t * W + 3] = id ? id[i] : (uint32_t)i;
-    if (p) {
-#pragma unroll
-      for (int d = 0; d < 3; ++d) sh[t * W + 4 + d] = __float_as_uint(p[d * n + i]);
-    }
-  }
+  const int64_t k = t * (n - 1) / kPackThreads;
+  const uint32_t at = perm[k], next = perm[k + 1];
+  // samples in the tail, and (from bit 16) those whose successor comes next
+  uint32_t c = (int64_t)at < i0 ? 0u : (next == at + 1 ? 0x10001u : 1u);
+  c = __reduce_add_sync(0xffffffffu, c);
+  if ((t & 31) == 0) seen[t >> 5] = c;
   __syncthreads();
-  const int words = (int)((n - first < kPackThreads ? n - first : kPackThreads) * W);
-  uint32_t* const out = rec + (size_t)blockIdx.x * kPackThreads * W;
-  for (int k = t; k < words; k += kPackThreads) out[k] = sh[k];
+  c = 0;
+#pragma unroll
+  for (int w = 0; w < kPackThreads / 32; ++w) c += seen[w];
+  const bool pack = 3 * (c & 0xffffu) > 4 * (c >> 16);  // runs shorter than four on average
+  if (blockIdx.x == 0 && t == 0) *flag = pack ? 1u : 0u;
+  if (!pack) return;
+  for (int64_t first = i0 + (int64_t)blockIdx.x * kPackThreads; first < n; first += (int64_t)gridDim.x * kPackThreads) {
+    const int64_t i = first + t;
+    if (i < n) {
+      sh[t * W] = u[i];
+      sh[t * W + 1] = u[n + i];
+      sh[t * W + 2] = u[2 * n + i];
+      sh[t * W + 3] = id ? id[i] : (uint32_t)i;
+      if (p) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sh[t * W + 4 + d] = __float_as_uint(p[d * n + i]);
+      }
+    }
+    __syncthreads();
+    const int words = (int)((n - first < kPackThreads ? n - first : kPackThreads) * W);
+    uint32_t* const out = rec + (size_t)(first - i0) * W;
+    for (int q = t; q < words; q += kPackThreads) out[q] = sh[q];
+    __syncthreads();
+  }
 }
 
 // The first nbb CTAs find the bucket starts in the sorted keys (bstart[k] = number of keys
-// below k; nb1 of them), the others gather the particles (from index i0 on from rec).
+// below k; nb1 of them), the others gather the particles (from index i0 on from rec if there is a
+// flag and it is set).
 __global__ void k_gather(const uint32_t* u, const float* p,
                          const uint32_t* id, int64_t n,
                          const uint32_t* perm, uint32_t* __restrict__ us,
                          float* __restrict__ ps, uint32_t* __restrict__ ids, const uint32_t* skeys,
                          long long nb1, unsigned nbb, uint32_t* __restrict__ bstart,
-                         const uint32_t* rec, int64_t i0) {
+                         const uint32_t* rec, int64_t i0, const uint32_t* flag) {
   pdl_begin();
   if (blockIdx.x < nbb) {
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -481,7 +502,7 @@ __global__ void k_gather(const uint32_t* u, const float* p,
   int64_t k = (int64_t)(blockIdx.x - nbb) * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const uint32_t i = perm[k];
-  if ((int64_t)i >= i0) {
+  if (flag && (int64_t)i >= i0 && *flag) {
     const uint32_t* const r = rec + (size_t)(i - i0) * (p ? 7 : 4);
     Particle q = {{r[0], r[1], r[2]}, r[3], {0.f, 0.f, 0.f}};
     if (p) {
@@ -758,22 +779,25 @@ void gather_sorted(pm_ctx* c, const uint32_t* u, const float* p, const uint32_t*
                    const uint32_t* perm, cudaStream_t s) {
   if (n == 0) return;
   // The neutrinos through records where scattered sectors are what the gather costs: from 2^21 of
-  // them on (fewer stay in the second-level cache), if they fit the free half of the sort's
-  // buffers (16 bytes a particle of the capacity).  35 M particles, half neutrinos: 2096 us
-  // without, 148 + 631 with.
-  int64_t i0 = std::min<int64_t>(n, c->mt.n_cdm);
+  // them on with momenta, 2^22 without (fewer stay in the second-level cache), if they fit the free
+  // half of the sort's buffers (16 bytes a particle of the capacity); the kernel leaves out those in
+  // tile order.  us without / with records, 4 and 7 words a particle: 0.9 M of 17.7 M neutrinos
+  // 144 / 159 and 230 / 242, 2.3 M of 19 M 183 / 184 and 318 / 285, 18 M of 35 M 1005 / 525 and
+  // 2073 / 818; the last in tile order 235 / 340 and 324 / 475 if they were packed.
+  const int64_t i0 = std::min<int64_t>(n, c->mt.n_cdm);
   uint32_t* const rec = c->keys[0] == c->sortbuf ? c->rs_k2 : c->sortbuf;
   const int64_t rec_bytes = (n - i0) * (p ? 28 : 16);
-  if (n - i0 >= (1 << 21) && rec_bytes <= 16 * std::max<int64_t>(c->n_max, 1)) {
+  const uint32_t* flag = nullptr;
+  if (n - i0 >= (p ? 1 << 21 : 1 << 22) && rec_bytes <= 16 * std::max<int64_t>(c->n_max, 1)) {
     LaunchScope L(c, s, K_GATHER);
-    pdl_launch(k_pack, (unsigned)((n - i0 + kPackThreads - 1) / kPackThreads), kPackThreads, 0, s, u, p, id, n, i0, rec);
-  } else {
-    i0 = n;
+    const unsigned grid = (unsigned)std::min<int64_t>(kPackCtas, (n - i0 + kPackThreads - 1) / kPackThreads);
+    pdl_launch(k_pack, grid, kPackThreads, 0, s, u, p, id, n, i0, perm, rec, c->pack_flag);
+    flag = c->pack_flag;
   }
   LaunchScope L(c, s, K_GATHER);
   const unsigned nbb = (unsigned)((c->nbuckets + 1 + 255) / 256);
   pdl_launch(k_gather, nbb + (unsigned)((n + 255) / 256), 256, 0, s, u, p, id, n, perm, c->us, c->ps, c->ids, c->keys[0],
-                                                            c->nbuckets + 1, nbb, c->bstart, rec, i0);
+                                                            c->nbuckets + 1, nbb, c->bstart, rec, i0, flag);
 }
 
 int clear_resort(pm_ctx* c, cudaStream_t s) {

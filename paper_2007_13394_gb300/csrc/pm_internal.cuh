@@ -138,12 +138,13 @@ struct pm_ctx {
   uint32_t* bprev = nullptr;
   int64_t rs_n = -1;
   // one allocation: counts, rs_low and rs_dev, zeroed (clear_words) before each drift that
-  // counts, then the scan's tile sums
+  // counts, then the scan's tile sums and the gather's flag
   uint32_t* counts = nullptr;     // 3 (nbuckets + 1)
   size_t clear_words = 0;
   uint32_t* rs_low = nullptr;     // movers from a lower old key, per new key (nbuckets + 1)
   uint32_t* rs_dev = nullptr;     // flag bits of k_kick_drift_keys<true>
   uint32_t* scan_sums = nullptr;
+  uint32_t* pack_flag = nullptr;  // the gather's records are written (k_pack)
   uint32_t* rs_k2 = nullptr;      // second (key, index) buffer pair of the movers' radix
   uint32_t* rs_v2 = nullptr;
   long long* rs_stats = nullptr;  // device: re-sorts near-sorted, from scratch, movers of the last near-sorted one
