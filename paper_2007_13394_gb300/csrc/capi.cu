@@ -141,7 +141,8 @@ void free_all(pm_ctx* c) {
   for (auto e : c->prof_pool) cudaEventDestroy(e);
 }
 
-// sort (u, n) -> vals[0] = perm, keys[0] = sorted keys, bstart = bucket starts
+// sort (u, n) -> vals[0] = perm, keys[0] = sorted keys; the bucket starts (bstart) come with the
+// gather (gather_sorted), which every call that paints or reads out makes next
 int sort_into_scratch(pm_ctx* c, const uint32_t* u, int64_t n, cudaStream_t s) {
   if (n > c->n_max) return PM_EINVAL;
   return sort_particles(c, u, n, s);

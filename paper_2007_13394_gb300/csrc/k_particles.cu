@@ -820,8 +820,9 @@ void readout_fd4_kick(pm_ctx* c, const uint32_t* us, const float* ps, const uint
   LaunchScope L(c, s, K_READOUT_FD4_KICK);
   const float inv12h = (float)((double)c->g.n / (12.0 * c->cfg.box));
   const unsigned grid = (unsigned)(c->nt * c->nt * c->nt);
-  // Forces at the nodes first where tiles are full: see the kernel for both sides.  Meshes below
-  // 256^3 keep the gathering form, and with it their bits.
+  // Forces at the nodes first where tiles are full: see the kernel for both sides, measured with 4096
+  // tiles (256^3).  Meshes below keep the gathering form at any filling for the sake of their bits,
+  // not of speed: the node form was not measured there.
   const bool nodes = c->g.n >= 256 && n >= (int64_t)kNodesMin * grid;
   const bool few = !nodes && tile_threads(c) == 1024;  // (at 128^3 five CTAs of 256 hold more warps than two of 512)
   const int threads = nodes ? kNodeThreads : (few ? 1024 : 256);

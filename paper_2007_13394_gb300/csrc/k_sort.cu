@@ -11,10 +11,10 @@
 // staging offsets, and the keys go out through shared memory in coalesced runs.  A bucket's
 // start is a binary search in the sorted keys, done by the gather.
 //
-// Bound by latency inside a tile, then by DRAM (20 bytes a particle and pass).  us a pass (counts,
-// scan and scatter), 19 M particles, 9 bits: 28 + 3 + 137 (with a
-// warp match per round, 4096-key blocks and a three-launch scan: 42 + 15 + 215); the key kernel,
-// which no longer counts buckets with global atomics, 103 -> 56.
+// The scatter is bound by instruction issue and by latency inside a tile (SM 60 %, DRAM 21 to 27 %
+// of peak at 512^3).  us a pass (counts, scan and scatter), 19 M particles, 9 bits: 28 + 3 + 137
+// (with a warp match per round, 4096-key blocks and a three-launch scan: 42 + 15 + 215); the key
+// kernel, which no longer counts buckets with global atomics, 103 -> 56.
 //
 // Near-sorted re-sort (pm_step): the state is in the order of the last step's sort,
 // bucket starts bprev, and most particles keep their key.  A stayer (same key, inside
